@@ -899,30 +899,34 @@ fmdp_status fmdp_sep_check(fmdp_ctx* c, int64_t t0, const float* xyz, int32_t n,
     return guard(c, [&] {
         require(xyz && out && n >= 1, FMDP_ERR_ARG, "null trajectory or output");
         const int32_t S_scan = round_up(c->book.S_hw, 32);
-        c->traj.ensure((size_t)n * 3);
-        c->sepo.ensure(1);
-        CK(cudaMemcpyAsync(c->traj.p, xyz, (size_t)n * 12, cudaMemcpyHostToDevice, c->stream));
-        LAUNCH(c, launch_sep_reset(c->sepo.p, 1, c->stream));
-        SepArgs sa{};
-        sa.m = c->model;
-        sa.tab = table_view(c);
-        sa.S_scan = S_scan;
-        sa.cap = n;
-        sa.traj = c->traj.p;
-        sa.rout = nullptr;
-        sa.reqs = nullptr;
-        sa.t0_fixed = t0;
-        sa.n_fixed = n;
-        sa.out = c->sepo.p;
-        {
-            KernelTimer t(c, 1);
-            LAUNCH(c, launch_sepcheck(sa, 1, n, c->stream));
-            t.stop();
-        }
         SepOut so;
-        CK(cudaMemcpyAsync(&so, c->sepo.p, sizeof(so), cudaMemcpyDeviceToHost, c->stream));
-        CK(cudaStreamSynchronize(c->stream));
-        if (c->profiling) collect_timers(c);
+        if (c->index_on) {
+            so = check_now(c, t0, xyz, n);
+        } else {
+            c->traj.ensure((size_t)n * 3);
+            c->sepo.ensure(1);
+            CK(cudaMemcpyAsync(c->traj.p, xyz, (size_t)n * 12, cudaMemcpyHostToDevice, c->stream));
+            LAUNCH(c, launch_sep_reset(c->sepo.p, 1, c->stream));
+            SepArgs sa{};
+            sa.m = c->model;
+            sa.tab = table_view(c);
+            sa.S_scan = S_scan;
+            sa.cap = n;
+            sa.traj = c->traj.p;
+            sa.rout = nullptr;
+            sa.reqs = nullptr;
+            sa.t0_fixed = t0;
+            sa.n_fixed = n;
+            sa.out = c->sepo.p;
+            {
+                KernelTimer t(c, 1);
+                launch_check(c, sa, n);
+                t.stop();
+            }
+            CK(cudaMemcpyAsync(&so, c->sepo.p, sizeof(so), cudaMemcpyDeviceToHost, c->stream));
+            CK(cudaStreamSynchronize(c->stream));
+            if (c->profiling) collect_timers(c);
+        }
         c->stats.sep_pairs += (int64_t)n * S_scan;
         out->first_conflict_step = so.first_conflict == INT_MAX ? -1 : so.first_conflict;
         out->first_terrain_step = so.first_terrain == INT_MAX ? -1 : so.first_terrain;

@@ -344,10 +344,7 @@ struct SepRowsArgs {
     const int32_t* n_dev;  // their number (<= n_max)
     int32_t n_max;
     SepOut* out;
-    const float4* items;    // spatial index (nullptr: read the table planes)
-    const int32_t* cstart;
-    const int32_t* nextra;
-    int32_t ncell;
+    IndexView iv;           // spatial index (iv.items nullptr: read the table planes)
     const int32_t* skip;    // request r is not checked when skip[r] (nullptr: none)
     // ordinal filter (pipelined FCFS, where the table may already hold plans admitted after
     // a request): request r is checked only against items whose slot's ordinal is below
@@ -359,6 +356,42 @@ struct SepRowsArgs {
     int32_t row0, nrows;
 };
 cudaError_t launch_sepcheck_rows(const SepRowsArgs& a, cudaStream_t s);
+// The same check against the spatial index, one warp per sample: of each row only the cells
+// that can hold a conflict or a separation below the least one found (sepcheck_cells_kernel).
+struct SepCellsArgs {
+    Model m;
+    TableView tab;
+    IndexView iv;
+    const float* traj;         // [n][cap][3]
+    int32_t cap;
+    const RolloutOut* rout;    // n_points per request (nullptr: n_fixed)
+    const fmdp_request* reqs;  // t0 = depart_step (nullptr: t0_fixed)
+    int64_t t0_fixed;
+    int32_t n_fixed;
+    const int32_t* idx;        // request of work item (nullptr: identity)
+    const int32_t* n_dev;      // number of work items on the device (nullptr: all launched)
+    const int32_t* skip;       // as SepRowsArgs
+    const int32_t* slot_ord;
+    const int32_t* req_ord;
+    SepOut* out;
+    int32_t terrain_all;       // 1: terrain is tested at samples outside the table window too
+    // one launch per call (n_req 1): the last block writes the report to host-mapped memory,
+    // then the token, and resets `out` and the counter for the next call (nullptr: none of this)
+    int32_t* blocks_done;
+    struct CheckReport* h_rep;
+    int32_t token;
+};
+struct CheckReport {
+    SepOut out;
+    int32_t token;  // written last
+    int32_t pad[3];
+};
+struct CheckAccum {  // device: the accumulators between two such calls are in their reset state
+    SepOut out;
+    int32_t blocks_done;
+    int32_t pad[3];
+};
+cudaError_t launch_sepcheck_cells(const SepCellsArgs& a, int n_req, int max_points, cudaStream_t s);
 size_t sepcheck_rows_smem(int n_max);
 cudaError_t prepare_sepcheck_rows(size_t smem);
 

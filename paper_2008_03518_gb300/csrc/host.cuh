@@ -89,6 +89,27 @@ struct PinnedArray {
     }
 };
 
+// Pinned host memory mapped into the device address space.
+template <class T>
+struct MappedArray {
+    T* p = nullptr;  // host pointer
+    T* d = nullptr;  // device pointer of the same memory
+    size_t n = 0;
+    void ensure(size_t want) {
+        if (want <= n) return;
+        release();
+        const size_t m = std::max<size_t>(want, 16);
+        CK(cudaHostAlloc((void**)&p, m * sizeof(T), cudaHostAllocMapped | cudaHostAllocPortable));
+        n = m;
+        CK(cudaHostGetDevicePointer((void**)&d, p, 0));
+    }
+    void release() {
+        if (p) cudaFreeHost(p);
+        p = d = nullptr;
+        n = 0;
+    }
+};
+
 inline int32_t round_up(int32_t x, int32_t m) { return (x + m - 1) / m * m; }
 
 constexpr int32_t kExtraLimit = 48;  // appended items per index row before the row is rebuilt
@@ -197,6 +218,12 @@ struct fmdp_ctx {
     // batch co-simulation: per-step aircraft records and the grid barrier words
     DevArray<double> cs_mem;
     DevArray<int32_t> cs_bar;
+
+    // one-launch separation check (fmdp_sep_check): trajectory and report in mapped host memory
+    MappedArray<float> chk_xyz;
+    MappedArray<CheckReport> chk_rep;
+    DevArray<CheckAccum> chk_acc;
+    int32_t chk_token = 0;
 
     // work buffers
     SeqBuffers seq;     // fmdp_schedule / fmdp_schedule_many
@@ -389,6 +416,8 @@ Geometry geometry(fmdp_ctx* c, int32_t S_hw);
 void check_request(fmdp_ctx* c, const fmdp_request& r);
 int32_t take_slot(fmdp_ctx* c);
 void recompute_hw(fmdp_ctx* c);
+void launch_check(fmdp_ctx* c, const SepArgs& a, int32_t max_points);
+SepOut check_now(fmdp_ctx* c, int64_t t0, const float* xyz, int32_t n);
 void enqueue_sequence(fmdp_ctx* c, SeqBuffers& B, const fmdp_request* host_reqs, int32_t n, int32_t cap,
                       const Geometry& g, bool plan = true);
 int32_t read_error_word(fmdp_ctx* c);

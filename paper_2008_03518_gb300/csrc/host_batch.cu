@@ -122,12 +122,7 @@ void enqueue_wave(fmdp_ctx* c, const Geometry& g, int n_clusters, BatchBuffers& 
         sp.n_dev = B.ctr.p + 1;
         sp.n_max = n_cap;
         sp.out = c->p_sep.p;
-        if (c->index_on) {
-            sp.items = c->ix_items;
-            sp.cstart = c->ix_cstart;
-            sp.nextra = c->ix_nextra;
-            sp.ncell = c->ix_ncell;
-        }
+        if (c->index_on) sp.iv = index_view(c);
         LAUNCH(c, launch_sepcheck_rows(sp, s));
         JudgeArgs ja{};
         ja.reqs = B.rq;
@@ -206,12 +201,7 @@ void enqueue_wave(fmdp_ctx* c, const Geometry& g, int n_clusters, BatchBuffers& 
         sa.n_max = n_cap;
         sa.out = B.sepo.p;
         sa.skip = c->learned_mode ? c->p_acc.p : nullptr;
-        if (c->index_on) {
-            sa.items = c->ix_items;
-            sa.cstart = c->ix_cstart;
-            sa.nextra = c->ix_nextra;
-            sa.ncell = c->ix_ncell;
-        }
+        if (c->index_on) sa.iv = index_view(c);
         KernelTimer t(c, timed ? 1 : -1);
         LAUNCH(c, launch_sepcheck_rows(sa, s));
         t.stop();
@@ -487,12 +477,7 @@ void run_departures(fmdp_ctx* c, const fmdp_request* reqs, int32_t n, const int6
         sa.n_dev = B.ctr.p + 1;
         sa.n_max = D;
         sa.out = B.sepo.p;
-        if (c->index_on) {
-            sa.items = c->ix_items;
-            sa.cstart = c->ix_cstart;
-            sa.nextra = c->ix_nextra;
-            sa.ncell = c->ix_ncell;
-        }
+        if (c->index_on) sa.iv = index_view(c);
         LAUNCH(c, launch_sepcheck_rows(sa, c->stream));
         CK(cudaMemcpyAsync(B.h_rout.p, B.rout.p, D * sizeof(RolloutOut), cudaMemcpyDeviceToHost, c->stream));
         CK(cudaMemcpyAsync(B.h_sep.p, B.sepo.p, D * sizeof(SepOut), cudaMemcpyDeviceToHost, c->stream));

@@ -209,10 +209,7 @@ void learned_evaluate(fmdp_ctx* c, const fmdp_request* reqs, int32_t n, double s
         sp.n_dev = B.ctr.p + 1;
         sp.n_max = m;
         sp.out = c->p_sep.p;
-        sp.items = c->ix_items;
-        sp.cstart = c->ix_cstart;
-        sp.nextra = c->ix_nextra;
-        sp.ncell = c->ix_ncell;
+        sp.iv = index_view(c);
         LAUNCH(c, launch_sepcheck_rows(sp, c->stream));
         CK(cudaStreamSynchronize(c->stream));  // the count word is reused by the next chunk
     }

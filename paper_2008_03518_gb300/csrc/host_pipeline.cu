@@ -42,27 +42,6 @@ namespace fmdp {
 
 namespace {
 
-// Pinned host memory mapped into the device address space.
-template <class T>
-struct MappedArray {
-    T* p = nullptr;  // host pointer
-    T* d = nullptr;  // device pointer of the same memory
-    size_t n = 0;
-    void ensure(size_t want) {
-        if (want <= n) return;
-        release();
-        const size_t m = std::max<size_t>(want, 16);
-        CK(cudaHostAlloc((void**)&p, m * sizeof(T), cudaHostAllocMapped | cudaHostAllocPortable));
-        n = m;
-        CK(cudaHostGetDevicePointer((void**)&d, p, 0));
-    }
-    void release() {
-        if (p) cudaFreeHost(p);
-        p = d = nullptr;
-        n = 0;
-    }
-};
-
 constexpr int kQueueCap = 4096;           // ring entries (a power of two)
 constexpr int kRepSlots = 8;              // staging slots of the asynchronous separation reports
 constexpr int kRepChunk = 64;             // finished requests per report while the launch runs
@@ -476,10 +455,7 @@ int32_t run_pipeline(fmdp_ctx* c, const fmdp_request* reqs, int32_t n, fmdp_resu
             sp.n_dev = dn;
             sp.n_max = m;
             sp.out = B.sepo.p;
-            sp.items = c->ix_items;
-            sp.cstart = c->ix_cstart;
-            sp.nextra = c->ix_nextra;
-            sp.ncell = c->ix_ncell;
+            sp.iv = index_view(c);
             sp.slot_ord = P.slot_ord.p;
             sp.req_ord = P.req_ord.p;
             if (t_hi > t_lo) {

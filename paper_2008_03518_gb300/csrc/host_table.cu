@@ -330,6 +330,88 @@ void recompute_hw(fmdp_ctx* c) {
     c->book.S_hw = c->book.slot_bound();
 }
 
+// Separation check of one trajectory of at most max_points samples: against the spatial
+// index when there is one, else against every slot of the table.
+void launch_check(fmdp_ctx* c, const SepArgs& a, int32_t max_points) {
+    if (!c->index_on) {
+        LAUNCH(c, launch_sepcheck(a, 1, max_points, c->stream));
+        return;
+    }
+    SepCellsArgs s{};
+    s.m = a.m;
+    s.tab = a.tab;
+    s.iv = index_view(c);
+    s.traj = a.traj;
+    s.cap = a.cap;
+    s.rout = a.rout;
+    s.reqs = a.reqs;
+    s.t0_fixed = a.t0_fixed;
+    s.n_fixed = a.n_fixed;
+    s.out = a.out;
+    s.terrain_all = 1;
+    LAUNCH(c, launch_sepcheck_cells(s, 1, max_points, c->stream));
+}
+
+// Separation check of a host trajectory against the spatial index, in one launch: the kernel
+// reads the samples from mapped host memory and its last block writes the report there, so
+// that no copy, reset or second launch lies on the call's path, and the host waits on the
+// report's token. 200 plans, 311 samples: 27.6 us a call with copies both ways and a reset
+// launch, 17.5 us now. Trajectories beyond kMappedPoints are copied to the device first (a warp's 12-byte
+// read of host memory is slower than its share of a copy).
+constexpr int32_t kMappedPoints = 16384;
+
+SepOut check_now(fmdp_ctx* c, int64_t t0, const float* xyz, int32_t n) {
+    c->chk_rep.ensure(1);
+    if (c->chk_acc.n == 0) {  // the first call: accumulators in their reset state
+        c->chk_acc.ensure(1);
+        CK(cudaMemsetAsync(c->chk_acc.p, 0, sizeof(CheckAccum), c->stream));
+        LAUNCH(c, launch_sep_reset(&c->chk_acc.p->out, 1, c->stream));
+        c->chk_rep.p->token = c->chk_token;
+    }
+    SepCellsArgs s{};
+    if (n <= kMappedPoints) {
+        c->chk_xyz.ensure((size_t)3 * std::max(n, 2048));
+        std::memcpy(c->chk_xyz.p, xyz, (size_t)n * 12);
+        s.traj = c->chk_xyz.d;
+    } else {
+        c->traj.ensure((size_t)n * 3);
+        CK(cudaMemcpyAsync(c->traj.p, xyz, (size_t)n * 12, cudaMemcpyHostToDevice, c->stream));
+        s.traj = c->traj.p;
+    }
+    s.m = c->model;
+    s.tab = table_view(c);
+    s.iv = index_view(c);
+    s.cap = n;
+    s.t0_fixed = t0;
+    s.n_fixed = n;
+    s.out = &c->chk_acc.p->out;
+    s.terrain_all = 1;
+    s.blocks_done = &c->chk_acc.p->blocks_done;
+    s.h_rep = c->chk_rep.d;
+    s.token = ++c->chk_token;
+    std::atomic_thread_fence(std::memory_order_seq_cst);
+    {
+        KernelTimer t(c, 1);
+        LAUNCH(c, launch_sepcheck_cells(s, 1, n, c->stream));
+        t.stop();
+    }
+    volatile CheckReport* rep = c->chk_rep.p;
+    for (int spin = 1; rep->token != s.token; ++spin) {
+        if (spin % 4096) continue;
+        const cudaError_t e = cudaStreamQuery(c->stream);  // a failed launch never writes the token
+        if (e == cudaErrorNotReady) continue;
+        CK(e);
+        require(rep->token == s.token, FMDP_ERR_CUDA, "internal: the separation check wrote no report");
+    }
+    std::atomic_thread_fence(std::memory_order_acquire);
+    const SepOut out = c->chk_rep.p->out;
+    if (c->profiling) {
+        CK(cudaStreamSynchronize(c->stream));
+        collect_timers(c);
+    }
+    return out;
+}
+
 // Enqueue rollout -> sep_check -> admission for n requests (device array c->reqs, slots in
 // c->slots) in FCFS order on the context's stream.
 void enqueue_sequence(fmdp_ctx* c, SeqBuffers& B, const fmdp_request* host_reqs, int32_t n, int32_t cap,
@@ -373,7 +455,7 @@ void enqueue_sequence(fmdp_ctx* c, SeqBuffers& B, const fmdp_request* host_reqs,
         sa.out = B.sepo.p + i;
         {
             KernelTimer t(c, 1);
-            LAUNCH(c, launch_sepcheck(sa, 1, cap, c->stream));
+            launch_check(c, sa, cap);
             t.stop();
         }
         AdmitArgs aa{};
@@ -559,6 +641,7 @@ void destroy_ctx(fmdp_ctx* c) {
                     (void*)c->items_ctr})
         if (p) cudaFree(p);
     c->seq.release(); c->stg.release(); c->bat.release();
+    c->chk_xyz.release(); c->chk_rep.release(); c->chk_acc.release();
     c->mlp_p.release(); c->mlp_g.release(); c->mlp_m1.release(); c->mlp_m2.release(); c->mlp_wt.release();
     c->mlp_wp.release(); c->tX.release(); c->ty.release(); c->trX.release(); c->trH.release(); c->trdZ.release();
     c->trZ.release(); c->trdZf.release(); c->trdH.release(); c->tr_loss.release(); c->tr_idx.release();

@@ -64,7 +64,7 @@ extern "C" fmdp_status fmdp_sep_check_noalloc(fmdp_ctx* c, int64_t t0_step, cons
         sa.out = &d->acc;
         {
             KernelTimer t(c, 1);
-            LAUNCH(c, launch_sepcheck(sa, 1, n, c->stream));
+            launch_check(c, sa, n);
             t.stop();
         }
         SepOut so;

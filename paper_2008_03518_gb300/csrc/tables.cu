@@ -99,19 +99,21 @@ __global__ void __launch_bounds__(kSepThreads) sepcheck_kernel(const __grid_cons
     }
 }
 
+__device__ __forceinline__ SepOut sep_none() {  // a report before any pair
+    SepOut o;
+    o.first_conflict = INT_MAX;
+    o.first_terrain = INT_MAX;
+    o.conflicts = 0ull;
+    o.min_h_bits = 0x7f800000u;
+    o.min_v_bits = 0x7f800000u;
+    o.verdict = -1;
+    o.pad = 0;
+    return o;
+}
+
 __global__ void sep_reset_kernel(SepOut* out, int n) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) {
-        SepOut o;
-        o.first_conflict = INT_MAX;
-        o.first_terrain = INT_MAX;
-        o.conflicts = 0ull;
-        o.min_h_bits = 0x7f800000u;
-        o.min_v_bits = 0x7f800000u;
-        o.verdict = -1;
-        o.pad = 0;
-        out[i] = o;
-    }
+    if (i < n) out[i] = sep_none();
 }
 
 // FCFS admission (Sec. V): the verdict of request r is decided on the device from its
@@ -218,18 +220,17 @@ cudaError_t launch_admit(const AdmitArgs& a, int n_req, int max_points, cudaStre
     return cudaSuccess;
 }
 
-// Row-major separation check (batch waves). Each block gathers the work items' samples at
-// its step into shared memory, one thread per sample, then streams the row's plan samples
-// through shared memory in tiles; a thread keeps its sample's count, minima and conflict
-// flag in registers (the minimum horizontal distance as a squared distance: the square
-// root is monotone, so the root of the minimum is the minimum of the roots) and folds them
-// into its request's report once at the end.
+// Row-major separation check of a batch without the spatial index. Each block gathers the
+// work items' samples at its step into shared memory, one thread per sample, then streams
+// the row of the table planes through shared memory in tiles; a thread keeps its sample's
+// count, minima and conflict flag in registers (the minimum horizontal distance as a squared
+// distance: the square root is monotone, so the root of the minimum is the minimum of the
+// roots) and folds them into its request's report once at the end.
 constexpr int kRowThreads = 256;
 constexpr int kRowTile = 2048;
 
 size_t sepcheck_rows_smem(int n_max) {
-    return (size_t)kRowTile * (sizeof(float4) + sizeof(int)) + (size_t)n_max * (sizeof(float4) + 3 * sizeof(int)) +
-           16;
+    return (size_t)kRowTile * sizeof(float4) + (size_t)n_max * (sizeof(float4) + 2 * sizeof(int)) + 16;
 }
 
 __global__ void __launch_bounds__(kRowThreads) sepcheck_rows_kernel(const __grid_constant__ SepRowsArgs a) {
@@ -238,14 +239,11 @@ __global__ void __launch_bounds__(kRowThreads) sepcheck_rows_kernel(const __grid
     float4* pts = tile + kRowTile;
     int* pr = reinterpret_cast<int*>(pts + a.n_max);
     int* pk = pr + a.n_max;
-    int* po = pk + a.n_max;       // ordinal of the sample's request (ordinal filter)
-    int* tord = po + a.n_max;     // [kRowTile] ordinal of the tile's items' slots
-    int* npts_s = tord + kRowTile;
+    int* npts_s = pk + a.n_max;
     const int tid = threadIdx.x, NT = blockDim.x;
     const int32_t W = a.tab.T_win;
     const int64_t T = a.tab.t_base + a.row0 + blockIdx.x;
-    int64_t row = T % W;
-    if (row < 0) row += W;
+    const int64_t row = ring_row(T, W);
     if (tid == 0) *npts_s = 0;
     __syncthreads();
     const int n = *a.n_dev;
@@ -261,7 +259,6 @@ __global__ void __launch_bounds__(kRowThreads) sepcheck_rows_kernel(const __grid
             pts[q] = make_float4(p[0], p[1], p[2], 0.f);
             pr[q] = r;
             pk[q] = k;
-            po[q] = a.slot_ord ? a.req_ord[r] : 0;
         }
     }
     __syncthreads();
@@ -269,26 +266,13 @@ __global__ void __launch_bounds__(kRowThreads) sepcheck_rows_kernel(const __grid
     if (npts == 0) return;
     const Model& m = a.m;
     const SepConsts sk = sep_consts(m.sep_h, m.sep_v);
-    // terrain collision of each sample (fp32 outside a band, FP64 inside)
     if (m.hm) {
         for (int q = tid; q < npts; q += NT) {
             const float4 P = pts[q];
-            const float c = P.z - terrain32(m, P.x, P.y);
-            bool below = c < 0.f;
-            if (fabsf(c) < kTerrBand) below = below_terrain_exact(m, P.x, P.y, P.z);
-            if (below) atomicMin(&a.out[pr[q]].first_terrain, pk[q]);
+            if (below_terrain(m, P.x, P.y, P.z)) atomicMin(&a.out[pr[q]].first_terrain, pk[q]);
         }
     }
-    // plan samples of the row: index items (one per finite sample) or the table planes
-    int nslots;
-    const float4* it = nullptr;
-    if (a.items) {
-        const int32_t* cs_row = a.cstart + row * (int64_t)(a.ncell + 1);
-        nslots = cs_row[a.ncell] + a.nextra[row];
-        it = a.items + (size_t)row * a.tab.S_pad * 2;
-    } else {
-        nslots = a.S_scan;
-    }
+    const int nslots = a.S_scan;
     const size_t poff = (size_t)row * a.tab.S_pad;
     // thread t: sample pg + t % P of the current group of P samples, slots of group t / P
     // (G = NT / P groups share out each tile); lanes of a warp read the same slot
@@ -298,34 +282,20 @@ __global__ void __launch_bounds__(kRowThreads) sepcheck_rows_kernel(const __grid
         const int q = pg + tid % P, g = tid / P;
         const bool act = g < G;
         const float4 P4 = act ? pts[q] : make_float4(0.f, 0.f, 0.f, 0.f);
-        const int my_ord = act ? po[q] : 0;
-        const bool filt = a.slot_ord != nullptr && it != nullptr;
         unsigned cnt = 0;
         float minh2 = INFINITY, minv = INFINITY;
         for (int s0 = 0; s0 < nslots; s0 += kRowTile) {
             const int tn = min(kRowTile, nslots - s0);
             __syncthreads();
             for (int j = tid; j < tn; j += NT) {
-                if (it) {
-                    const float4 Q = it[2 * (size_t)(s0 + j)];
-                    tile[j] = Q;
-                    if (filt) {  // the ordinal of the item's plan: a stored plan's slot ordinal, a
-                                 // tentative plan's own; a withdrawn item is never counted
-                        const int tag = __float_as_int(Q.w);
-                        tord[j] = tag >= 0 ? ((unsigned)tag < (unsigned)a.tab.S_pad ? a.slot_ord[tag] : INT_MIN)
-                                           : (tag == kTagDead ? INT_MAX : -tag - 2);
-                    }
-                } else {
-                    const size_t o = poff + s0 + j;
-                    tile[j] = make_float4(a.tab.X[o], a.tab.Y[o], a.tab.Z[o], 0.f);
-                }
+                const size_t o = poff + s0 + j;
+                tile[j] = make_float4(a.tab.X[o], a.tab.Y[o], a.tab.Z[o], 0.f);
             }
             __syncthreads();
             if (act) {
 #pragma unroll 4
                 for (int j = g; j < tn; j += G) {
                     const float4 Q = tile[j];
-                    if (filt && tord[j] >= my_ord) continue;  // admitted after this request
                     float h2, dz;
                     bool hin, vin;
                     sep_pair(sk, P4.x, P4.y, P4.z, Q.x, Q.y, Q.z, h2, dz, hin, vin);
@@ -349,6 +319,367 @@ __global__ void __launch_bounds__(kRowThreads) sepcheck_rows_kernel(const __grid
     }
 }
 
+// Separation check against the spatial index.
+//
+// What the report needs of a row is every pair inside the horizontal minimum (conflicts, the
+// least vertical separation) and the least horizontal distance among the pairs inside the
+// vertical minimum. Both come from the plans around the sample, so only cells are read: a
+// square that covers the horizontal minimum and, by the row's density, some 64 plan samples
+// (less where a smaller distance is known already); then wider ones while the least distance
+// known for the trajectory is larger than the radius covered. A plan outside the cells read
+// lies farther than that radius (less a margin for the rounding of cell numbers), so it can
+// neither conflict nor lower the minimum: the report is the one of the whole row, bit for
+// bit. Rows of up to kFlatItems items, and the extra list of every row, are read whole.
+// One warp reads a sample's first square. Bound by the latency of its dependent loads (row
+// header, cell starts, items).
+constexpr int kCellThreads = 256;
+constexpr int kCellWarps = kCellThreads / 32;
+constexpr int kFlatItems = 96;
+constexpr int kWholeItems = 1024;
+constexpr float kTargetItems = 64.f;
+
+// Cells of the square of half side q around a sample at offset (ux, uy) from the grid's
+// corner, and the radius within which every plan outside the extra list lies in one of them
+// (infinite when they are all the cells).
+struct CellSquare {
+    int x0, x1, y0, y1;
+    float far;
+};
+__device__ __forceinline__ CellSquare cell_square(const IndexView& iv, float ux, float uy, float q, float cell,
+                                                  float margin) {
+    CellSquare c;
+    auto cell_at = [&](float u, int n) { return (int)fminf(fmaxf(floorf(u * iv.inv_cell), 0.f), (float)(n - 1)); };
+    c.x0 = cell_at(ux - q, iv.ncx);
+    c.x1 = cell_at(ux + q, iv.ncx);
+    c.y0 = cell_at(uy - q, iv.ncy);
+    c.y1 = cell_at(uy + q, iv.ncy);
+    const float left = c.x0 > 0 ? ux - (float)c.x0 * cell : INFINITY;
+    const float right = c.x1 < iv.ncx - 1 ? (float)(c.x1 + 1) * cell - ux : INFINITY;
+    const float down = c.y0 > 0 ? uy - (float)c.y0 * cell : INFINITY;
+    const float up = c.y1 < iv.ncy - 1 ? (float)(c.y1 + 1) * cell - uy : INFINITY;
+    c.far = fminf(fminf(left, right), fminf(down, up)) - margin;
+    return c;
+}
+
+// One warp's (or block's) reading of plan samples around a trajectory sample; the minima and
+// the count are each lane's own.
+struct CellScan {
+    const SepCellsArgs& a;
+    const IndexView& iv;
+    const SepConsts sk;
+    const float cell, margin, q_sep;  // q_sep: a square of this half side holds every pair inside the minimum
+    const int lane;
+    float px, py, pz;
+    int my_ord;
+    const int32_t* cs;    // the row's cell starts
+    const float4* items;  // the row's items
+    int64_t row;
+    float minh2, minv;
+    unsigned cnt;
+
+    __device__ __forceinline__ explicit CellScan(const SepCellsArgs& args)
+        : a(args), iv(args.iv), sk(sep_consts(args.m.sep_h, args.m.sep_v)), cell(1.f / args.iv.inv_cell),
+          margin(0.5f + 1e-6f * (float)(args.iv.ncx + args.iv.ncy) * cell),
+          q_sep((float)args.m.sep_h * 1.000001f + 1.f + 2.f * margin), lane(threadIdx.x & 31), my_ord(0),
+          minh2(INFINITY), minv(INFINITY), cnt(0u) {}
+    __device__ __forceinline__ void sample(float x, float y, float z, int64_t ring) {
+        px = x, py = y, pz = z;
+        row = ring;
+        cs = iv.cstart + ring * ((int64_t)iv.ncell + 1);
+        items = iv.items + (size_t)ring * a.tab.S_pad * 2;
+    }
+    __device__ __forceinline__ void test(const float4 Q, bool counted) {
+        float h2, dz;
+        bool hin, vin;
+        sep_pair(sk, px, py, pz, Q.x, Q.y, Q.z, h2, dz, hin, vin);
+        if (!(hin || (vin && h2 < minh2))) return;
+        if (a.slot_ord) {  // the ordinal of the item's plan: a stored plan's slot ordinal, a tentative
+                           // plan's own; plans admitted after this request, and withdrawn items, are
+                           // not part of its table
+            const int tag = __float_as_int(Q.w);
+            const int ord = tag >= 0 ? ((unsigned)tag < (unsigned)a.tab.S_pad ? a.slot_ord[tag] : INT_MIN)
+                                     : (tag == kTagDead ? INT_MAX : -tag - 2);
+            if (ord >= my_ord) return;
+        }
+        if (vin) minh2 = fminf(minh2, h2);
+        if (hin) {
+            minv = fminf(minv, dz);
+            if (vin && counted) ++cnt;
+        }
+    }
+    // Reads the cells of a square (one warp): up to 32 cell rows at a time, one per lane, whose
+    // items the lanes share out as one flat list.
+    __device__ __forceinline__ void read_square(const CellSquare& c, bool counted) {
+        const float4 none = make_float4(__int_as_float(0x7fc00000), 0.f, __int_as_float(0x7fc00000), 0.f);
+        for (int yb = c.y0; yb <= c.y1; yb += 32) {
+            int beg = 0, num = 0;
+            if (yb + lane <= c.y1) {
+                const int32_t* e = cs + (yb + lane) * iv.ncx;
+                beg = e[c.x0];
+                num = e[c.x1 + 1] - beg;
+            }
+            int at = num;  // inclusive prefix of the rows' item counts
+            for (int o = 1; o < 32; o <<= 1) {
+                const int y = __shfl_up_sync(0xffffffffu, at, o);
+                if (lane >= o) at += y;
+            }
+            const int total = __shfl_sync(0xffffffffu, at, 31);
+            const int base = beg - (at - num);  // item i of the flat list: base of its row + i
+            constexpr int U = 4;                // items in flight per lane
+            for (int i0 = 0; i0 < total; i0 += 32 * U) {
+                float4 Q[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const int i = i0 + u * 32 + lane;
+                    int lo = 0;  // the row of item i: the first whose prefix exceeds i
+#pragma unroll
+                    for (int o = 16; o; o >>= 1) lo += __shfl_sync(0xffffffffu, at, lo + o - 1) <= i ? o : 0;
+                    const int b = __shfl_sync(0xffffffffu, base, lo);
+                    Q[u] = i < total ? items[2 * (size_t)(b + i)] : none;
+                }
+#pragma unroll
+                for (int u = 0; u < U; ++u) test(Q[u], counted);
+            }
+        }
+    }
+    // The first square of the sample (one warp), with the squared distance known so far;
+    // returns the radius covered.
+    __device__ __forceinline__ float first_square(float bound2) {
+        const int built = cs[iv.ncell], extra = iv.nextra[row];
+        const bool flat = built + extra <= kFlatItems;  // (the extra list follows the cells' items)
+        for (int i = (flat ? 0 : built) + lane; i < built + extra; i += 32) test(items[2 * (size_t)i], true);
+        if (flat) return INFINITY;
+        // half the side of a square of kTargetItems samples at the row's mean density
+        const float dens = 0.5f * cell * sqrtf(kTargetItems * (float)iv.ncell / (float)max(built, 1));
+        const CellSquare c = cell_square(iv, px - iv.x0, py - iv.y0,
+                                         fmaxf(q_sep, fminf(dens, sqrtf(bound2) + 2.f * margin)), cell, margin);
+        read_square(c, true);
+        return c.far;
+    }
+    // More cells, when a square of radius `far` may leave out a distance below the bound: those up
+    // to the bound; while there is none, all of a row of up to kWholeItems items (one round of
+    // loads in flight beats the rounds of growing squares), else a square three times as wide.
+    __device__ __forceinline__ float wider_square(float far, float bound2) {
+        const int built = cs[iv.ncell];
+        if (bound2 == INFINITY && built <= kWholeItems) {
+#pragma unroll 8
+            for (int i = lane; i < built; i += 32) test(items[2 * (size_t)i], false);
+            return INFINITY;
+        }
+        const CellSquare c =
+            cell_square(iv, px - iv.x0, py - iv.y0,
+                        fminf(sqrtf(bound2) * 1.000001f, 3.f * fmaxf(far, cell)) + 2.f * margin, cell, margin);
+        read_square(c, false);
+        return c.far;
+    }
+    __device__ __forceinline__ float least2() {  // the warp's least squared distance
+        return __uint_as_float(__reduce_min_sync(0xffffffffu, __float_as_uint(minh2)));
+    }
+};
+
+// squared distance bound of a report in progress (other warps lower it), rounded up
+__device__ __forceinline__ float known_bound2(const SepOut* out) {
+    const float h = __uint_as_float(*(const volatile uint32_t*)&out->min_h_bits);
+    return h * h * 1.000001f;
+}
+
+// One trajectory: one warp per sample. After its samples' first squares a block publishes the
+// least distance along them; a sample reads more only where the least distance that any
+// block has published by then is larger than the radius it covered.
+// 100 000 known plans, 1791 samples: 997 us with sepcheck_kernel, which reads every slot of the
+// table (6 % of them hold a sample); the whole call now takes 20 us (1000 us).
+__global__ void __launch_bounds__(kCellThreads) sepcheck_cells_kernel(const __grid_constant__ SepCellsArgs a) {
+    __shared__ unsigned s_minh, s_minv, s_cnt;  // minima as float bits (non-negative: ordered as integers)
+    __shared__ int s_first, s_terr;
+    const int w = blockIdx.y;
+    if (a.n_dev && w >= *a.n_dev) return;
+    const int r = a.idx ? a.idx[w] : w;
+    if (a.skip && a.skip[r]) return;
+    const int n = a.rout ? a.rout[r].n_points : a.n_fixed;
+    if ((int)blockIdx.x * kCellWarps >= n) return;  // (the whole block)
+    const int lane = threadIdx.x & 31;
+    const int k = blockIdx.x * kCellWarps + (threadIdx.x >> 5);  // the warp's sample
+    const int64_t T = (a.reqs ? a.reqs[r].depart_step : a.t0_fixed) + k;
+    const Model& m = a.m;
+    SepOut* out = a.out + r;
+    if (threadIdx.x == 0) {
+        s_first = s_terr = INT_MAX;
+        s_cnt = 0u;
+        s_minh = s_minv = 0x7f800000u;
+    }
+    CellScan S(a);
+    S.my_ord = a.slot_ord ? a.req_ord[r] : 0;
+    int terr = INT_MAX;
+    float far = INFINITY;
+    __syncthreads();
+    if (k < n) {
+        const float* p = a.traj + ((size_t)r * a.cap + k) * 3;
+        const float px = p[0], py = p[1], pz = p[2];
+        const bool held = T >= a.tab.t_base && T < a.tab.t_base + a.tab.T_win;
+        if (held) {
+            S.sample(px, py, pz, ring_row(T, a.tab.T_win));
+            far = S.first_square(known_bound2(out));
+        }
+        if (m.hm && (held || a.terrain_all) && lane == 0 && below_terrain(m, px, py, pz)) terr = k;
+        const float least = S.least2();
+        if (lane == 0) atomicMin(&s_minh, __float_as_uint(least));
+    }
+    __syncthreads();
+    if (threadIdx.x == 0 && s_minh < 0x7f800000u)
+        atomicMin(&out->min_h_bits, __float_as_uint(sqrtf(__uint_as_float(s_minh))));
+    float bound2 = __uint_as_float(s_minh);
+    __syncthreads();
+    if (far * far < bound2) {  // (the same in every lane)
+        bound2 = fminf(bound2, __shfl_sync(0xffffffffu, known_bound2(out), 0));
+        while (far < INFINITY && far * far < bound2) {
+            far = S.wider_square(far, bound2);
+            bound2 = fminf(bound2, S.least2());
+        }
+    }
+    // block reduction, then one atomic per block and quantity
+    terr = __reduce_min_sync(0xffffffffu, terr);
+    const unsigned cnt = __reduce_add_sync(0xffffffffu, S.cnt);
+    const unsigned uh = __float_as_uint(S.least2());
+    const unsigned uv = __reduce_min_sync(0xffffffffu, __float_as_uint(S.minv));
+    if (lane == 0) {
+        if (cnt) {
+            atomicAdd(&s_cnt, cnt);
+            atomicMin(&s_first, k);
+        }
+        if (terr != INT_MAX) atomicMin(&s_terr, terr);
+        atomicMin(&s_minh, uh);
+        atomicMin(&s_minv, uv);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        if (s_cnt) {
+            atomicAdd(&out->conflicts, (unsigned long long)s_cnt);
+            atomicMin(&out->first_conflict, s_first);
+        }
+        if (s_terr != INT_MAX) atomicMin(&out->first_terrain, s_terr);
+        if (s_minh < 0x7f800000u) atomicMin(&out->min_h_bits, __float_as_uint(sqrtf(__uint_as_float(s_minh))));
+        if (s_minv < 0x7f800000u) atomicMin(&out->min_v_bits, s_minv);
+        if (a.h_rep) {
+            __threadfence();
+            if (atomicAdd(a.blocks_done, 1) == (int)gridDim.x - 1) {  // every block has added its part
+                __threadfence();
+                const volatile SepOut* v = out;
+                SepOut o;
+                o.first_conflict = v->first_conflict;
+                o.first_terrain = v->first_terrain;
+                o.conflicts = v->conflicts;
+                o.min_h_bits = v->min_h_bits;
+                o.min_v_bits = v->min_v_bits;
+                o.verdict = -1;
+                o.pad = 0;
+                a.h_rep->out = o;
+                *out = sep_none();
+                *a.blocks_done = 0;
+                asm volatile("st.release.sys.global.s32 [%0], %1;" ::"l"(&a.h_rep->token), "r"(a.token) : "memory");
+            }
+        }
+    }
+}
+
+cudaError_t launch_sepcheck_cells(const SepCellsArgs& a, int n_req, int max_points, cudaStream_t s) {
+    if (n_req <= 0 || max_points <= 0) return cudaSuccess;
+    if (n_req > 65535) return cudaErrorInvalidValue;
+    sepcheck_cells_kernel<<<dim3((unsigned)((max_points + kCellWarps - 1) / kCellWarps), (unsigned)n_req), kCellThreads, 0,
+                            s>>>(a);
+    return cudaGetLastError();
+}
+
+// A batch: one block per step, so that the blocks in flight read neighbouring rows. (With
+// consecutive samples of one trajectory per block, as above, every sample touched another row,
+// and the 2.7 GB of items of a 20 000-plan table are some 1300 pages: address translation
+// bounded the check: 7.2 ms for 512 requests, where the kernel that measured every sample
+// against its whole row took 4.1 ms and this one takes 0.31 ms.) The warps share out the row's samples. A sample whose first square leaves out a distance below
+// the least one known waits until the row's other samples are done: by then the blocks of
+// its trajectory's other steps have mostly lowered the bound and nothing is left to read.
+size_t sepcheck_row_cells_smem(int n_max) { return (size_t)n_max * (sizeof(float4) + 3 * sizeof(int)) + 16; }
+
+__global__ void __launch_bounds__(kCellThreads) sepcheck_row_cells_kernel(const __grid_constant__ SepCellsArgs a,
+                                                                          int32_t row0, int32_t n_max) {
+    extern __shared__ __align__(16) unsigned char srm[];
+    float4* pts = reinterpret_cast<float4*>(srm);  // the samples at this step
+    int* pr = reinterpret_cast<int*>(pts + n_max);
+    int* pk = pr + n_max;
+    float* pfar = reinterpret_cast<float*>(pk + n_max);
+    int* npts_s = reinterpret_cast<int*>(pfar + n_max);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int64_t T = a.tab.t_base + row0 + blockIdx.x;
+    if (tid == 0) *npts_s = 0;
+    __syncthreads();
+    const int n = *a.n_dev;
+    for (int w = tid; w < n; w += kCellThreads) {
+        const int r = a.idx[w];
+        if (a.skip && a.skip[r]) continue;
+        const int64_t d = a.reqs[r].depart_step;
+        if (T >= d && T < d + a.rout[r].n_points) {
+            const int q = atomicAdd(npts_s, 1);
+            const int k = (int)(T - d);
+            const float* p = a.traj + ((size_t)r * a.cap + k) * 3;
+            pts[q] = make_float4(p[0], p[1], p[2], 0.f);
+            pr[q] = r;
+            pk[q] = k;
+        }
+    }
+    __syncthreads();
+    const int npts = *npts_s;
+    if (npts == 0) return;
+    const Model& m = a.m;
+    if (m.hm)
+        for (int q = tid; q < npts; q += kCellThreads)
+            if (below_terrain(m, pts[q].x, pts[q].y, pts[q].z)) atomicMin(&a.out[pr[q]].first_terrain, pk[q]);
+    const int64_t row = ring_row(T, a.tab.T_win);
+    CellScan S(a);
+    auto fold = [&](SepOut* out, int k, float known2) {  // the sample's minima and conflicts into its report
+        const unsigned cnt = __reduce_add_sync(0xffffffffu, S.cnt);
+        const float h2 = S.least2();
+        const unsigned v = __reduce_min_sync(0xffffffffu, __float_as_uint(S.minv));
+        if (lane == 0) {
+            if (cnt) {
+                atomicAdd(&out->conflicts, (unsigned long long)cnt);
+                atomicMin(&out->first_conflict, k);
+            }
+            if (h2 < known2) atomicMin(&out->min_h_bits, __float_as_uint(sqrtf(h2)));
+            if (v < 0x7f800000u) atomicMin(&out->min_v_bits, v);
+        }
+        return h2;
+    };
+    auto begin = [&](int q) {
+        const float4 P = pts[q];
+        S.sample(P.x, P.y, P.z, row);
+        S.my_ord = a.slot_ord ? a.req_ord[pr[q]] : 0;
+        S.minh2 = S.minv = INFINITY;
+        S.cnt = 0u;
+    };
+    for (int q = warp; q < npts; q += kCellWarps) {
+        SepOut* out = a.out + pr[q];
+        const float known2 = known_bound2(out);
+        begin(q);
+        const float far = S.first_square(known2);
+        fold(out, pk[q], known2);
+        if (lane == 0) pfar[q] = far;
+    }
+    __syncwarp();
+    for (int q = warp; q < npts; q += kCellWarps) {
+        float far = pfar[q];
+        if (far == INFINITY) continue;
+        SepOut* out = a.out + pr[q];
+        float bound2 = __shfl_sync(0xffffffffu, known_bound2(out), 0);
+        if (far * far >= bound2) continue;
+        const float known2 = bound2;
+        begin(q);
+        while (far < INFINITY && far * far < bound2) {
+            far = S.wider_square(far, bound2);
+            bound2 = fminf(bound2, S.least2());
+        }
+        S.cnt = 0u;  // (the first square counted the conflicts)
+        fold(out, pk[q], known2);
+    }
+}
+
 cudaError_t prepare_sepcheck_rows(size_t smem) {
     return cudaFuncSetAttribute(sepcheck_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
 }
@@ -356,6 +687,24 @@ cudaError_t prepare_sepcheck_rows(size_t smem) {
 cudaError_t launch_sepcheck_rows(const SepRowsArgs& a, cudaStream_t s) {
     const int32_t rows = a.nrows > 0 ? a.nrows : a.tab.T_win;
     if (a.row0 < 0 || a.row0 + rows > a.tab.T_win) return cudaErrorInvalidValue;
+    if (a.iv.items) {
+        SepCellsArgs c{};
+        c.m = a.m;
+        c.tab = a.tab;
+        c.iv = a.iv;
+        c.traj = a.traj;
+        c.cap = a.cap;
+        c.rout = a.rout;
+        c.reqs = a.reqs;
+        c.idx = a.idx;
+        c.n_dev = a.n_dev;
+        c.skip = a.skip;
+        c.slot_ord = a.slot_ord;
+        c.req_ord = a.req_ord;
+        c.out = a.out;
+        sepcheck_row_cells_kernel<<<(unsigned)rows, kCellThreads, sepcheck_row_cells_smem(a.n_max), s>>>(c, a.row0, a.n_max);
+        return cudaGetLastError();
+    }
     sepcheck_rows_kernel<<<(unsigned)rows, kRowThreads, sepcheck_rows_smem(a.n_max), s>>>(a);
     return cudaGetLastError();
 }
@@ -495,15 +844,7 @@ __global__ void __launch_bounds__(128) influence_kernel(const __grid_constant__ 
 __global__ void sep_reset_idx_kernel(SepOut* out, const int32_t* idx, const int32_t* n_dev, int n_max) {
     const int w = blockIdx.x * blockDim.x + threadIdx.x;
     if (w >= n_max || w >= *n_dev) return;
-    SepOut o;
-    o.first_conflict = INT_MAX;
-    o.first_terrain = INT_MAX;
-    o.conflicts = 0ull;
-    o.min_h_bits = 0x7f800000u;
-    o.min_v_bits = 0x7f800000u;
-    o.verdict = -1;
-    o.pad = 0;
-    out[idx[w]] = o;
+    out[idx[w]] = sep_none();
 }
 
 cudaError_t launch_influence(const InfluenceArgs& a, int n_max, int /*max_points*/, cudaStream_t s) {
@@ -560,6 +901,8 @@ cudaError_t preload_table_kernels() {
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, admit_kernel);
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, fill_nan_kernel);
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, sepcheck_rows_kernel);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, sepcheck_cells_kernel);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, sepcheck_row_cells_kernel);
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, batch_minsep_kernel);
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, influence_kernel);
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, sep_reset_idx_kernel);
