@@ -106,8 +106,9 @@ typedef struct {
     double index_vmax_mps;    /* index: plans faster than this (m/s) are scanned at every
                                  step (0 = 50) */
     double index_cell_m;      /* index: cell edge in metres (0 = automatic) */
-    int32_t index_stage_items; /* index: plan samples a rollout step stages in shared memory
-                                  (0 = 1536; more are read from global memory) */
+    int32_t index_stage_items; /* index: shared memory for plan samples, in samples over the eight
+                                  steps prepared ahead: a step's list holds an eighth (0 = 1536;
+                                  a step with more samples in reach reads them from the index) */
     int32_t batch_mode;       /* fmdp_schedule_batch, staged batches and fmdp_serve:
                                  0 = pipelined where it applies (spatial index, W = 1, FastMDP
                                  rollouts): continuous batching without waves, see
@@ -353,22 +354,23 @@ fmdp_status fmdp_selftest_wait_timeout(fmdp_ctx* ctx, int32_t* observed);
 /* ---- Autotuner of the batched rollout's launch shape (no counterpart in the paper; the
  * rollout is Alg. 1 whatever the shape, and results are bit-identical across shapes).
  *
- * With the spatial index a speculative wave runs one CTA per request: a control warp, an
- * evaluator warp, an index producer warp and (threads_per_cta / 32 - 3) scanner warps that
- * share out the plan samples near the state, index_stage_items of them staged in shared
- * memory per step. Fewer scanners and less staging let two or more CTAs share a
+ * With the spatial index a speculative wave runs one CTA per request: a control, a successor
+ * and one or two well-folding warps that form the chain from state to state, a recorder warp
+ * behind it, and warps that prepare the lists of plan samples near the next states ahead of
+ * it (threads_per_cta decides how many); index_stage_items is the shared memory of those
+ * lists. Fewer warps and shorter lists let two or more CTAs share a
  * multiprocessor, which pays when a wave holds more requests than there are
- * multiprocessors; more scanners shorten each step, which is what a small wave (the
+ * multiprocessors; more warps shorten each step, which is what a small wave (the
  * re-plans of a speculative batch) needs. fmdp_autotune times the rollouts of the first W
  * sample requests (nothing is admitted) under every candidate shape, threads per CTA in
- * {128, 192, 256, 320, 384} x staged samples in {512, 1024, 1536, 2048} (those whose
- * staging buffers fit in shared memory), for W = min(n,
+ * {128, 192, 256, 320, 384} x index_stage_items in {512, 1024, 1536, 2048} (those whose
+ * lists fit in shared memory), for W = min(n,
  * batch size) and its halvings down to 8, and caches the fastest shape under the key
  * (n_actions, combine, plan-count bucket, wave-size bucket). Each wave of a batched call in
  * wave mode (fmdp_schedule_batch, fmdp_serve, fmdp_schedule_learned, staged batches) then
  * launches with the cached shape of its key, or of the nearest tuned wave-size bucket. The
  * pipelined mode's persistent launch holds at most one CTA per multiprocessor and takes
- * the widest shape (384 threads, 1536 staged samples). options.threads_per_cta and
+ * the widest shape (384 threads, 1536 samples). options.threads_per_cta and
  * options.index_stage_items, when set, take precedence in both modes. */
 typedef struct {
     int32_t n_actions, combine;
@@ -386,7 +388,7 @@ typedef struct {
     int32_t from_cache;          /* 1: the largest wave's key was cached and nothing was timed */
     int32_t sample;              /* requests in the largest timed wave */
     int32_t reserved;
-    double default_ms;           /* the largest wave at 384 threads and 1536 staged samples */
+    double default_ms;           /* the largest wave at 384 threads and 1536 samples */
 } fmdp_tune_report;
 /* Requires the spatial index (options.full_scan = 0). sample: host requests, at least one;
  * the largest timed wave is the first min(n, batch size). force = 1 re-times cached keys. */
@@ -489,10 +491,12 @@ typedef struct {
     int64_t sep_pairs;                        /* (sample, slot) pairs scanned by sep_check */
     int32_t cluster_size, threads_per_cta, slots_per_cta;
     int32_t reserved;
-    int64_t phase_cycles[6];  /* on = 2: summed SM cycles of rollout phases: control warp waiting
-                                 at the step barrier, control per-action work, control waiting
-                                 for the scanners, exchange + argmax + advance, one scanner
-                                 warp's cull + wells, producer issue + wait */
+    int64_t phase_cycles[6];  /* on = 2: summed SM cycles of rollout phases. Spatial index: control
+                                 warp before successors and wells are ready, 0, its wait for
+                                 them, action values and choice, preparing lists (all list
+                                 warps), recorder. Full scan: control warp waiting at the step
+                                 barrier, per-action work, waiting for the scanners, exchange +
+                                 argmax + advance, one scanner warp's cull + wells, 0 */
     int64_t batch_waves;         /* speculative waves run by fmdp_schedule_batch */
     int64_t batch_rollouts;      /* rollouts run by those waves (first plans and re-plans) */
     int64_t batch_replans;       /* re-plans among them */

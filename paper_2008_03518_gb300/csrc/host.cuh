@@ -349,7 +349,7 @@ struct KernelTimer {
 // launch shape of a rollout
 struct Geometry {
     int32_t S_scan, cs, threads, chunk, ring;
-    int32_t icap = 0;  // indexed mode: plan samples staged per step
+    int32_t icap = 0;  // indexed mode: options.index_stage_items (a step's list holds an eighth of it)
     size_t smem;
 };
 // platform-independent random numbers (splitmix64; Box-Muller normals)
@@ -385,6 +385,7 @@ void grow_keep(fmdp_ctx* c, DevArray<T>& a, size_t want, size_t keep) {
 
 constexpr int32_t kBatchDefault = 256;
 constexpr int32_t kBatchMax = 1024;
+constexpr int32_t kMaxStageItems = 2234;  // options.index_stage_items beyond this are refused when a plan starts
 
 // ------------------------------------------------------------------ host runtime (host_table.cu)
 

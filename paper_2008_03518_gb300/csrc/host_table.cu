@@ -276,7 +276,8 @@ Geometry geometry_indexed(fmdp_ctx* c, int32_t S_scan, int32_t wave) {
     if (c->opt.threads_per_cta > 0) g.threads = c->opt.threads_per_cta;
     if (c->icap_user > 0) g.icap = c->icap_user;
     g.smem = rollout_smem_bytes(0, 0, g.icap);
-    require((int)g.smem <= c->max_smem, FMDP_ERR_ARG, "index staging buffers exceed shared memory");
+    require(g.icap <= kMaxStageItems && (int)g.smem <= c->max_smem, FMDP_ERR_ARG,
+            "index_stage_items exceeds shared memory");
     c->last_cs = 1;
     c->last_threads = g.threads;
     c->last_chunk = 0;

@@ -1,22 +1,24 @@
 // Persistent FastMDP rollout kernel (sm_103a).
 //
-// One thread-block cluster plans one request from departure to capture, horizon or
-// dead end without returning to the host (the paper's CPU loop of Fig. 3 runs nine
-// kernels and a device-to-host copy per step; here the whole loop is one launch).
-//
-// Roles inside each CTA (the CTA owns a contiguous partition of the plan-table slots):
-//   warp 0      control: per-action work that does not depend on other plans (box test,
-//               goal term, terrain clearance, static wells; Alg. 1, Alg. 4, Alg. 6) while
-//               the other warps scan, then the exchange, argmax and state advance;
-//   warps 1..   scanners: stride over the partition's slots of slice t+1 (wells) and t+2
-//               (plan velocity); a slot whose wells cannot reach any successor is culled
-//               with one distance test, and for each near slot the whole warp evaluates
-//               the five wells of Table 3 with lane a scoring action a (Alg. 5-7);
-//   warp 1 l.0  producer: TMA bulk copies of upcoming slices into an 8-deep ring (the
-//               table does not depend on the aircraft, so it runs steps ahead).
-// Per-action maxima of log2(|r| gamma^d) are combined within the CTA by shared-memory
-// atomics and across the cluster by DSMEM pushes (st.async + mbarrier), so no cluster-wide
-// barrier is needed per step.
+// One launch plans requests from departure to capture, horizon or dead end without
+// returning to the host (the paper's CPU loop of Fig. 3 runs nine kernels and a
+// device-to-host copy per step). Two forms, with the same results:
+//   indexed    (the default) one CTA per request reads the plans near its state from the
+//              spatial index: plan_indexed.cuh;
+//   full scan  (option full_scan, below) one thread-block cluster per request streams every
+//              slot of each step. Roles inside each CTA, which owns a contiguous partition
+//              of the plan-table slots:
+//     warp 0      control: the successor of every action, then the exchange, argmax and
+//                 state advance;
+//     warp 1      evaluator: per-action terms that do not depend on other plans (box test,
+//                 goal term, terrain clearance, static wells; Alg. 1, Alg. 4, Alg. 6); its
+//                 lane 0 is the producer: TMA bulk copies of upcoming slices into a ring;
+//     warps 2..   scanners: a slot whose wells cannot reach any successor is culled with one
+//                 distance test, and for each near slot the whole warp evaluates the wells of
+//                 Table 3 with lane a scoring action a (Alg. 5-7).
+//   Per-action maxima of log2(|r| gamma^d) are combined within the CTA by shared-memory
+//   atomics and across the cluster by DSMEM pushes (st.async + mbarrier), so no cluster-wide
+//   barrier is needed per step.
 //
 // Numerics. GB300 executes FP64 at 1/64 of the FP32 rate with ~63-cycle latency, so the
 // serial per-step chain is FP32: the state is carried as an exact FP64 triple (advanced by
@@ -99,10 +101,6 @@ __device__ __forceinline__ uint32_t cluster_rank() {
     asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
     return r;
 }
-// named CTA barrier over `threads` threads (a multiple of 32, whole warps)
-__device__ __forceinline__ void named_barrier(int id, int threads) {
-    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
-}
 __device__ __forceinline__ void cluster_barrier() {
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
@@ -152,7 +150,11 @@ __device__ __forceinline__ void df_add(float& hi, float& lo, float dh, float dl)
     e = __fadd_rn(e, __fadd_rn(lo, dl));
     fast_two_sum(s, e, hi, lo);
 }
-__device__ __forceinline__ float approx_sqrt(float x) { return x > 0.f ? x * rsqrtf(x) : 0.f; }
+// a . b, the z product fused last and the y product rounded
+__device__ __forceinline__ float dot3(float ax, float ay, float az, float bx, float by, float bz) {
+    return fmaf(az, bz, fmaf(ax, bx, __fmul_rn(ay, by)));
+}
+__device__ __forceinline__ float approx_sqrt(float x) { return x > 0.f ? __fmul_rn(x, rsqrtf(x)) : 0.f; }
 
 struct StepState {
     float wlim2[kMaxWells];  // per well: (R + largest successor offset + 1 m)^2, the reach test
@@ -177,35 +179,17 @@ struct StepState {
     int last_best[2];   // action chosen at step k (99: none), by k & 1
 };
 
-// Shared-memory carve-up (identical on host and device).
-// Indexed mode: what one staging buffer holds. The first n_s of the `total` items are in
-// shared memory; the rest are read from the index in global memory through the ranges.
-constexpr int kMaxRanges = 8;
-struct IdxMeta {
-    int total, n_s, nr;
-    int pub;  // pipelined mode: admissions published when the extra list's length was read
-    long long row_off;  // first float4 of the row's items
-    int beg[kMaxRanges], cnt[kMaxRanges];
-};
-constexpr int kIBufs = 3;  // staging buffers: the step being scanned and the next two
-
+// Shared-memory carve-up of the full-scan form (identical on host and device).
 struct Layout {
-    size_t ring, ibuf, imeta, bars, xbar, st, tabs, keys, sums, xkeys, xsums, xab, stat, aux, misc, total;
+    size_t ring, bars, xbar, st, tabs, keys, sums, xkeys, xsums, xab, stat, aux, misc, total;
 };
-// chunk, depth: full-scan slice ring (chunk = 0 in indexed mode); icap: indexed staging
-// buffer capacity in items (0 in full-scan mode)
-__host__ __device__ inline Layout make_layout(int chunk, int depth, int icap) {
+// chunk, depth: the slice ring
+__host__ __device__ inline Layout make_layout(int chunk, int depth) {
     Layout L;
     size_t o = 0;
     auto al = [&](size_t a) { o = (o + a - 1) & ~(a - 1); };
     L.ring = o;
     o += (size_t)depth * 3 * chunk * sizeof(float);
-    al(128);
-    L.ibuf = o;  // [kIBufs][icap] items of two float4
-    o += icap > 0 ? (size_t)kIBufs * icap * 2 * sizeof(float4) : 0;
-    al(16);
-    L.imeta = o;
-    o += icap > 0 ? kIBufs * sizeof(IdxMeta) : 0;
     al(16);
     L.bars = o;
     o += kRingDepth * sizeof(uint64_t);
@@ -234,22 +218,20 @@ __host__ __device__ inline Layout make_layout(int chunk, int depth, int icap) {
     L.stat = o;  // static-well centres as double-float: hi[64][3], lo[64][3]
     o += 2 * kMaxStatic * 3 * sizeof(float);
     al(16);
-    L.aux = o;   // valid, Delta, deck, goal term; key, class, log2|Q|, log2 scale by step parity
-    o += 12 * kMaxActions * sizeof(int);
-    L.misc = o;  // work-queue slot of the persistent batch mode; pipelined mode: [0..3] the
-                 // item taken, [4..6] the tail check's first conflict and terrain sample and
-                 // the admissions published before it read the index, [8..9] the item's window
-    o += 48;
+    L.aux = o;   // valid, Delta, deck; key, class, log2|Q|, log2 scale by step parity
+    o += 11 * kMaxActions * sizeof(int);
+    L.misc = o;  // work-queue slot of the persistent batch mode
+    o += 16;
     L.total = (o + 127) & ~size_t(127);
     return L;
 }
 
 
 // Exact (FP64, method order) well-edge decision for a plan well.
-__device__ __noinline__ bool well_inside_exact(const Model& m, const StepState* st, double Dx, double Dy,
+__device__ __noinline__ bool well_inside_exact(const Model& m, const double* s, double Dx, double Dy,
                                                double Dz, float p1x, float p1y, float p1z, float p2x, float p2y,
                                                float p2z, bool has2, int w) {
-    const double x = __dadd_rn(st->s[0], Dx), y = __dadd_rn(st->s[1], Dy), z = __dadd_rn(st->s[2], Dz);
+    const double x = __dadd_rn(s[0], Dx), y = __dadd_rn(s[1], Dy), z = __dadd_rn(s[2], Dz);
     double vx = 0.0, vy = 0.0, vz = 0.0;
     if (has2) {
         vx = __ddiv_rn(__dsub_rn((double)p2x, (double)p1x), m.dt);
@@ -263,20 +245,20 @@ __device__ __noinline__ bool well_inside_exact(const Model& m, const StepState* 
     return norm3_64(__dsub_rn(x, cx), __dsub_rn(y, cy), __dsub_rn(z, cz)) < m.w_R64[w];
 }
 
-__device__ __noinline__ bool static_inside_exact(const Model& m, const StepState* st, double Dx, double Dy,
+__device__ __noinline__ bool static_inside_exact(const Model& m, const double* s, double Dx, double Dy,
                                                  double Dz, int w) {
-    const double x = __dadd_rn(st->s[0], Dx), y = __dadd_rn(st->s[1], Dy), z = __dadd_rn(st->s[2], Dz);
+    const double x = __dadd_rn(s[0], Dx), y = __dadd_rn(s[1], Dy), z = __dadd_rn(s[2], Dz);
     const double* c = m.statics + 6 * w;
     return norm3_64(__dsub_rn(x, c[0]), __dsub_rn(y, c[1]), __dsub_rn(z, c[2])) < c[3];
 }
 
-__device__ __noinline__ bool box_inside_exact(const Model& m, const StepState* st, double Dx, double Dy, double Dz) {
-    const double x = __dadd_rn(st->s[0], Dx), y = __dadd_rn(st->s[1], Dy), z = __dadd_rn(st->s[2], Dz);
+__device__ __noinline__ bool box_inside_exact(const Model& m, const double* s, double Dx, double Dy, double Dz) {
+    const double x = __dadd_rn(s[0], Dx), y = __dadd_rn(s[1], Dy), z = __dadd_rn(s[2], Dz);
     return x >= m.box[0] && x <= m.box[3] && y >= m.box[1] && y <= m.box[4] && z >= m.box[2] && z <= m.box[5];
 }
 
-__device__ __noinline__ float deck_exact(const Model& m, const StepState* st, double Dx, double Dy, double Dz) {
-    const double x = __dadd_rn(st->s[0], Dx), y = __dadd_rn(st->s[1], Dy), z = __dadd_rn(st->s[2], Dz);
+__device__ __noinline__ float deck_exact(const Model& m, const double* s, double Dx, double Dy, double Dz) {
+    const double x = __dadd_rn(s[0], Dx), y = __dadd_rn(s[1], Dy), z = __dadd_rn(s[2], Dz);
     const double c = __dsub_rn(z, terrain64(m, x, y));
     return c < m.clearance ? (float)__dsub_rn(m.deck, c) : 0.f;
 }
@@ -296,20 +278,20 @@ __device__ __noinline__ bool capture_exact_at(double x, double y, double z, cons
 __device__ __forceinline__ void goal_log_split(float Ghx, float Ghy, float Ghz, float Glx, float Gly, float Glz,
                                                float lg_hi, float lg_lo, float l2r_hi, float l2r_lo, int& n0,
                                                float& phi) {
-    const float p0 = Ghx * Ghx, p1 = Ghy * Ghy, p2 = Ghz * Ghz;
+    const float p0 = __fmul_rn(Ghx, Ghx), p1 = __fmul_rn(Ghy, Ghy), p2 = __fmul_rn(Ghz, Ghz);
     const float e0 = fmaf(Ghx, Ghx, -p0), e1 = fmaf(Ghy, Ghy, -p1), e2 = fmaf(Ghz, Ghz, -p2);
     float s1, t1, s2, t2;
     two_sum(p0, p1, s1, t1);
     two_sum(s1, p2, s2, t2);
-    const float lo = t1 + t2 + e0 + e1 + e2 + 2.f * (Ghx * Glx + Ghy * Gly + Ghz * Glz);
+    const float lo = fmaf(2.f, dot3(Ghx, Ghy, Ghz, Glx, Gly, Glz), t1 + t2 + e0 + e1 + e2);
     float Sh, Sl;
     fast_two_sum(s2, lo, Sh, Sl);
     const float rt = approx_sqrt(Sh);
     const float rr = fmaf(-rt, rt, Sh);
-    const float rl = rt > 0.f ? (rr + Sl) * (0.5f * rsqrtf(Sh)) : 0.f;
-    const float p = rt * lg_hi;
+    const float rl = rt > 0.f ? __fmul_rn(__fadd_rn(rr, Sl), 0.5f * rsqrtf(Sh)) : 0.f;
+    const float p = __fmul_rn(rt, lg_hi);
     const float pe = fmaf(rt, lg_hi, -p);
-    const float lo2 = pe + rt * lg_lo + rl * lg_hi;
+    const float lo2 = fmaf(rl, lg_hi, fmaf(rt, lg_lo, pe));
     float Lh, Le;
     two_sum(p, l2r_hi, Lh, Le);
     Le = Le + (lo2 + l2r_lo);
@@ -337,7 +319,7 @@ __device__ __noinline__ void fold_statics(const Model& m, const StepState* st, c
         const float d2 = fmaf(ex, ex, fmaf(ey, ey, ez * ez));
         const float R2 = m.st_R2[w], bw = m.st_band[w];
         if (d2 < R2 + bw) {
-            const bool inside = d2 < R2 - bw ? true : static_inside_exact(m, st, Dxh, Dyh, Dza, w);
+            const bool inside = d2 < R2 - bw ? true : static_inside_exact(m, st->s, Dxh, Dyh, Dza, w);
             if (inside) {
                 const float l = fmaf(approx_sqrt(d2), m.st_lg[w], m.st_L[w]);
                 mloc = fmaxf(mloc, l);
@@ -410,6 +392,81 @@ __device__ __forceinline__ unsigned long long sum_term(float l, float ref) {
     return (unsigned long long)__float2ull_rn(t);
 }
 
+// Per-action terms shared by the indexed and the full-scan plan. Sums of products are written
+// with explicit fused operations: left to the compiler, which product of a sum is fused may
+// differ from one inlined copy to the next, and two actions' values often differ by less than
+// that rounding.
+struct TerrainCell {  // heightmap cell under a successor, and the position in it
+    int ix, iy;
+    float ax, ay;
+    float h00, h10, h01, h11;
+};
+__device__ __forceinline__ TerrainCell terrain_cell(float sx, float sy, float box0, float box1, float hm_sx, float hm_sy,
+                                                    int hm_nx, int hm_ny) {
+    TerrainCell t;
+    const float ux = __fsub_rn(sx, box0), uy = __fsub_rn(sy, box1);
+    t.ix = (int)floorf(__fmul_rn(ux, hm_sx)), t.iy = (int)floorf(__fmul_rn(uy, hm_sy));
+    t.ix = min(max(t.ix, 0), hm_nx - 2);
+    t.iy = min(max(t.iy, 0), hm_ny - 2);
+    t.ax = fmaf(ux, hm_sx, -(float)t.ix);
+    t.ay = fmaf(uy, hm_sy, -(float)t.iy);
+    return t;
+}
+__device__ __forceinline__ void terrain_nodes(TerrainCell& t, const float* __restrict__ hm, int hm_nx) {
+    const float* r0 = hm + (size_t)t.iy * hm_nx + t.ix;
+    t.h00 = __ldg(r0);
+    t.h10 = __ldg(r0 + 1);
+    t.h01 = __ldg(r0 + hm_nx);
+    t.h11 = __ldg(r0 + hm_nx + 1);
+}
+__device__ __forceinline__ float terrain_height(const TerrainCell& t) {
+    const float bx = __fsub_rn(1.f, t.ax), by = __fsub_rn(1.f, t.ay);
+    const float lo = fmaf(bx, t.h00, __fmul_rn(t.ax, t.h10)), hi = fmaf(bx, t.h01, __fmul_rn(t.ax, t.h11));
+    return fmaf(by, lo, __fmul_rn(t.ay, hi));
+}
+// least distance of a successor to a box face (negative outside)
+__device__ __forceinline__ float box_margin(float sx, float sy, float sz, float box0, float box1, float box2, float box3,
+                                            float box4, float box5) {
+    const float mlo = fminf(fminf(sx - box0, sy - box1), sz - box2);
+    const float mhi = fminf(fminf(box3 - sx, box4 - sy), box5 - sz);
+    return fminf(mlo, mhi);
+}
+// goal distance change |G - delta| - |G| of a move delta from a state at goal offset G
+__device__ __forceinline__ float goal_change(float Gx, float Gy, float Gz, float dxa, float dya, float dza) {
+    const float Gn = approx_sqrt(dot3(Gx, Gy, Gz, Gx, Gy, Gz));
+    const float fx = __fsub_rn(Gx, dxa), fy = __fsub_rn(Gy, dya), fz = __fsub_rn(Gz, dza);
+    const float da = approx_sqrt(dot3(fx, fy, fz, fx, fy, fz));
+    const float num = fmaf(-2.0f, dot3(Gx, Gy, Gz, dxa, dya, dza), dot3(dxa, dya, dza, dxa, dya, dza));
+    const float den = __fadd_rn(da, Gn);
+    return den > 0.f ? __fdividef(num, den) : 0.f;
+}
+// Action value Q = g - P - V as (sign class, log2 |Q|): g the goal term, Nl = P + V. Without
+// branches: in one warp the divergent forms cost more than computing all of them.
+struct ActionValue {
+    int cls;   // 2: Q > 0, 1: Q = 0, 0: Q < 0
+    float k2;  // larger is better within a class
+    float la;  // log2 |Q|
+};
+__device__ __forceinline__ void action_value(bool combine, bool has_goal, unsigned long long ssum, float Lp, float Vd,
+                                             float sum_unit, float phi, float Dl, float lg32, int n0, float sc0,
+                                             ActionValue& v, float& Nl) {
+    const float lgh = fmaf(Dl, lg32, phi);  // log2(g) - n0
+    const bool pen = (combine ? ssum != 0ull : Lp > -INFINITY) || Vd > 0.f;
+    const float P = combine ? fmaf((float)ssum, sum_unit, Vd) : __fadd_rn(exp2f(Lp), Vd);  // (2^-inf = 0)
+    Nl = pen ? P : 0.f;
+    const float gh = has_goal ? exp2f(lgh) : 0.f;  // g / 2^n0
+    const float Nh = __fmul_rn(Nl, sc0);           // N / 2^n0 (inf when that overflows fp32)
+    const float d = __fsub_rn(gh, Nh);
+    const bool over = !(Nh < INFINITY);            // then log2 |Q| is that of N itself
+    const float lq = __log2f(over ? Nl : fabsf(d));
+    const float fn0 = (float)n0;
+    const float la = __fadd_rn(lq, over ? 0.f : fn0);
+    const bool pos = has_goal && d > 0.f, zero = d == 0.f;
+    v.cls = pen ? (pos ? 2 : (zero ? 1 : 0)) : (has_goal ? 2 : 1);
+    v.k2 = pen ? (pos ? lq : (zero ? 0.f : -la)) : (has_goal ? lgh : 0.f);
+    v.la = pen ? (zero ? -INFINITY : la) : (has_goal ? __fadd_rn(lgh, fn0) : -INFINITY);
+}
+
 // Scores one well of a plan for this lane's action: max-fold of log2(|r| gamma^d).
 __device__ __forceinline__ void fold_well(const StepState* st, int w, float qx, float qy, float qz, float vx,
                                           float vy, float vz, float dxa, float dya, float dza, float& mloc,
@@ -431,24 +488,20 @@ __device__ __forceinline__ void fold_well(const StepState* st, int w, float qx, 
     }
 }
 
+#include "plan_indexed.cuh"
+
 }  // namespace
 
-// Plans request r with this CTA (and its cluster peers). Every thread of the cluster calls
-// it; all shared memory it uses is re-initialised, so a CTA can plan requests back to back.
-// k0 > 0 (pipelined mode): the plan keeps its first k0 steps and resumes from its state at
-// step k0, as stored by the run that planned them. tbase: the first step of the table window
-// the plan reads (the launch's, or in pipelined mode the one its item was dispatched with). IDX: indexed mode (one CTA, no cluster),
-// compiled apart from the full-scan mode so that each step's code stays small; GEN: the
-// general instance, with the uncommon features (the per-phase clock stamps of
-// fmdp_set_profiling(2), the trace of fmdp_rollout_trace, the SUM combination, static wells); without it the
-// step's code holds only the common configuration (the stamps' code alone lengthens a step by
-// about 3 %).
-template <bool IDX, bool GEN>
+// Plans request r with this CTA and its cluster peers (full scan). Every thread of the cluster
+// calls it; all shared memory it uses is re-initialised, so a CTA can plan requests back to
+// back. GEN: the general instance, with the uncommon features (the per-phase clock stamps of
+// fmdp_set_profiling(2), the trace of fmdp_rollout_trace, the SUM combination, static wells).
+template <bool GEN>
 __device__ __forceinline__ void plan_request(const RolloutArgs& a, const int r, unsigned char* smem,
-                                             const int64_t tbase, const int k0 = 0) {
+                                             const int64_t tbase) {
     const Model& m = a.m;
     const int tid = threadIdx.x, NT = blockDim.x, lane = tid & 31, warp = tid >> 5, NW = NT >> 5;
-    const int cs = IDX ? 1 : a.cs;
+    const int cs = a.cs;
     const uint32_t rank = cs > 1 ? cluster_rank() : 0u;
     const fmdp_request req = a.reqs[r];
     const int A = m.A;
@@ -457,12 +510,7 @@ __device__ __forceinline__ void plan_request(const RolloutArgs& a, const int r, 
     const int c_len = max(0, min(chunk, a.S_scan - c_begin));
     const int depth = a.ring;                    // 4 or 8 slices
     const int dshift = depth == 8 ? 3 : 2;
-    constexpr bool indexed = IDX;
-    const int icap = a.icap;
-    const Layout L = make_layout(chunk, depth, indexed ? icap : 0);
-    float4* ibuf = reinterpret_cast<float4*>(smem + L.ibuf);
-    IdxMeta* imeta = reinterpret_cast<IdxMeta*>(smem + L.imeta);
-
+    const Layout L = make_layout(chunk, depth);
     float* ring = reinterpret_cast<float*>(smem + L.ring);
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + L.bars);
     uint64_t* xbar = reinterpret_cast<uint64_t*>(smem + L.xbar);
@@ -486,9 +534,8 @@ __device__ __forceinline__ void plan_request(const RolloutArgs& a, const int r, 
     int* valid_s = reinterpret_cast<int*>(smem + L.aux);
     float* Dl_s = reinterpret_cast<float*>(valid_s + kMaxActions);
     float* Vd_s = Dl_s + kMaxActions;
-    float* gh_s = Vd_s + kMaxActions;  // goal term at the successor over 2^n0
     // keys of a step for the deferred near-tie flag, [2][32] by step parity
-    uint32_t* qkey_s = reinterpret_cast<uint32_t*>(gh_s + kMaxActions);
+    uint32_t* qkey_s = reinterpret_cast<uint32_t*>(Vd_s + kMaxActions);
     int* cls_s = reinterpret_cast<int*>(qkey_s + 2 * kMaxActions);
     float* la_s = reinterpret_cast<float*>(cls_s + 2 * kMaxActions);
     float* lt_s = la_s + 2 * kMaxActions;
@@ -499,8 +546,6 @@ __device__ __forceinline__ void plan_request(const RolloutArgs& a, const int r, 
     const int64_t t_lo = tbase, t_hi = tbase + a.tab.T_win;  // the table window this plan reads
     const int64_t last_j = (int64_t)req.horizon + 1;
     const int KEY_NONE = float_key(-INFINITY);
-    // FCFS ordinal of this request: tentative plans of later requests are not part of its table
-    const int32_t my_ord = a.pipe.on ? a.pipe.ord0 + r : INT_MAX;
 
     // ---------------------------------------------------------------- prologue
     if (tid < kHeadings) {
@@ -576,26 +621,6 @@ __device__ __forceinline__ void plan_request(const RolloutArgs& a, const int r, 
         st->n_points = 1;
         st->near_ties = 0;
         st->steps = 0;
-        if (k0 > 0) {
-            // resume at step k0: the state as the step that reached it published it, and the
-            // goal vector formed from its double-float copy exactly as a step forms it
-            const size_t o = (size_t)r * a.cap + k0;
-            for (int q = 0; q < 3; ++q) {
-                st->s[q] = a.pipe.st_s[3 * o + q];
-                st->s_hi[q] = a.pipe.st_df[6 * o + 2 * q];
-                st->s_lo[q] = a.pipe.st_df[6 * o + 2 * q + 1];
-                float gh = (float)g0[q];
-                float gl = (float)__dsub_rn(g0[q], (double)gh);
-                df_add(gh, gl, -st->s_hi[q], -st->s_lo[q]);
-                st->G_hi[q] = gh;
-                st->G_lo[q] = gl;
-            }
-            st->h = a.pipe.st_h[o];
-            st->done = 0;  // the run that planned these steps went on from step k0
-            st->status = FMDP_REJ_HORIZON;
-            st->n_points = k0 + 1;
-            st->steps = k0;
-        }
         st->abort_flag[0] = st->abort_flag[1] = 0;
         st->last_best[0] = st->last_best[1] = 99;
         for (int e = 0; e < kRingDepth; ++e) st->ent_valid[e] = 0;
@@ -608,12 +633,6 @@ __device__ __forceinline__ void plan_request(const RolloutArgs& a, const int r, 
         }
     }
     if (cs > 1) cluster_barrier(); else __syncthreads();  // mbarriers initialised cluster-wide
-    if (k0 > 0) {  // near ties of the kept steps
-        int nt = 0;
-        for (int i = tid; i < k0; i += NT) nt += a.pipe.ties[(size_t)r * a.cap + i];
-        if (nt) atomicAdd(&st->near_ties, nt);
-    }
-
     // ---- producer state (thread 32: warp 1, lane 0)
     const bool producer = (tid == 32);
     int64_t issued = 0, waited = 0;
@@ -654,151 +673,8 @@ __device__ __forceinline__ void plan_request(const RolloutArgs& a, const int r, 
         }
         return 0;
     };
-    // ---- indexed mode: the producer warp (warp 2) keeps a software pipeline over the spatial
-    // index. At step k (state s_k known) it reads the cell starts of the query for step k + 2
-    // (one cell row per lane; prefetched into L2 one step earlier), copies those items into a
-    // staging buffer, and waits for the items of step k + 1, copied one step earlier. It runs
-    // beside the step rather than in it: the other warps' reduction barrier leaves it out,
-    // and it joins them at the start of the next step. The query for step j, made from state s_a (a <= j - 1), covers every
-    // cell within Rq + (j - 1 - a) * step of s_a horizontally: an item whose wells can reach a
-    // successor of s_j lies within reach0 + tau_max * vmax of s_j (items outside the extra
-    // list move no faster than vmax), and s_j lies within (j - a) steps of s_a.
-    IdxMeta* imeta_all = imeta;
-    // pipeline state, identical in every lane of warp 2 (lane 0 waits, the warp follows)
-    uint32_t ifill[kIBufs] = {0u, 0u, 0u};
-    bool ipend[kIBufs] = {false, false, false};
-    const IndexView& iv = a.iv;
-    const int64_t cst_row_len = (int64_t)iv.ncell + 1;
-    auto row_of = [&](int64_t T) {
-        int64_t row = T % a.tab.T_win;
-        return row < 0 ? row + a.tab.T_win : row;
-    };
-    auto cell_of = [&](float v, float o, int n) {
-        const float f = floorf((v - o) * iv.inv_cell);
-        return f < 0.f ? 0 : (f > (float)(n - 1) ? n - 1 : (int)f);
-    };
-    auto excl_scan = [&](int v, int& total) {  // warp exclusive prefix sum
-        int x = v;
-        for (int o = 1; o < 32; o <<= 1) {
-            const int y = __shfl_up_sync(kFull, x, o);
-            if (lane >= o) x += y;
-        }
-        total = __shfl_sync(kFull, x, 31);
-        return x - v;
-    };
-    // bounded wait (lane 0) on a buffer's mbarrier; returns 1 on timeout, in every lane
-    auto wait_bar = [&](uint64_t* bar, uint32_t& fills, bool& pend) -> int {
-        if (!pend) return 0;
-        int bad = 0;
-        if (lane == 0) {
-            bad = mbar_wait_bounded(bar, fills & 1u) ? 0 : 1;
-            if (bad) atomicExch(a.err, FMDP_ERR_TIMEOUT);
-        }
-        bad = __shfl_sync(kFull, bad, 0);
-        ++fills;
-        pend = false;
-        return bad;
-    };
-    // lanes 0 .. kMaxRanges-1 each carry one item range (cnt 0: none): record them in
-    // buffer b's metadata and copy the first icap items into shared memory
-    auto issue_items = [&](int b, int my_beg, int my_cnt, long long row_off, int pub) {
-        IdxMeta& M = imeta_all[b];
-        int total;
-        const int off = excl_scan(lane < kMaxRanges ? my_cnt : 0, total);
-        const int n_s = min(total, icap);
-        if (lane < kMaxRanges) {
-            M.beg[lane] = my_beg;
-            M.cnt[lane] = my_cnt;
-        }
-        if (lane == 0) {
-            M.total = total;
-            M.n_s = n_s;
-            M.nr = kMaxRanges;
-            M.row_off = row_off;
-            M.pub = pub;
-            if (a.items_ctr && total > 0) atomicAdd(a.items_ctr, (unsigned long long)total);
-            if (n_s > 0) mbar_arrive_expect_tx(&bars[b], (uint32_t)n_s * 32u);
-            else mbar_arrive(&bars[b]);
-        }
-        __syncwarp();
-        const int take = lane < kMaxRanges ? max(0, min(my_cnt, n_s - off)) : 0;
-        if (take > 0)
-            tma_bulk_load(ibuf + ((size_t)b * icap + off) * 2, iv.items + row_off + (long long)my_beg * 2,
-                          (uint32_t)take * 32u, &bars[b]);
-        ipend[b] = true;
-    };
-    // cell box of a query; lanes 0 .. nrows-1 take one cell row each (whole: one range over
-    // full cell rows, its two ends in lanes 0 and 1); the extra list is range kMaxRanges-1
-    struct Box { int cx0, cx1, cy0, cy1, nrows, whole; };
-    auto box_of = [&](float sx, float sy, float R) {
-        Box q;
-        q.cx0 = cell_of(sx - R, iv.x0, iv.ncx);
-        q.cx1 = cell_of(sx + R, iv.x0, iv.ncx);
-        q.cy0 = cell_of(sy - R, iv.y0, iv.ncy);
-        q.cy1 = cell_of(sy + R, iv.y0, iv.ncy);
-        q.nrows = q.cy1 - q.cy0 + 1;
-        q.whole = q.nrows > kMaxRanges - 1;
-        return q;
-    };
-    // read the cell starts of step T's query (ring row `row` = T mod T_win) and issue it
-    auto issue_direct = [&](int b, int64_t T, int64_t row, float sx, float sy, float R) {
-        int my_beg = 0, my_cnt = 0;
-        long long row_off = 0;
-        int pub = INT_MAX;  // pipelined mode: published admissions this query can see (all: none in the row)
-        if (T >= t_lo && T < t_hi) {
-            const int32_t* cs_row = iv.cstart + row * cst_row_len;
-            const Box q = box_of(sx, sy, R);
-            int e0 = 0, e1 = 0;
-            // L2 loads (.cg): the index may change between launches of a persistent kernel
-            // (rows rebuilt, extra lists published), so nothing of it is kept in L1
-            if (!q.whole && lane < q.nrows) {
-                e0 = __ldcg(cs_row + (q.cy0 + lane) * iv.ncx + q.cx0);
-                e1 = __ldcg(cs_row + (q.cy0 + lane) * iv.ncx + q.cx1 + 1);
-            } else if (q.whole && lane == 0) {
-                e0 = __ldcg(cs_row + q.cy0 * iv.ncx);
-                e1 = __ldcg(cs_row + (q.cy1 + 1) * iv.ncx);
-            } else if (lane == kMaxRanges - 1) {
-                // the count of published admissions first (acquire), then the extra list's
-                // length: every admission counted is in the list this query copies
-                if (a.pipe.pub_seq) pub = ld_acquire_gpu(a.pipe.pub_seq);
-                e0 = __ldcg(cs_row + iv.ncell);
-                e1 = e0 + __ldcg(iv.nextra + row);
-            }
-            my_beg = e0;
-            my_cnt = max(0, e1 - e0);
-            row_off = (long long)row * a.tab.S_pad * 2;
-        }
-        pub = __shfl_sync(kFull, pub, kMaxRanges - 1);
-        issue_items(b, my_beg, my_cnt, row_off, pub);
-    };
-    // L2 prefetch of the cell starts a query of step T would read (issued one step early, so
-    // that the next step's issue finds them in L2 instead of waiting on DRAM)
-    auto prefetch_cells = [&](int64_t T, int64_t row, float sx, float sy, float R) {
-        if (T < t_lo || T >= t_hi) return;
-        const int32_t* cs_row = iv.cstart + row * cst_row_len;
-        const Box q = box_of(sx, sy, R);
-        const int32_t* p0 = nullptr;
-        const int32_t* p1 = nullptr;
-        if (!q.whole && lane < q.nrows) {
-            p0 = cs_row + (q.cy0 + lane) * iv.ncx + q.cx0;
-            p1 = cs_row + (q.cy0 + lane) * iv.ncx + q.cx1 + 1;
-        } else if (q.whole && lane == 0) {
-            p0 = cs_row + q.cy0 * iv.ncx;
-            p1 = cs_row + (q.cy1 + 1) * iv.ncx;
-        } else if (lane == kMaxRanges - 1) {
-            p0 = cs_row + iv.ncell;
-            p1 = iv.nextra + row;
-        }
-        if (p0) asm volatile("prefetch.global.L2 [%0];" ::"l"(p0));
-        if (p1) asm volatile("prefetch.global.L2 [%0];" ::"l"(p1));
-    };
-    // all outstanding copies, before the buffers are reused or the CTA leaves
-    auto drain = [&]() {
-        for (int b = 0; b < kIBufs; ++b) wait_bar(&bars[b], ifill[b], ipend[b]);
-    };
-
     bool stalled = false;
-    if (producer && !indexed && !st->done) {
+    if (producer && !st->done) {
         const int64_t T1 = req.depart_step + 1;
         int64_t row = T1 % a.tab.T_win;
         if (row < 0) row += a.tab.T_win;
@@ -818,21 +694,6 @@ __device__ __forceinline__ void plan_request(const RolloutArgs& a, const int r, 
     const double cap2 = st->cap2;
     const float reach0 = m.reach_base + stepf + dzmax;
     const float inv_dt = (float)(1.0 / m.dt);
-    const float Rq = reach0 + m.tau_absmax * a.iv.vmax * 1.0001f + stepf + 2.0f;  // indexed query radius
-    if (indexed && warp == 2 && !st->done) {
-        // steps k0 and k0 + 1 from the state at step k0 (the origin when k0 = 0)
-        const float ox = k0 > 0 ? st->s_hi[0] + st->s_lo[0] : (float)req.ox;
-        const float oy = k0 > 0 ? st->s_hi[1] + st->s_lo[1] : (float)req.oy;
-        const int b0 = k0 % kIBufs, b1 = (k0 + 1) % kIBufs;
-        issue_direct(b0, req.depart_step + k0 + 1, row_of(req.depart_step + k0 + 1), ox, oy, Rq);
-        issue_direct(b1, req.depart_step + k0 + 2, row_of(req.depart_step + k0 + 2), ox, oy, Rq);
-        const int to = wait_bar(&bars[b0], ifill[b0], ipend[b0]);
-        if (lane == 0) st->abort_flag[k0 & 1] = to;
-        stalled = to != 0;
-    }
-    // ring row of the query the producer issues at step k (for step k + 2): advanced by one
-    // row per step, so the loop needs no 64-bit modulo
-    int64_t prow = indexed ? row_of(req.depart_step + k0 + 3) : 0;
     float ghi[3], glo[3];  // goal as double-float
     {
         const double g0[3] = {req.gx, req.gy, req.gz};
@@ -869,13 +730,10 @@ __device__ __forceinline__ void plan_request(const RolloutArgs& a, const int r, 
 
     const bool timing = GEN && a.phase != nullptr && lead;
     unsigned long long ph[6] = {0, 0, 0, 0, 0, 0};
-    // indexed scanners' work (statistics): items culled, items inside the cull radius,
-    // (item, reachable well) pairs evaluated for every action
-    unsigned qe_items = 0u, qe_dnear = 0u, qe_wells = 0u;
     long long tp = 0;
 
     // ---------------------------------------------------------------- step loop
-    int k = k0;
+    int k = 0;
     for (;; ++k) {
         if (timing && tid == 0) tp = clock64();
         __syncthreads();  // S1: state and ring entries published
@@ -927,73 +785,41 @@ __device__ __forceinline__ void plan_request(const RolloutArgs& a, const int r, 
             }
             if (timing && tid == 0) { const long long t = clock64(); ph[1] += t - tp; tp = t; }
         } else if (warp == 1) {
-            // evaluator warp: the per-action terms that do not involve other plans, and the
-            // goal term over 2^n0 for the combine (its near-tie flag of the previous step
-            // comes after the reduction barrier)
+            // evaluator warp: the per-action terms that do not involve other plans (its near-tie
+            // flag of the previous step comes after the reduction barrier)
             if (lane < A) {
                 // successor estimate (fp32); terrain loads first, they are the longest wait
                 const float sx = shx + (slx + dxa), sy = shy + (sly + dya), sz = shz + (slz + dza);
-                float h00 = 0.f, h10 = 0.f, h01 = 0.f, h11 = 0.f, ax = 0.f, ay = 0.f;
+                TerrainCell tc;
                 if (hm) {
-                    const float gxf = (sx - box0) * hm_sx;
-                    const float gyf = (sy - box1) * hm_sy;
-                    int ix = (int)floorf(gxf), iy = (int)floorf(gyf);
-                    ix = min(max(ix, 0), hm_nx - 2);
-                    iy = min(max(iy, 0), hm_ny - 2);
-                    ax = gxf - (float)ix;
-                    ay = gyf - (float)iy;
-                    const float* r0 = hm + (size_t)iy * hm_nx + ix;
-                    h00 = __ldg(r0);
-                    h10 = __ldg(r0 + 1);
-                    h01 = __ldg(r0 + hm_nx);
-                    h11 = __ldg(r0 + hm_nx + 1);
+                    tc = terrain_cell(sx, sy, box0, box1, hm_sx, hm_sy, hm_nx, hm_ny);
+                    terrain_nodes(tc, hm, hm_nx);
                 }
                 // box validity: fp32 margin, exact comparison near a face
-                const float mlo = fminf(fminf(sx - box0, sy - box1), sz - box2);
-                const float mhi = fminf(fminf(box3 - sx, box4 - sy), box5 - sz);
-                const float mb = fminf(mlo, mhi);
+                const float mb = box_margin(sx, sy, sz, box0, box1, box2, box3, box4, box5);
                 bool valid;
                 if (mb > kBoxBand) valid = true;
                 else if (mb < -kBoxBand) valid = false;
-                else valid = box_inside_exact(m, st, Dx[hn], Dy[hn], my_Dz);
+                else valid = box_inside_exact(m, st->s, Dx[hn], Dy[hn], my_Dz);
                 // goal distance change Delta = |G - delta| - |G| at the current state
                 const float Gx = st->G_hi[0] + st->G_lo[0], Gy = st->G_hi[1] + st->G_lo[1],
                             Gz = st->G_hi[2] + st->G_lo[2];
-                const float Gn = approx_sqrt(Gx * Gx + Gy * Gy + Gz * Gz);
-                const float fx = Gx - dxa, fy = Gy - dya, fz = Gz - dza;
-                const float da = approx_sqrt(fx * fx + fy * fy + fz * fz);
-                const float num = (dxa * dxa + dya * dya + dza * dza) - 2.0f * (Gx * dxa + Gy * dya + Gz * dza);
-                const float den = da + Gn;
-                const float Dl = den > 0.f ? __fdividef(num, den) : 0.f;
+                const float Dl = goal_change(Gx, Gy, Gz, dxa, dya, dza);
                 // hard deck: terrain clearance at the successor (Alg. 1)
                 float Vd = 0.f;
                 if (hm) {
-                    const float hz = (1.f - ay) * ((1.f - ax) * h00 + ax * h10) + ay * ((1.f - ax) * h01 + ax * h11);
-                    const float c = sz - hz;
-                    if (fabsf(c - clr) < kClrBand) Vd = deck_exact(m, st, Dx[hn], Dy[hn], my_Dz);
+                    const float c = sz - terrain_height(tc);
+                    if (fabsf(c - clr) < kClrBand) Vd = deck_exact(m, st->s, Dx[hn], Dy[hn], my_Dz);
                     else if (c < clr) Vd = deckf - c;
                 }
                 valid_s[lane] = valid ? 1 : 0;
                 Dl_s[lane] = Dl;
                 Vd_s[lane] = Vd;
-                gh_s[lane] = has_goal ? exp2f(st->phi + Dl * lg32) : 0.f;  // g / 2^n0
                 // static negative peaks (restricted volumes / terrain wells), CTA 0 only
                 if (GEN && lead && n_static > 0)
                     fold_statics(m, st, sch, scl, shx, shy, shz, slx, sly, slz, dxa, dya, dza, Dx[hn], Dy[hn], my_Dz,
                                  mloc, sloc);
             }
-        } else if (indexed && warp == 2) {
-            // ---- indexed mode: the pipeline (items for k + 2, wait for k + 1)
-            int to = 1;
-            if (!stalled) {
-                issue_direct((k + 2) % kIBufs, req.depart_step + k + 3, prow, shx + slx, shy + sly, Rq + stepf);
-                prow = prow + 1 == a.tab.T_win ? 0 : prow + 1;  // ring row of the next step's query
-                prefetch_cells(req.depart_step + k + 4, prow, shx + slx, shy + sly, Rq + 2.f * stepf);
-                const int b1 = (k + 1) % kIBufs;
-                to = wait_bar(&bars[b1], ifill[b1], ipend[b1]);
-                if (to) stalled = true;
-            }
-            if (lane == 0) st->abort_flag[par ^ 1] = to;
         } else {
             // ---- scanners: cull, then wells of near slots with lanes as actions
             const long long ts = (timing && tid == NT - 32) ? clock64() : 0;
@@ -1031,7 +857,7 @@ __device__ __forceinline__ void plan_request(const RolloutArgs& a, const int r, 
                     const bool has2 = p2x == p2x;
                     for (; band; band &= band - 1u) {
                         const int w = __ffs(band) - 1;
-                        if (well_inside_exact(m, st, Dx[hn], Dy[hn], my_Dz, p1x, p1y, p1z, has2 ? p2x : 0.f,
+                        if (well_inside_exact(m, st->s, Dx[hn], Dy[hn], my_Dz, p1x, p1y, p1z, has2 ? p2x : 0.f,
                                               has2 ? p2y : 0.f, has2 ? p2z : 0.f, has2, w)) {
                             const float tau = st->w_tau[w];
                             const float ex = dxa - fmaf(tau, bvx, bqx), ey = dya - fmaf(tau, bvy, bqy),
@@ -1046,86 +872,6 @@ __device__ __forceinline__ void plan_request(const RolloutArgs& a, const int r, 
                 mloc = fmaxf(mloc, mb);
                 sloc += sb;
             };
-            if (indexed) {
-                // items staged for this step (buffer par), the overflow read from the index
-                const int b = k % kIBufs;
-                const IdxMeta& M = imeta[b];
-                const int total = M.total, n_s = M.n_s;
-                const float4* sb4 = ibuf + (size_t)b * icap * 2;
-                int itag = 0;  // tag of the item item_at read last
-                auto item_at = [&](int i, float& p1x, float& p1y, float& p1z, float& p2x, float& p2y, float& p2z) {
-                    float4 P1, P2;
-                    if (i < n_s) {
-                        P1 = sb4[2 * i];
-                        P2 = sb4[2 * i + 1];
-                    } else {
-                        int q = 0, off = i;
-                        while (q < M.nr - 1 && off >= M.cnt[q]) { off -= M.cnt[q]; ++q; }
-                        const float4* g = a.iv.items + M.row_off + 2ll * (M.beg[q] + off);
-                        P1 = __ldcg(g);
-                        P2 = __ldcg(g + 1);
-                    }
-                    p1x = P1.x; p1y = P1.y; p1z = P1.z;
-                    p2x = P2.x; p2y = P2.y; p2z = P2.z;
-                    itag = __float_as_int(P1.w);
-                };
-                // items interleaved over the scanner warps (item i to warp i mod nscan): the
-                // items within reach, each costing a well evaluation per action, sit next to
-                // one another in the index (same cells), so this spreads them over the warps
-                const int nscan = NW - 3, sw = warp - 3;
-                const int wn = total > sw ? (total - sw + nscan - 1) / nscan : 0;  // items of this warp
-                // one item per lane per pass: a warp rarely holds more than 32 items of a step,
-                // and a second unrolled copy of the fold only lengthens the step's code
-                constexpr int U = 1;
-                for (int base = 0; base < wn; base += 32 * U) {
-                    float qx[U], qy[U], qz[U], vx[U], vy[U], vz[U];
-                    bool near[U];
-                    unsigned wm[U];
-#pragma unroll
-                    for (int u = 0; u < U; ++u) {
-                        const int j = base + u * 32 + lane;
-                        const int i = sw + j * nscan;
-                        near[u] = false;
-                        qx[u] = qy[u] = qz[u] = vx[u] = vy[u] = vz[u] = 0.f;
-                        if (j < wn) {
-                            float p1x, p1y, p1z, p2x, p2y, p2z;
-                            item_at(i, p1x, p1y, p1z, p2x, p2y, p2z);
-                            // not in this request's table (a later request's tentative plan,
-                            // or a withdrawn one): culled like a plan far away
-                            if (!tag_visible(itag, my_ord)) p1x = p2x = __int_as_float(0x7fc00000);
-                            qx[u] = (p1x - shx) - slx;
-                            qy[u] = (p1y - shy) - sly;
-                            qz[u] = (p1z - shz) - slz;
-                            if (p2x == p2x) {
-                                vx[u] = (p2x - p1x) * inv_dt;
-                                vy[u] = (p2y - p1y) * inv_dt;
-                                vz[u] = (p2z - p1z) * inv_dt;
-                            }
-                            const float reach =
-                                fmaf(tau_absmax, approx_sqrt(vx[u] * vx[u] + vy[u] * vy[u] + vz[u] * vz[u]), reach0);
-                            near[u] = (qx[u] * qx[u] + qy[u] * qy[u] + qz[u] * qz[u]) < reach * reach;
-                            ++qe_items;
-                        }
-                        qe_dnear += near[u] ? 1u : 0u;
-                        wm[u] = near[u] ? well_mask(qx[u], qy[u], qz[u], vx[u], vy[u], vz[u]) : 0u;
-                        near[u] = wm[u] != 0u;
-                        qe_wells += __popc(wm[u]);
-                    }
-#pragma unroll
-                    for (int u = 0; u < U; ++u) {
-                        unsigned mask = __ballot_sync(kFull, near[u]);
-                        while (mask) {
-                            const int b = __ffs(mask) - 1;
-                            mask &= mask - 1;
-                            const int ii = sw + (base + u * 32 + b) * nscan;
-                            fold_near(item_at, ii, __shfl_sync(kFull, qx[u], b), __shfl_sync(kFull, qy[u], b),
-                                      __shfl_sync(kFull, qz[u], b), __shfl_sync(kFull, vx[u], b),
-                                      __shfl_sync(kFull, vy[u], b), __shfl_sync(kFull, vz[u], b),
-                                      __shfl_sync(kFull, wm[u], b));
-                        }
-                    }
-                }
-            } else {
             const int e1 = entry_of(k + 1), e2 = entry_of(k + 2);
             const bool v1 = st->ent_valid[e1] != 0;
             const bool v2 = (k + 2 <= last_j) && st->ent_valid[e2] != 0;
@@ -1188,7 +934,6 @@ __device__ __forceinline__ void plan_request(const RolloutArgs& a, const int r, 
                     }
                 }
             }
-            }
             if (ts) ph[4] += clock64() - ts;
         }
         if (lane < A) {
@@ -1197,13 +942,7 @@ __device__ __forceinline__ void plan_request(const RolloutArgs& a, const int r, 
         }
         __syncwarp();
         if (timing && tid == 0) tp = clock64();
-        // S3: per-action partials of this CTA complete (indexed mode: the producer warp, which
-        // adds no partials, goes on to the next step's start instead)
-        if (indexed) {
-            if (warp != 2) named_barrier(1, NT - 32);
-        } else {
-            __syncthreads();
-        }
+        __syncthreads();  // S3: per-action partials of this CTA complete
         if (timing && tid == 0) { const long long t = clock64(); ph[2] += t - tp; tp = t; }
 
         if (warp == 0) {
@@ -1257,37 +996,11 @@ __device__ __forceinline__ void plan_request(const RolloutArgs& a, const int r, 
             float Lp;
             if (combine) Lp = ssum ? __log2f((float)ssum) + (sum_ref - (float)kSumBits) : -INFINITY;
             else Lp = key_float(key);
-            const float lgh = phi + Dl * lg32;  // log2(g) - n0
-            // penalty + deck N, linear; the goal term g / 2^n0 comes from the evaluator
-            const bool pen = (combine ? ssum != 0ull : Lp > -INFINITY) || Vd > 0.f;
-            float Nl = 0.f;
-            if (pen) Nl = (combine ? (float)ssum * sum_unit : (Lp > -INFINITY ? exp2f(Lp) : 0.f)) + Vd;
-            int cls;   // 2: Q > 0, 1: Q = 0, 0: Q < 0
-            float k2;  // larger is better within a class
-            float la;  // log2 |Q|
-            if (!pen) {
-                cls = has_goal ? 2 : 1;
-                k2 = has_goal ? lgh : 0.f;
-                la = has_goal ? lgh + (float)n0 : -INFINITY;
-            } else {
-                const float gh = gh_s[lane];
-                const float Nh = Nl * sc0;  // N / 2^n0 (inf when that overflows fp32)
-                const float d = gh - Nh;
-                if (has_goal && d > 0.f) {
-                    cls = 2;
-                    k2 = __log2f(d);
-                    la = k2 + (float)n0;
-                } else if (d == 0.f) {
-                    cls = 1;
-                    k2 = 0.f;
-                    la = -INFINITY;
-                } else {
-                    cls = 0;
-                    la = Nh < INFINITY ? __log2f(-d) + (float)n0 : __log2f(Nl);  // log2 (N - g)
-                    k2 = -la;
-                }
-            }
-            const uint32_t qkey = (lane < A && valid) ? action_key(cls, k2) : 0u;
+            ActionValue v;
+            float Nl;
+            action_value(combine, has_goal, ssum, Lp, Vd, sum_unit, phi, Dl, lg32, n0, sc0, v, Nl);
+            const float lgh = fmaf(Dl, lg32, phi);  // log2(g) - n0
+            const uint32_t qkey = (lane < A && valid) ? action_key(v.cls, v.k2) : 0u;
             const uint32_t kmax = __reduce_max_sync(kFull, qkey);
             const unsigned bm = __ballot_sync(kFull, qkey == kmax && kmax != 0u);
             const int best = bm ? __ffs(bm) - 1 : 99;
@@ -1316,15 +1029,6 @@ __device__ __forceinline__ void plan_request(const RolloutArgs& a, const int r, 
                     traj[3 * np + 1] = tfy;
                     traj[3 * np + 2] = tfz;
                     acts[k] = (uint8_t)best;
-                    if (a.pipe.obs) {  // what a resumed plan and the host's influence test need
-                        const size_t o = (size_t)r * a.cap;
-                        a.pipe.obs[o + k] = imeta[k % kIBufs].pub;
-                        double* ps = a.pipe.st_s + 3 * (o + np);
-                        ps[0] = X; ps[1] = Y; ps[2] = Z;
-                        float* pd = a.pipe.st_df + 6 * (o + np);
-                        pd[0] = nhx; pd[1] = nlx; pd[2] = nhy; pd[3] = nly; pd[4] = nhz; pd[5] = nlz;
-                        a.pipe.st_h[o + np] = (uint8_t)hn;
-                    }
                     if (GEN && a.trace && r == 0) {
                         a.st_trace[3 * np] = X;
                         a.st_trace[3 * np + 1] = Y;
@@ -1334,10 +1038,10 @@ __device__ __forceinline__ void plan_request(const RolloutArgs& a, const int r, 
                 }
             }
             // keys of this step for the evaluator warp's deferred near-tie flag
-            const float logN = pen ? __log2f(Nl) : -INFINITY;
+            const float logN = Nl > 0.f ? __log2f(Nl) : -INFINITY;
             qkey_s[par * kMaxActions + lane] = qkey;
-            cls_s[par * kMaxActions + lane] = cls;
-            la_s[par * kMaxActions + lane] = la;
+            cls_s[par * kMaxActions + lane] = v.cls;
+            la_s[par * kMaxActions + lane] = v.la;
             lt_s[par * kMaxActions + lane] = fmaxf(has_goal ? lgh + (float)n0 : -INFINITY, logN);  // log2 max(g, N)
             if (lane == 0) st->last_best[par] = (ab || best >= 99) ? 99 : best;
             if (trace0 && lane < A)  // FP64 action values for the trace (not used for the decision)
@@ -1345,11 +1049,11 @@ __device__ __forceinline__ void plan_request(const RolloutArgs& a, const int r, 
             if (timing && tid == 0) ph[3] += clock64() - tp;
         } else {
             // evaluator warp: near-tie flag of the previous step, off the step's critical path
-            if (warp == 1 && k > k0)
+            if (warp == 1 && k > 0)
                 deferred_tie(st, qkey_s, cls_s, la_s, lt_s, par ^ 1, lane,
-                             trace0 ? a.tie_trace + (k - 1) : (a.pipe.ties ? a.pipe.ties + (size_t)r * a.cap + (k - 1) : nullptr));
+                             trace0 ? a.tie_trace + (k - 1) : nullptr);
         }
-        if (producer && !indexed) {
+        if (producer) {
             // ---- producer: slices needed two or more steps ahead
             const long long t0 = timing ? clock64() : 0;
             int to = 0;
@@ -1367,11 +1071,10 @@ __device__ __forceinline__ void plan_request(const RolloutArgs& a, const int r, 
     }
 
     // ---- epilogue: near-tie flag of the last step, drain the ring, outputs
-    if (warp == 1 && k > k0)
+    if (warp == 1 && k > 0)
         deferred_tie(st, qkey_s, cls_s, la_s, lt_s, (k - 1) & 1, lane,
-                     trace0 ? a.tie_trace + (k - 1) : (a.pipe.ties ? a.pipe.ties + (size_t)r * a.cap + (k - 1) : nullptr));
+                     trace0 ? a.tie_trace + (k - 1) : nullptr);
     __syncthreads();
-    if (indexed && warp == 2) drain();
     if (producer) {
         while (waited < issued) {
             const int64_t j = waited + 1;
@@ -1393,20 +1096,8 @@ __device__ __forceinline__ void plan_request(const RolloutArgs& a, const int r, 
     if (timing && (tid == 0 || tid == NT - 32 || producer))
         for (int i = 0; i < 6; ++i)
             if (ph[i]) atomicAdd(&a.phase[i], ph[i]);
-    if (a.qe_ctr && warp >= 3) {
-        for (int off = 16; off; off >>= 1) {
-            qe_items += __shfl_xor_sync(kFull, qe_items, off);
-            qe_dnear += __shfl_xor_sync(kFull, qe_dnear, off);
-            qe_wells += __shfl_xor_sync(kFull, qe_wells, off);
-        }
-        if (lane == 0 && qe_items) {
-            atomicAdd(&a.qe_ctr[0], (unsigned long long)qe_items);
-            atomicAdd(&a.qe_ctr[1], (unsigned long long)qe_dnear);
-            atomicAdd(&a.qe_ctr[2], (unsigned long long)qe_wells);
-        }
-    }
     if (cs > 1) cluster_barrier(); else __syncthreads();  // peers may still address this CTA's shared memory
-    if ((a.queue || a.pipe.on) && tid == 0) {  // the next request of this CTA initialises them again
+    if (a.queue && tid == 0) {  // the next request of this CTA initialises them again
         for (int e = 0; e < kRingDepth; ++e) mbar_inval(&bars[e]);
         mbar_inval(&xbar[0]);
         mbar_inval(&xbar[1]);
@@ -1568,18 +1259,65 @@ __device__ void pipe_finish(const RolloutArgs& a, int r, int token, int* red, lo
     __syncthreads();
 }
 
-// Persistent pipelined launch (indexed mode, one CTA per work item): plans the items the
-// host appends to the ring until it is told to stop, stays idle too long, or a wait expires.
+// One launch plans a set of requests. Full scan: without a work queue, cluster c plans request c;
+// with one (batch mode), each resident cluster pulls work items from a device counter until
+// none are left, which balances requests of uneven horizon: the lead CTA takes the item and its
+// peers read it from the lead's shared memory.
 template <bool GEN>
-__device__ void pipe_loop(const RolloutArgs& a, unsigned char* smem) {
-    const Layout L = make_layout(a.chunk, a.ring, a.icap);
-    int* slot = reinterpret_cast<int*>(smem + L.misc);  // [0] ring position, [1] request, [2] token, [3] start
-    long long* slot_tb = reinterpret_cast<long long*>(slot + 8);  // the item's window
+__device__ __forceinline__ void full_scan_loop(const RolloutArgs& a, unsigned char* smem) {
+    const int cs = a.cs;
+    int* next = reinterpret_cast<int*>(smem + make_layout(a.chunk, a.ring).misc);
+    const int n = a.n_dev ? *a.n_dev : a.n_req;
+    const bool lead = cs == 1 || cluster_rank() == 0;
+    for (;;) {
+        int w = blockIdx.x / cs;
+        if (a.queue) {
+            if (threadIdx.x == 0 && lead)  // after a device error, stop taking work
+                *next = *reinterpret_cast<volatile int32_t*>(a.err) != 0 ? n : atomicAdd(a.queue, 1);
+            if (cs > 1) {
+                cluster_barrier();
+                w = ld_cluster_s32(dsmem_addr(smem_u32(next), 0));
+                cluster_barrier();  // every CTA has read the item before the lead takes the next
+            } else {
+                __syncthreads();
+                w = *reinterpret_cast<volatile int*>(next);
+                __syncthreads();
+            }
+        }
+        if (w >= n) break;
+        const int r = a.idx ? a.idx[w] : w;
+        // uniform over the cluster: every CTA read the same item
+        if (!(a.skip && a.skip[r])) plan_request<GEN>(a, r, smem, a.tab.t_base);
+        if (!a.queue) break;
+    }
+}
+
+// Indexed form, one CTA per request: request blockIdx.x, the items of a device counter (batch
+// mode), or the items the host appends to the ring until it tells the launch to stop, it stays
+// idle too long, or a wait expires (pipelined mode). One loop, so that the plan's code is in the
+// kernel once.
+template <bool GEN>
+__device__ __forceinline__ void indexed_loop(const RolloutArgs& a, unsigned char* smem) {
+    // [0] work item or ring position, [1] request, [2] token, [3] start; [4..6] the tail check's
+    // first conflict and terrain sample and the operations published before it read the index;
+    // [8..9] the window
+    int* slot = reinterpret_cast<int*>(smem + idx_misc_offset(a.icap));
+    long long* slot_tb = reinterpret_cast<long long*>(slot + 8);
+    const bool pipe = a.pipe.on != 0;
+    const int n = a.n_dev ? *a.n_dev : a.n_req;
     for (;;) {
         if (threadIdx.x == 0) {
             int r = 0, tok = 0, k0 = 0;
-            long long tb = 0;
-            const int w = pipe_take(a, &r, &tok, &k0, &tb);
+            long long tb = a.tab.t_base;
+            int w;
+            if (pipe) {
+                w = pipe_take(a, &r, &tok, &k0, &tb);
+            } else {
+                w = !a.queue ? (int)blockIdx.x
+                             : (*reinterpret_cast<volatile int32_t*>(a.err) != 0 ? n : atomicAdd(a.queue, 1));
+                if (w >= n) w = -1;  // (after a device error, no more work is taken)
+                if (w >= 0) r = a.idx ? a.idx[w] : w;
+            }
             slot[0] = w;
             slot[1] = r;
             slot[2] = tok;
@@ -1594,57 +1332,25 @@ __device__ void pipe_loop(const RolloutArgs& a, unsigned char* smem) {
         const long long tb = *reinterpret_cast<volatile long long*>(slot_tb);
         __syncthreads();
         if (w < 0) break;
-        if (k0 >= 0) plan_request<true, GEN>(a, r, smem, tb, k0);  // k0 < 0: the plan stands, only its check again
-        pipe_finish(a, r, tok, slot + 4, tb);
+        // k0 < 0: the plan stands, only its check again
+        if (k0 >= 0 && !(a.skip && a.skip[r])) plan_indexed<GEN>(a, r, smem, tb, k0);
+        if (pipe) pipe_finish(a, r, tok, slot + 4, tb);
+        else if (!a.queue) break;
     }
 }
 
-// One launch plans a set of requests. Without a work queue, cluster c plans request c.
-// With a work queue (batch mode), each resident cluster pulls work items from a device
-// counter until none are left, which balances requests of uneven horizon: the lead CTA
-// takes the item and its peers read it from the lead's shared memory.
-// IDX: the indexed-mode instance (cluster size 1; the pipelined mode runs only there);
-// GEN: with the phase clock stamps.
+// IDX: the indexed form (cluster size 1); GEN: the general instance.
 template <bool IDX, bool GEN>
 __global__ void __launch_bounds__(384, 1) rollout_kernel(const __grid_constant__ RolloutArgs a) {
     extern __shared__ __align__(128) unsigned char smem[];
-    const int cs = IDX ? 1 : a.cs;
-    if constexpr (IDX) {
-        if (a.pipe.on) {
-            pipe_loop<GEN>(a, smem);
-            return;
-        }
-    }
-    if (a.queue == nullptr) {
-        const int r = blockIdx.x / cs;
-        if (r < a.n_req) plan_request<IDX, GEN>(a, r, smem, a.tab.t_base);  // uniform over the cluster
-        return;
-    }
-    const Layout L = make_layout(a.chunk, a.ring, IDX ? a.icap : 0);
-    int* next = reinterpret_cast<int*>(smem + L.misc);
-    const int n = a.n_dev ? *a.n_dev : a.n_req;
-    const bool lead = cs == 1 || cluster_rank() == 0;
-    for (;;) {
-        if (threadIdx.x == 0 && lead)  // after a device error, stop taking work
-            *next = *reinterpret_cast<volatile int32_t*>(a.err) != 0 ? n : atomicAdd(a.queue, 1);
-        int w;
-        if (cs > 1) {
-            cluster_barrier();
-            w = ld_cluster_s32(dsmem_addr(smem_u32(next), 0));
-            cluster_barrier();  // every CTA has read the item before the lead takes the next
-        } else {
-            __syncthreads();
-            w = *reinterpret_cast<volatile int*>(next);
-            __syncthreads();
-        }
-        if (w >= n) break;
-        const int r = a.idx ? a.idx[w] : w;
-        if (a.skip && a.skip[r]) continue;  // uniform over the cluster: every CTA read the same item
-        plan_request<IDX, GEN>(a, r, smem, a.tab.t_base);
-    }
+    if constexpr (IDX) indexed_loop<GEN>(a, smem);
+    else full_scan_loop<GEN>(a, smem);
 }
 
-size_t rollout_smem_bytes(int chunk, int depth, int icap) { return make_layout(chunk, depth, icap).total; }
+// chunk, depth: the full-scan form's slices; icap > 0: the indexed form
+size_t rollout_smem_bytes(int chunk, int depth, int icap) {
+    return icap > 0 ? idx_smem_bytes(icap) : make_layout(chunk, depth).total;
+}
 
 cudaError_t prepare_rollout_kernel(size_t smem) {
     const void* fs[4] = {(const void*)rollout_kernel<true, false>, (const void*)rollout_kernel<false, false>,
