@@ -105,6 +105,7 @@ fmdp_status fmdp_create(const fmdp_airspace* air, double gamma, const fmdp_actio
         CK(preload_table_kernels());
         CK(prepare_sepcheck_rows(sepcheck_rows_smem(kBatchMax)));
         CK(prepare_policy_kernel());
+        CK(prepare_train_kernels());
         CK(prepare_lookahead_kernel());
 
         c->T_win = a.n_slices_window;
@@ -593,17 +594,16 @@ fmdp_status fmdp_learned_loss_grad(fmdp_ctx* c, const float* X, const uint8_t* y
         require(X && y && loss && grad && rows >= 1 && rows <= 8192, FMDP_ERR_ARG, "null arrays or rows out of range");
         require(c->mlp_ready, FMDP_ERR_ARG, "the proposal network has no parameters");
         for (int32_t i = 0; i < rows; ++i) require(y[i] < c->A, FMDP_ERR_ARG, "label beyond the action set");
-        std::vector<__nv_bfloat16> h((size_t)rows * kFeat);
-        for (size_t i = 0; i < h.size(); ++i) h[i] = __float2bfloat16_rn(X[i]);
         c->trX.ensure((size_t)rows * kFeat);
+        c->trXf.ensure((size_t)rows * kFeat);
         c->tr_y.ensure(rows);
-        CK(cudaMemcpyAsync(c->trX.p, h.data(), h.size() * sizeof(__nv_bfloat16), cudaMemcpyHostToDevice, c->stream));
+        CK(cudaMemcpyAsync(c->trXf.p, X, (size_t)rows * kFeat * sizeof(float), cudaMemcpyHostToDevice, c->stream));
         CK(cudaMemcpyAsync(c->tr_y.p, y, rows, cudaMemcpyHostToDevice, c->stream));
         CK(cudaMemsetAsync(c->tr_loss.p, 0, sizeof(float), c->stream));
-        mlp_fwd_bwd(c, c->trX.p, c->tr_y.p, rows);
+        mlp_fwd_bwd(c, c->trXf.p, c->trX.p, c->tr_y.p, rows);
         CK(cudaMemcpyAsync(loss, c->tr_loss.p, sizeof(float), cudaMemcpyDeviceToHost, c->stream));
         CK(cudaMemcpyAsync(grad, c->mlp_g.p, n_params_total() * sizeof(float), cudaMemcpyDeviceToHost, c->stream));
-        CK(cudaStreamSynchronize(c->stream));
+        require(read_error_word(c) == 0, FMDP_ERR_TIMEOUT, "a bounded device wait expired in the gradient");
     });
 }
 

@@ -248,13 +248,13 @@ struct fmdp_ctx {
     // layout and the policy kernel's chunks); the training set; per-request proposal buffers
     bool mlp_ready = false;
     DevArray<float> mlp_p, mlp_g, mlp_m1, mlp_m2;
-    DevArray<__nv_bfloat16> mlp_wt, mlp_wp;
+    DevArray<__nv_bfloat16> mlp_wp;
     int64_t adam_t = 0;
     DevArray<__nv_bfloat16> tX;
     DevArray<uint8_t> ty;
     int64_t t_rows = 0;
     DevArray<__nv_bfloat16> trX, trH, trdZ;
-    DevArray<float> trZ, trdZf, trdH, tr_loss;
+    DevArray<float> trXf, tr_sums, tr_part, tr_loss;
     DevArray<int32_t> tr_idx;
     DevArray<uint8_t> tr_y;
     DevArray<float> p_traj;
@@ -460,10 +460,9 @@ void autotune(fmdp_ctx* c, const fmdp_request* sample, int32_t n, bool force, fm
 
 // ------------------------------------------------------------------ learned proposal (host_learned.cu)
 
-size_t wt_offset(int l);
 void mlp_ensure(fmdp_ctx* c);
 void mlp_upload(fmdp_ctx* c, const float* params);
-void mlp_fwd_bwd(fmdp_ctx* c, const __nv_bfloat16* X, const uint8_t* y, int B);
+void mlp_fwd_bwd(fmdp_ctx* c, const float* Xf, __nv_bfloat16* X, const uint8_t* y, int B);
 void mlp_train(fmdp_ctx* c, int32_t epochs, int32_t batch, float lr, uint64_t seed, float* losses);
 void learned_collect(fmdp_ctx* c, const fmdp_request* reqs, int32_t n);
 void learned_evaluate(fmdp_ctx* c, const fmdp_request* reqs, int32_t n, double slack, fmdp_learned_report* rep,

@@ -9,19 +9,12 @@ namespace fmdp {
 // ------------------------------------------------------------------ learned proposal
 
 
-size_t wt_offset(int l) {
-    size_t o = 0;
-    for (int i = 0; i < l; ++i) o += (size_t)layer_in(i) * layer_out_pad(i);
-    return o;
-}
-
 void mlp_ensure(fmdp_ctx* c) {
     const size_t P = n_params_total();
     c->mlp_p.ensure(P);
     c->mlp_g.ensure(P);
     c->mlp_m1.ensure(P);
     c->mlp_m2.ensure(P);
-    c->mlp_wt.ensure(wt_offset(kLayers));
     c->mlp_wp.ensure(wp_total());
     c->tr_loss.ensure(1);
 }
@@ -33,45 +26,35 @@ void mlp_upload(fmdp_ctx* c, const float* params) {
     CK(cudaMemsetAsync(c->mlp_m1.p, 0, P * sizeof(float), c->stream));
     CK(cudaMemsetAsync(c->mlp_m2.p, 0, P * sizeof(float), c->stream));
     c->adam_t = 0;
-    LAUNCH(c, launch_export_weights(c->mlp_p.p, c->mlp_wt.p, c->mlp_wp.p, c->stream));
+    LAUNCH(c, launch_export_weights(c->mlp_p.p, c->mlp_wp.p, c->stream));
     CK(cudaStreamSynchronize(c->stream));
     c->mlp_ready = true;
 }
 
-// forward and backward of one batch (X: B rows of bf16 features on the device, y labels):
-// the batch's mean loss is added to tr_loss[0], the gradient written to mlp_g
-void mlp_fwd_bwd(fmdp_ctx* c, const __nv_bfloat16* X, const uint8_t* y, int B) {
-    cudaStream_t s = c->stream;
+// loss and gradient of one batch (X: B rows of bf16 features on the device, or to be rounded
+// from the fp32 features Xf; y labels): the batch's mean loss is added to tr_loss[0], the
+// gradient written to mlp_g
+void mlp_fwd_bwd(fmdp_ctx* c, const float* Xf, __nv_bfloat16* X, const uint8_t* y, int B) {
     c->trH.ensure((size_t)4 * B * kHid);
-    c->trZ.ensure((size_t)B * kHid);
-    c->trdZ.ensure((size_t)B * kHid);
-    c->trdZf.ensure((size_t)B * kHid);
-    c->trdH.ensure((size_t)B * kHid);
-    auto H = [&](int l) -> const __nv_bfloat16* { return l == 0 ? X : c->trH.p + (size_t)(l - 1) * B * kHid; };
-    auto ldH = [&](int l) { return l == 0 ? kFeat : kHid; };
-    const __nv_bfloat16* Wt = c->mlp_wt.p;
-    const float* P = c->mlp_p.p;
-    float* G = c->mlp_g.p;
-    for (int l = 0; l < kLayers - 1; ++l) {
-        LAUNCH(c, launch_gemm_bf16(B, kHid, layer_in(l), H(l), ldH(l), 1, Wt + wt_offset(l), kHid, 1, c->trZ.p, kHid, 0, s));
-        LAUNCH(c, launch_bias_act(c->trZ.p, P + param_offset_b(l), c->trH.p + (size_t)l * B * kHid, B, kHid, kHid, kHid,
-                                  1, s));
-    }
-    const int L4 = kLayers - 1;
-    LAUNCH(c, launch_gemm_bf16(B, kOutPad, kHid, H(L4), kHid, 1, Wt + wt_offset(L4), kOutPad, 1, c->trZ.p, kOutPad, 0, s));
-    LAUNCH(c, launch_softmax_ce(c->trZ.p, kOutPad, P + param_offset_b(L4), y, B, c->A, c->trdZ.p, kOutPad, c->trdZf.p,
-                                c->tr_loss.p, s));
-    for (int l = kLayers - 1; l >= 0; --l) {
-        const int ld_dz = l == kLayers - 1 ? kOutPad : kHid, out = layer_out(l);
-        LAUNCH(c, launch_gemm_bf16(layer_in(l), out, B, H(l), 1, ldH(l), c->trdZ.p, ld_dz, 1, G + param_offset_W(l), out,
-                                   0, s));
-        LAUNCH(c, launch_colsum(c->trdZf.p, B, out, ld_dz, G + param_offset_b(l), s));
-        if (l > 0) {
-            LAUNCH(c, launch_gemm_bf16(B, layer_in(l), out, c->trdZ.p, ld_dz, 1, Wt + wt_offset(l), 1,
-                                       layer_out_pad(l), c->trdH.p, kHid, 0, s));
-            LAUNCH(c, launch_relu_bwd(c->trdH.p, H(l), B, kHid, c->trdZ.p, c->trdZf.p, s));
-        }
-    }
+    c->trdZ.ensure((size_t)B * (4 * kHid + kOutPad));
+    c->tr_sums.ensure((size_t)train_blocks(B) * kTrainSums);
+    c->tr_part.ensure((size_t)kTrainSplit * n_params_total());
+    TrainArgs a{};
+    a.Xf = Xf;
+    a.X = X;
+    a.y = y;
+    a.M = B;
+    a.n_valid = c->A;
+    a.Wp = c->mlp_wp.p;
+    a.params = c->mlp_p.p;
+    a.H = c->trH.p;
+    a.dZ = c->trdZ.p;
+    a.sums = c->tr_sums.p;
+    a.part = c->tr_part.p;
+    a.grad = c->mlp_g.p;
+    a.loss = c->tr_loss.p;
+    a.err = c->err;
+    LAUNCH(c, launch_train(a, c->stream));
 }
 
 void mlp_train(fmdp_ctx* c, int32_t epochs, int32_t batch, float lr, uint64_t seed, float* losses) {
@@ -93,10 +76,10 @@ void mlp_train(fmdp_ctx* c, int32_t epochs, int32_t batch, float lr, uint64_t se
         for (int64_t b0 = 0; b0 < rows; b0 += batch, ++nb) {
             const int Bn = (int)std::min<int64_t>(batch, rows - b0);
             LAUNCH(c, launch_gather_rows(c->tX.p, c->tr_idx.p + b0, Bn, c->trX.p, c->ty.p, c->tr_y.p, c->stream));
-            mlp_fwd_bwd(c, c->trX.p, c->tr_y.p, Bn);
+            mlp_fwd_bwd(c, nullptr, c->trX.p, c->tr_y.p, Bn);
             LAUNCH(c, launch_adam(c->mlp_p.p, c->mlp_g.p, c->mlp_m1.p, c->mlp_m2.p, n_params_total(), lr, 0.9f, 0.999f,
                                   1e-8f, (int)++c->adam_t, c->stream));
-            LAUNCH(c, launch_export_weights(c->mlp_p.p, c->mlp_wt.p, c->mlp_wp.p, c->stream));
+            LAUNCH(c, launch_export_weights(c->mlp_p.p, c->mlp_wp.p, c->stream));
         }
         float tot = 0.f;
         CK(cudaMemcpyAsync(&tot, c->tr_loss.p, sizeof(float), cudaMemcpyDeviceToHost, c->stream));

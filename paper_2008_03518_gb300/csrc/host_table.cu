@@ -643,9 +643,9 @@ void destroy_ctx(fmdp_ctx* c) {
         if (p) cudaFree(p);
     c->seq.release(); c->stg.release(); c->bat.release();
     c->chk_xyz.release(); c->chk_rep.release(); c->chk_acc.release();
-    c->mlp_p.release(); c->mlp_g.release(); c->mlp_m1.release(); c->mlp_m2.release(); c->mlp_wt.release();
+    c->mlp_p.release(); c->mlp_g.release(); c->mlp_m1.release(); c->mlp_m2.release();
     c->mlp_wp.release(); c->tX.release(); c->ty.release(); c->trX.release(); c->trH.release(); c->trdZ.release();
-    c->trZ.release(); c->trdZf.release(); c->trdH.release(); c->tr_loss.release(); c->tr_idx.release();
+    c->trXf.release(); c->tr_sums.release(); c->tr_part.release(); c->tr_loss.release(); c->tr_idx.release();
     c->tr_y.release(); c->p_traj.release(); c->p_acts.release(); c->p_rout.release(); c->p_sep.release();
     c->p_acc.release(); c->p_queue.release(); c->p_ident.release(); c->row0.release();
     for (auto& g : c->graphs)

@@ -1,5 +1,5 @@
 // Learned proposal kernels (sm_103a): training-set collection from FastMDP rollouts, the
-// bf16 tensor-core GEMM and element-wise steps of training, and policy rollouts that run
+// optimiser (loss and gradient: train.cu), and policy rollouts that run
 // many requests in lock step through the MLP (mma.sync m16n8k16, weights staged by bulk
 // copy). The network, its inputs and its loss are stated in plain FP64 in the oracle.
 #include <climits>
@@ -11,53 +11,6 @@ namespace fmdp {
 namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
-
-__device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ void mma_bf16(float* d, const uint32_t* a, const uint32_t* b) {
-    asm volatile(
-        "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
-        "{%0,%1,%2,%3};"
-        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
-}
-
-__device__ __forceinline__ uint32_t ld32(const __nv_bfloat16* p) { return *reinterpret_cast<const uint32_t*>(p); }
-
-__device__ __forceinline__ void bar_init(uint64_t* bar) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(bar)) : "memory");
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-}
-__device__ __forceinline__ void bar_expect(uint64_t* bar, uint32_t bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(bar)), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ bool bar_try(uint64_t* bar, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(smem_addr(bar)), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-// bounded wait (about a second of SM cycles); false on timeout
-__device__ __forceinline__ bool bar_wait(uint64_t* bar, uint32_t parity) {
-    const long long t0 = clock64();
-    while (!bar_try(bar, parity))
-        if (clock64() - t0 > (1ll << 31)) return false;
-    return true;
-}
-__device__ __forceinline__ void bar_inval(uint64_t* bar) {
-    asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(smem_addr(bar)) : "memory");
-}
-__device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
-    asm volatile(
-        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-            smem_addr(dst)),
-        "l"(src), "r"(bytes), "r"(smem_addr(bar))
-        : "memory");
-}
 
 }  // namespace
 
@@ -120,152 +73,7 @@ cudaError_t launch_collect(const CollectArgs& a, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-// ------------------------------------------------------------------ training kernels
-
-// 64 x 64 output tile per block, 4 warps of 32 x 32, K in steps of 32 through shared memory.
-__global__ void __launch_bounds__(128) gemm_bf16_kernel(int M, int N, int K, const __nv_bfloat16* A, long sai,
-                                                        long sak, const __nv_bfloat16* B, long sbk, long sbj,
-                                                        float* C, int ldc, int accumulate) {
-    __shared__ __align__(16) __nv_bfloat16 As[64][40];
-    __shared__ __align__(16) __nv_bfloat16 Bs[64][40];  // [n][k]
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int g = lane >> 2, t = lane & 3;
-    const int bm = blockIdx.y * 64, bn = blockIdx.x * 64;
-    const int wm = (warp >> 1) * 32, wn = (warp & 1) * 32;
-    float acc[2][4][4];
-#pragma unroll
-    for (int i = 0; i < 2; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-#pragma unroll
-            for (int q = 0; q < 4; ++q) acc[i][j][q] = 0.f;
-    const __nv_bfloat16 zero = __float2bfloat16_rn(0.f);
-    for (int k0 = 0; k0 < K; k0 += 32) {
-        for (int e = tid; e < 64 * 32; e += 128) {
-            const int i = e >> 5, k = e & 31, gi = bm + i, gk = k0 + k;
-            As[i][k] = (gi < M && gk < K) ? A[gi * sai + gk * sak] : zero;
-            const int gj = bn + i;
-            Bs[i][k] = (gj < N && gk < K) ? B[gk * sbk + gj * sbj] : zero;
-        }
-        __syncthreads();
-#pragma unroll
-        for (int kk = 0; kk < 32; kk += 16) {
-            uint32_t af[2][4], bf[4][2];
-#pragma unroll
-            for (int mt = 0; mt < 2; ++mt) {
-                const int r0 = wm + mt * 16 + g;
-                af[mt][0] = ld32(&As[r0][kk + 2 * t]);
-                af[mt][1] = ld32(&As[r0 + 8][kk + 2 * t]);
-                af[mt][2] = ld32(&As[r0][kk + 8 + 2 * t]);
-                af[mt][3] = ld32(&As[r0 + 8][kk + 8 + 2 * t]);
-            }
-#pragma unroll
-            for (int nt = 0; nt < 4; ++nt) {
-                const int c0 = wn + nt * 8 + g;
-                bf[nt][0] = ld32(&Bs[c0][kk + 2 * t]);
-                bf[nt][1] = ld32(&Bs[c0][kk + 8 + 2 * t]);
-            }
-#pragma unroll
-            for (int mt = 0; mt < 2; ++mt)
-#pragma unroll
-                for (int nt = 0; nt < 4; ++nt) mma_bf16(acc[mt][nt], af[mt], bf[nt]);
-        }
-        __syncthreads();
-    }
-#pragma unroll
-    for (int mt = 0; mt < 2; ++mt)
-#pragma unroll
-        for (int nt = 0; nt < 4; ++nt)
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const int r = bm + wm + mt * 16 + g + (q >= 2 ? 8 : 0);
-                const int c = bn + wn + nt * 8 + 2 * t + (q & 1);
-                if (r < M && c < N) {
-                    float v = acc[mt][nt][q];
-                    if (accumulate) v += C[(size_t)r * ldc + c];
-                    C[(size_t)r * ldc + c] = v;
-                }
-            }
-}
-
-cudaError_t launch_gemm_bf16(int M, int N, int K, const __nv_bfloat16* A, long sa_i, long sa_k,
-                             const __nv_bfloat16* B, long sb_k, long sb_j, float* C, int ldc, int accumulate,
-                             cudaStream_t s) {
-    if (M <= 0 || N <= 0 || K <= 0) return cudaSuccess;
-    gemm_bf16_kernel<<<dim3((N + 63) / 64, (M + 63) / 64), 128, 0, s>>>(M, N, K, A, sa_i, sa_k, B, sb_k, sb_j, C,
-                                                                        ldc, accumulate);
-    return cudaGetLastError();
-}
-
-__global__ void bias_act_kernel(const float* Z, const float* b, __nv_bfloat16* H, int M, int N, int ldz, int ldh,
-                                int relu) {
-    const size_t n = (size_t)M * N;
-    for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
-        const int i = (int)(e / N), j = (int)(e % N);
-        float v = Z[(size_t)i * ldz + j] + b[j];
-        if (relu) v = fmaxf(v, 0.f);
-        H[(size_t)i * ldh + j] = __float2bfloat16_rn(v);
-    }
-}
-cudaError_t launch_bias_act(const float* Z, const float* b, __nv_bfloat16* H, int M, int N, int ldz, int ldh, int relu,
-                            cudaStream_t s) {
-    bias_act_kernel<<<592, 256, 0, s>>>(Z, b, H, M, N, ldz, ldh, relu);
-    return cudaGetLastError();
-}
-
-// one warp per row (logits of at most 32 actions, lanes = actions)
-__global__ void softmax_ce_kernel(const float* Z, int ldz, const float* bias, const uint8_t* y, int M, int n_valid,
-                                  __nv_bfloat16* dZ, int lddz, float* dZf, float* loss) {
-    const int lane = threadIdx.x & 31;
-    const int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (row >= M) return;
-    const float z = lane < n_valid ? Z[(size_t)row * ldz + lane] + bias[lane] : -INFINITY;
-    float mx = z;
-    for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(kFull, mx, o));
-    const float e = lane < n_valid ? expf(z - mx) : 0.f;
-    float sum = e;
-    for (int o = 16; o; o >>= 1) sum += __shfl_xor_sync(kFull, sum, o);
-    const float p = e / sum;
-    const int lab = y[row];
-    const float gval = (p - (lane == lab ? 1.f : 0.f)) / (float)M;
-    if (lane < lddz) {
-        dZ[(size_t)row * lddz + lane] = __float2bfloat16_rn(lane < n_valid ? gval : 0.f);
-        dZf[(size_t)row * lddz + lane] = lane < n_valid ? gval : 0.f;
-    }
-    if (lane == lab) atomicAdd(loss, -(logf(p)) / (float)M);
-}
-cudaError_t launch_softmax_ce(const float* Z, int ldz, const float* bias, const uint8_t* y, int M, int n_valid,
-                              __nv_bfloat16* dZ, int lddz, float* dZf, float* loss, cudaStream_t s) {
-    softmax_ce_kernel<<<(M * 32 + 255) / 256, 256, 0, s>>>(Z, ldz, bias, y, M, n_valid, dZ, lddz, dZf, loss);
-    return cudaGetLastError();
-}
-
-__global__ void relu_bwd_kernel(const float* dH, const __nv_bfloat16* H, int M, int N, __nv_bfloat16* dZ, float* dZf) {
-    const size_t n = (size_t)M * N;
-    for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
-        const float v = __bfloat162float(H[e]) > 0.f ? dH[e] : 0.f;
-        dZ[e] = __float2bfloat16_rn(v);
-        dZf[e] = v;
-    }
-}
-cudaError_t launch_relu_bwd(const float* dH, const __nv_bfloat16* H, int M, int N, __nv_bfloat16* dZ, float* dZf,
-                            cudaStream_t s) {
-    relu_bwd_kernel<<<592, 256, 0, s>>>(dH, H, M, N, dZ, dZf);
-    return cudaGetLastError();
-}
-
-// column sums of G (M x N): one thread per column
-__global__ void colsum_kernel(const float* G, int M, int N, int ld, float* out) {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= N) return;
-    float s = 0.f;
-    for (int i = 0; i < M; ++i) s += G[(size_t)i * ld + j];
-    out[j] = s;
-}
-cudaError_t launch_colsum(const float* G, int M, int N, int ld, float* out, cudaStream_t s) {
-    colsum_kernel<<<(N + 127) / 128, 128, 0, s>>>(G, M, N, ld, out);
-    return cudaGetLastError();
-}
+// ------------------------------------------------------------------ training rows and weights
 
 __global__ void gather_rows_kernel(const __nv_bfloat16* X, const int32_t* idx, int M, __nv_bfloat16* out,
                                    const uint8_t* y, uint8_t* y_out) {
@@ -300,10 +108,8 @@ cudaError_t launch_adam(float* p, const float* g, float* m1, float* m2, size_t n
     return cudaGetLastError();
 }
 
-// bf16 copies of the weights: Wt[l] = W_l (in x out_pad, row-major, zero padded) for
-// training, and the policy's chunked layout
-__global__ void export_kernel(const float* p, __nv_bfloat16* Wt, __nv_bfloat16* Wp) {
-    size_t o_t = 0;
+// bf16 copy of the weights in the chunked layout that the policy and the training kernels stream
+__global__ void export_kernel(const float* p, __nv_bfloat16* Wp) {
     for (int l = 0; l < kLayers; ++l) {
         const int in = layer_in(l), out = layer_out(l), op = layer_out_pad(l);
         const float* W = p + param_offset_W(l);
@@ -312,7 +118,6 @@ __global__ void export_kernel(const float* p, __nv_bfloat16* Wt, __nv_bfloat16* 
         for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
             const int i = (int)(e / op), j = (int)(e % op);
             const __nv_bfloat16 v = __float2bfloat16_rn(j < out ? W[(size_t)i * out + j] : 0.f);
-            Wt[o_t + e] = v;
             const int ch = i / kChunkK, kl = i % kChunkK;
             wp[(size_t)ch * wp_chunk_elems(l) + (size_t)j * kChunkPad + kl] = v;
         }
@@ -322,11 +127,10 @@ __global__ void export_kernel(const float* p, __nv_bfloat16* Wt, __nv_bfloat16* 
             const size_t rowi = e / (kChunkPad - kChunkK), q = e % (kChunkPad - kChunkK);
             wp[rowi * kChunkPad + kChunkK + q] = __float2bfloat16_rn(0.f);
         }
-        o_t += n;
     }
 }
-cudaError_t launch_export_weights(const float* p, __nv_bfloat16* Wt, __nv_bfloat16* Wp, cudaStream_t s) {
-    export_kernel<<<296, 256, 0, s>>>(p, Wt, Wp);
+cudaError_t launch_export_weights(const float* p, __nv_bfloat16* Wp, cudaStream_t s) {
+    export_kernel<<<296, 256, 0, s>>>(p, Wp);
     return cudaGetLastError();
 }
 

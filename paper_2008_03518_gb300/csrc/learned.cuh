@@ -41,6 +41,54 @@ __host__ __device__ inline size_t wp_layer_offset(int l) {
 }
 __host__ __device__ inline size_t wp_total() { return wp_layer_offset(kLayers); }
 
+// ---- tensor-core and bulk-copy steps shared by the network kernels
+__device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+
+__device__ __forceinline__ void mma_bf16(float* d, const uint32_t* a, const uint32_t* b) {
+    asm volatile(
+        "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
+        "{%0,%1,%2,%3};"
+        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
+}
+
+__device__ __forceinline__ uint32_t ld32(const __nv_bfloat16* p) { return *reinterpret_cast<const uint32_t*>(p); }
+
+__device__ __forceinline__ void bar_init(uint64_t* bar) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(bar)) : "memory");
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+}
+__device__ __forceinline__ void bar_expect(uint64_t* bar, uint32_t bytes) {
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(bar)), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ bool bar_try(uint64_t* bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(smem_addr(bar)), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+// bounded wait (about a second of SM cycles); false on timeout
+__device__ __forceinline__ bool bar_wait(uint64_t* bar, uint32_t parity) {
+    const long long t0 = clock64();
+    while (!bar_try(bar, parity))
+        if (clock64() - t0 > (1ll << 31)) return false;
+    return true;
+}
+__device__ __forceinline__ void bar_inval(uint64_t* bar) {
+    asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(smem_addr(bar)) : "memory");
+}
+__device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
+    asm volatile(
+        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+            smem_addr(dst)),
+        "l"(src), "r"(bytes), "r"(smem_addr(bar))
+        : "memory");
+}
+
 // Features of one state, computed by one warp into out[kFeat] (shared memory). s: position;
 // (hc, hs): heading cos / sin; T1: the step of the plan samples to read (the next step);
 // skey: kSectors words of scratch in shared memory. The order of reading and of the
@@ -217,28 +265,35 @@ struct CollectArgs {
 };
 cudaError_t launch_collect(const CollectArgs& a, cudaStream_t s);
 
-// C[M x N] (fp32, row stride ldc) = op(A) op(B) (+ C when accumulate): A(i, k) at
-// A[i * sa_i + k * sa_k], B(k, j) at B[k * sb_k + j * sb_j], both bf16.
-cudaError_t launch_gemm_bf16(int M, int N, int K, const __nv_bfloat16* A, long sa_i, long sa_k,
-                             const __nv_bfloat16* B, long sb_k, long sb_j, float* C, int ldc, int accumulate,
-                             cudaStream_t s);
-// H (bf16) = act(Z + b): relu for hidden layers
-cudaError_t launch_bias_act(const float* Z, const float* b, __nv_bfloat16* H, int M, int N, int ldz, int ldh, int relu,
-                            cudaStream_t s);
-// mean softmax cross-entropy: loss added to *loss, dZ (bf16, ld) = (softmax - onehot) / M
-cudaError_t launch_softmax_ce(const float* Z, int ldz, const float* bias, const uint8_t* y, int M, int n_valid,
-                              __nv_bfloat16* dZ, int lddz, float* dZf, float* loss, cudaStream_t s);
-// dZ (bf16 and fp32) = dH * (H > 0)
-cudaError_t launch_relu_bwd(const float* dH, const __nv_bfloat16* H, int M, int N, __nv_bfloat16* dZ, float* dZf,
-                            cudaStream_t s);
-cudaError_t launch_colsum(const float* G, int M, int N, int ld, float* out, cudaStream_t s);
+// Loss and gradient of one batch (train.cu). Weight gradients are summed over kTrainSplit
+// stretches of the batch at most, each into its own copy of the parameters.
+constexpr int kTrainRows = 16;                 // rows per block of the forward / backward kernel
+constexpr int kTrainSplit = 8;
+constexpr int kTrainSums = 4 * kHid + kOutPad + 4;  // per block: output-gradient column sums, loss
+struct TrainArgs {
+    const float* Xf;           // fp32 features [M][kFeat], rounded to X by the kernel (or nullptr)
+    __nv_bfloat16* X;          // bf16 features [M][kFeat]
+    const uint8_t* y;          // labels
+    int32_t M, n_valid;        // rows; actions
+    const __nv_bfloat16* Wp;   // chunked bf16 weights
+    const float* params;       // fp32 master parameters (biases)
+    __nv_bfloat16* H;          // [4][M][kHid]: hidden activations
+    __nv_bfloat16* dZ;         // [4][M][kHid] then [M][kOutPad]: gradients of the layers' outputs
+    float* sums;               // [blocks][kTrainSums]
+    float* part;               // [kTrainSplit][n_params_total()]
+    float* grad;               // [n_params_total()]
+    float* loss;               // the batch's mean loss is added
+    int32_t* err;
+};
+inline int train_blocks(int M) { return (M + kTrainRows - 1) / kTrainRows; }
+cudaError_t prepare_train_kernels();
+cudaError_t launch_train(const TrainArgs& a, cudaStream_t s);
 cudaError_t launch_gather_rows(const __nv_bfloat16* X, const int32_t* idx, int M, __nv_bfloat16* out,
                                const uint8_t* y, uint8_t* y_out, cudaStream_t s);
-// Adam on the fp32 master parameters, then the bf16 copies (training layout W[in][out],
-// and the policy's chunk layout)
+// Adam on the fp32 master parameters, then the bf16 copy in the chunk layout
 cudaError_t launch_adam(float* p, const float* g, float* m1, float* m2, size_t n, float lr, float b1, float b2,
                         float eps, int t, cudaStream_t s);
-cudaError_t launch_export_weights(const float* p, __nv_bfloat16* Wt, __nv_bfloat16* Wp, cudaStream_t s);
+cudaError_t launch_export_weights(const float* p, __nv_bfloat16* Wp, cudaStream_t s);
 
 // Policy rollouts: each CTA carries kPolicyRows requests in lock step (one matrix row each)
 // and refills a finished row from the work queue.
