@@ -89,6 +89,23 @@ __device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t b
         : "memory");
 }
 
+__device__ __forceinline__ void ldsm4(uint32_t* r, const void* p) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(smem_addr(p))
+                 : "memory");
+}
+__device__ __forceinline__ void ldsm4_t(uint32_t* r, const void* p) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(smem_addr(p))
+                 : "memory");
+}
+// A fragment (16 rows x 16 k) of a row-major tile
+__device__ __forceinline__ void frag_a(uint32_t* r, const __nv_bfloat16* tile, int pad, int k, int lane) {
+    ldsm4(r, tile + (size_t)(lane & 15) * pad + k + (lane >> 4) * 8);
+}
+
 // Features of one state, computed by one warp into out[kFeat] (shared memory). s: position;
 // (hc, hs): heading cos / sin; T1: the step of the plan samples to read (the next step);
 // skey: kSectors words of scratch in shared memory. The order of reading and of the
@@ -295,10 +312,11 @@ cudaError_t launch_adam(float* p, const float* g, float* m1, float* m2, size_t n
                         float eps, int t, cudaStream_t s);
 cudaError_t launch_export_weights(const float* p, __nv_bfloat16* Wp, cudaStream_t s);
 
-// Policy rollouts: each CTA carries kPolicyRows requests in lock step (one matrix row each)
-// and refills a finished row from the work queue.
-constexpr int kPolicyRows = 32;
-constexpr int kWBufs = 4;       // weight chunk buffers: three chunks stream while one is used
+// Policy rollouts: a cluster of CTAs carries up to kPolicyRows requests in lock step (one
+// matrix row each), every CTA the features and states of its share of them, and refills a
+// finished row from the work queue.
+constexpr int kPolicyCluster = 4;
+constexpr int kPolicyRows = 64;
 constexpr int kPolicyThreads = 256;
 struct PolicyArgs {
     Model m;
@@ -315,15 +333,22 @@ struct PolicyArgs {
     float* traj;              // [n][cap][3]
     uint8_t* acts;            // [n][cap]
     RolloutOut* out;          // [n]
-    int32_t* err;
-    int32_t rows;             // requests per CTA: 16 or 32
+    int32_t rows;             // requests per cluster: a multiple of 16 up to kPolicyRows
     // 1: stop a proposal at the judge's step bound (a longer one would be rejected anyway)
     int32_t step_bound;
     double slack, climb_step;
 };
-// rows per CTA for n work items on n_sm multiprocessors: 32 when that still gives every
-// multiprocessor a CTA, else 16
-inline int policy_rows_for(int n, int n_sm) { return (n + 31) / 32 >= n_sm ? 32 : 16; }
+// rows per cluster for n work items on n_sm multiprocessors: as few 16-row tiles as give every
+// item a row at once, and its CTAs
+inline int policy_rows_for(int n, int n_sm) {
+    const int clusters = n_sm / kPolicyCluster > 0 ? n_sm / kPolicyCluster : 1;
+    const int tiles = (n + 16 * clusters - 1) / (16 * clusters);
+    return 16 * (tiles < 1 ? 1 : (tiles > kPolicyRows / 16 ? kPolicyRows / 16 : tiles));
+}
+inline int policy_ctas_for(int n, int rows, int n_sm) {
+    const int clusters = n_sm / kPolicyCluster > 0 ? n_sm / kPolicyCluster : 1, want = (n + rows - 1) / rows;
+    return kPolicyCluster * (want < clusters ? want : clusters);
+}
 size_t policy_smem_bytes();
 cudaError_t prepare_policy_kernel();
 cudaError_t launch_policy(const PolicyArgs& a, int n_ctas, cudaStream_t s);

@@ -41,23 +41,6 @@ struct TrainSmem {
 };
 static_assert(sizeof(TrainSmem) <= 232448, "shared memory of one block");
 
-__device__ __forceinline__ void ldsm4(uint32_t* r, const void* p) {
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-                 : "r"(smem_addr(p))
-                 : "memory");
-}
-__device__ __forceinline__ void ldsm4_t(uint32_t* r, const void* p) {
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-                 : "r"(smem_addr(p))
-                 : "memory");
-}
-// A fragment (16 rows x 16 k) of a row-major tile
-__device__ __forceinline__ void frag_a(uint32_t* r, const __nv_bfloat16* tile, int pad, int k, int lane) {
-    ldsm4(r, tile + (size_t)(lane & 15) * pad + k + (lane >> 4) * 8);
-}
-
 // The q-th chunk of a block's weight stream: its layer and its 64 inputs. Forward: layer by
 // layer; backward: the same chunks of layers 4 to 1 (each gives the gradients of 64 inputs).
 __device__ __forceinline__ void train_chunk(int q, int& l, int& kc) {
