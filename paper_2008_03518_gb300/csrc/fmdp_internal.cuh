@@ -418,6 +418,8 @@ struct LookArgs {
     Model m;
     TableView tab;
     int32_t S_scan;  // slots scanned per slice
+    int32_t by_index;  // 1: read the plan samples within reach from iv instead
+    IndexView iv;
     int32_t W;       // 1 .. kMaxLookahead
     int32_t cap;
     int32_t n_req;
@@ -435,9 +437,8 @@ struct LookArgs {
     // and see each other's wells; each publishes its state per step in mem
     int32_t cosim;
     int64_t t_start;
-    double* mem;   // [2][n_req][8]: x, y, z, vx, vy, vz, flying, alive (by step parity)
-    int32_t* bar;  // [2]: arrivals, generation of the grid barrier (zero before launch)
-    int32_t absent;  // self-test only: arrivals the barrier waits for that never come
+    double* mem;   // [2][n_req] records of 6 x {value, stamp} by step parity, and one that stays zero
+    int32_t absent;  // self-test only: aircraft to wait for whose records never come
     // speculative waves (not with cosim): CTA w plans work item idx[w] while w < *n_dev
     const int32_t* idx;
     const int32_t* n_dev;

@@ -217,7 +217,6 @@ struct fmdp_ctx {
 
     // batch co-simulation: per-step aircraft records and the grid barrier words
     DevArray<double> cs_mem;
-    DevArray<int32_t> cs_bar;
 
     // one-launch separation check (fmdp_sep_check): trajectory and report in mapped host memory
     MappedArray<float> chk_xyz;
@@ -385,6 +384,7 @@ void grow_keep(fmdp_ctx* c, DevArray<T>& a, size_t want, size_t keep) {
 
 constexpr int32_t kBatchDefault = 256;
 constexpr int32_t kBatchMax = 1024;
+constexpr int32_t kLookScanSlots = 256;   // see set_look_index
 constexpr int32_t kMaxStageItems = 2234;  // options.index_stage_items beyond this are refused when a plan starts
 
 // ------------------------------------------------------------------ host runtime (host_table.cu)
@@ -412,6 +412,7 @@ void launch_window_rollout(fmdp_ctx* c, const Geometry& g, const fmdp_request* r
                            uint8_t* acts, RolloutOut* out, bool trace);
 std::array<int32_t, 4> tune_key(const fmdp_ctx* c, int32_t wave);
 const fmdp_tune_entry* tune_lookup(const fmdp_ctx* c, int32_t wave);
+void set_look_index(fmdp_ctx* c, LookArgs& la);
 Geometry geometry_indexed(fmdp_ctx* c, int32_t S_scan, int32_t wave = 0);
 Geometry geometry(fmdp_ctx* c, int32_t S_hw);
 void check_request(fmdp_ctx* c, const fmdp_request& r);

@@ -170,6 +170,7 @@ void enqueue_wave(fmdp_ctx* c, const Geometry& g, int n_clusters, BatchBuffers& 
             la.m = c->model;
             la.tab = tv;
             la.S_scan = g.S_scan;
+            set_look_index(c, la);
             la.W = window_of(c);
             la.cap = cap;
             la.n_req = n_cap;

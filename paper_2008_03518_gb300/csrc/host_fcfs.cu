@@ -48,13 +48,13 @@ int32_t run_fcfs(fmdp_ctx* c, const fmdp_request* reqs, int32_t n, fmdp_result* 
             CK(cudaMemcpyAsync(B.slots.p, sl.data(), m * sizeof(int32_t), cudaMemcpyHostToDevice, c->stream));
             if (cosim) {  // all m requests fly together first; admission below in array order
                 require(m == n, FMDP_ERR_FULL, "not enough free slots for the co-simulated batch");
-                c->cs_mem.ensure((size_t)2 * n * 8);
-                c->cs_bar.ensure(2);
-                CK(cudaMemsetAsync(c->cs_bar.p, 0, 2 * sizeof(int32_t), c->stream));
+                c->cs_mem.ensure((size_t)(2 * n + 1) * 12);
+                CK(cudaMemsetAsync(c->cs_mem.p, 0, (size_t)(2 * n + 1) * 12 * sizeof(double), c->stream));
                 LookArgs la{};
                 la.m = c->model;
                 la.tab = table_view(c);
                 la.S_scan = g.S_scan;
+                set_look_index(c, la);
                 la.W = window_of(c);
                 la.cap = cap;
                 la.n_req = n;
@@ -67,7 +67,6 @@ int32_t run_fcfs(fmdp_ctx* c, const fmdp_request* reqs, int32_t n, fmdp_result* 
                 la.t_start = reqs[0].depart_step;
                 for (int32_t i = 1; i < n; ++i) la.t_start = std::min(la.t_start, reqs[i].depart_step);
                 la.mem = c->cs_mem.p;
-                la.bar = c->cs_bar.p;
                 la.absent = absent;
                 KernelTimer t(c, 0);
                 LAUNCH(c, launch_lookahead(la, c->stream));

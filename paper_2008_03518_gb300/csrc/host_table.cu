@@ -210,6 +210,15 @@ int32_t batch_size_of(const fmdp_ctx* c) { return c->opt.batch_size > 0 ? c->opt
 // lookahead window of the rollouts (Sec. IV "Forward project"); 1 is the one-step rule
 int32_t window_of(const fmdp_ctx* c) { return c->opt.lookahead_W > 1 ? c->opt.lookahead_W : 1; }
 
+// Lookahead rollouts read the plan samples within reach from the index once a slice has more
+// slots than a CTA has threads: up to there one load per thread covers a
+// slice (3136 slots: 30 000 cycles of a co-simulated step, 600 beside the other work by index).
+void set_look_index(fmdp_ctx* c, LookArgs& la) {
+    if (!c->index_on || la.S_scan <= kLookScanSlots) return;
+    la.by_index = 1;
+    la.iv = index_view(c);
+}
+
 // The lookahead rollout of one request (W > 1), written like the rollout kernel's.
 void launch_window_rollout(fmdp_ctx* c, const Geometry& g, const fmdp_request* req_dev, int32_t cap, float* traj,
                            uint8_t* acts, RolloutOut* out, bool trace) {
@@ -217,6 +226,7 @@ void launch_window_rollout(fmdp_ctx* c, const Geometry& g, const fmdp_request* r
     la.m = c->model;
     la.tab = table_view(c);
     la.S_scan = g.S_scan;
+    set_look_index(c, la);
     la.W = window_of(c);
     la.cap = cap;
     la.n_req = 1;

@@ -158,7 +158,7 @@ namespace {
 // activations of a layer are written to all four CTAs (distributed shared memory, one cluster
 // barrier per layer). Each CTA keeps the states of a quarter of the rows, reads the index for
 // their features, and chooses and takes their actions.
-// On GB300, 256 requests against 20 000 plans: 27 us per step before, 12.6 us now.
+// On GB300, 256 requests against 20 000 plans: 27 us per step before, 12.8 us now.
 constexpr int kActPad = kHid + 8;  // bf16 per activation row (bank-conflict-free fragment reads)
 constexpr int kPolicyCols = kHid / kPolicyCluster;    // columns of a hidden layer per CTA
 constexpr int kPolicyOut = kOutPad / kPolicyCluster;  // logits per CTA

@@ -9,26 +9,30 @@
 //                sample at t + j, velocity from t + j to t + j + 1) - hard-deck penalty;
 //   Q(a) = max over j with x_j inside the box; a is valid when x_1 is inside.
 //
-// One CTA per request, 256 threads. Per step:
-//   1. one thread per action builds its W projected states (the exact FP64 chain) and
-//      their fp32 offsets from s;
-//   2. goal terms per (action, sub-step) as a log2 offset from the goal term at s, from
-//      the exact identity d - d_s = (|o|^2 - 2 G.o) / (d + d_s), G = goal - s, o the offset,
-//      which keeps fp32 accurate to micrometres at any distance; static wells and the
-//      terrain clearance per (action, sub-step) in fp32 with an FP64 re-evaluation inside
-//      their bands;
-//   3. every (sub-step, slot) pair of the W slices: a culled distance test per pair; a
-//      pair within reach is handed to the warp, whose lanes (one per action) score its
-//      wells for that sub-step in fp32, deciding d < R in FP64 inside the band;
-//   4. per action, the W values g - N compared as (sign, log2 |g - N|), so that a large
-//      penalty at one sub-step leaves the goal term's resolution at the others; Q in FP64;
-//   5. argmax (lowest index on ties), near-tie record, exact FP64 advance, terminal tests.
+// One CTA per request, 256 threads. A step is a chain of four short phases with a barrier after
+// each; no unit is busy, so what counts is the length of each phase's instruction stream:
+//   1. side by side: the projected states per (action, sub-step) with box test, goal terms as a
+//      log2 offset from the goal term at s (from the exact identity d - d_s =
+//      (|o|^2 - 2 G.o) / (d + d_s), G = goal - s, o the offset, which keeps fp32 accurate to
+//      micrometres at any distance) and static wells; and a list of the plan samples (and, in
+//      a co-simulation, the other aircraft) with a well that can reach a projected state,
+//      collected by the other warps from the table's slices or from the spatial index;
+//   2. the list's samples, shared out between the warps, lanes = actions: wells in fp32, d < R
+//      in FP64 inside its band;
+//   3. penalty and clearance per (action, sub-step): the W values g - N as (sign, log2 |g - N|),
+//      so that a large penalty at one sub-step leaves the goal term's resolution at the others;
+//   4. one warp: the best value per action, argmax (lowest index on ties), near-tie record,
+//      exact FP64 advance, terminal tests.
+// On GB300: 60 plans and W = 10, 8.1 us per step with every pair scored by the warp that found
+// it and seven barriers, 6.4 us now; a co-simulation of 128 aircraft among 3000 plans, 23 us per
+// step with every slot read and a grid barrier, 7.2 us now.
 // Every decision that is a threshold (box, well radius, clearance, capture) is taken in
 // FP64 with the oracle's operation order wherever fp32 could be on the wrong side.
 #include <climits>
 #include <cmath>
 
 #include "fmdp_internal.cuh"
+#include "terrain.cuh"
 
 namespace fmdp {
 
@@ -37,9 +41,19 @@ namespace {
 constexpr int kLookThreads = 256;
 constexpr unsigned kFullMask = 0xffffffffu;
 
+constexpr int kLookList = 1024;  // samples the list of a step holds (more are scored where they are found)
+
+// A sample whose wells `wells` may reach a projected state of sub-step j: offset from s, velocity.
+struct LookItem {
+    float qx, qy, qz;
+    int what;  // wells | j << 16 | kind << 24
+    float vx, vy, vz;
+    int ref;   // slot, index item (within the row) or aircraft
+};
+enum { kLookSlot, kLookIndex, kLookMember };
+
 struct LookLayout {
-    size_t ox, oy, oz, inb, rel, lN, vsg, vlv, vlr, vls, keys, sums, stat, Dx, Dy, Dz, Dh, Dz2, hna, sg, Lk, Lq, Ls,
-        misc, total;
+    size_t ox, oy, oz, inb, rel, vsg, vlv, cmp, vls, keys, sums, stat, Dx, Dy, Dz, Dh, Dz2, list, misc, total;
 };
 
 __host__ __device__ inline LookLayout look_layout(int A, int W) {
@@ -52,28 +66,23 @@ __host__ __device__ inline LookLayout look_layout(int A, int W) {
     L.oz = o; o += AW * 4;
     L.inb = o; o += AW * 4;   // projected state inside the box
     L.rel = o; o += AW * 4;   // log2 of the goal term at x_j minus log2 of the goal term at s
-    L.lN = o; o += AW * 4;    // log2 of (penalty + deck) at x_j, -inf when zero
     L.vsg = o; o += AW * 4;   // value g - N at x_j: sign class (2 bits) and whether vlv is absolute
     L.vlv = o; o += AW * 4;   // log2 |g - N| (relative to n0, or absolute when penalty dominated)
-    L.vlr = o; o += AW * 4;   // log2 |g - N| relative to n0 (for comparisons)
     L.vls = o; o += AW * 4;   // log2 of the term scale max(g, N) relative to n0
     L.keys = o; o += AW * 4;  // float keys of the largest well log-value (MAX)
     al(8);
+    L.cmp = o; o += AW * 8;   // what orders the values: class, log2 |g - N| relative to n0 (signed)
     L.sums = o; o += AW * 8;  // fixed-point sums of well values (SUM)
     L.stat = o; o += (size_t)kMaxStatic * 3 * 4;  // static-well centres minus s (fp32)
-    al(8);
+    al(16);
     L.Dx = o; o += kHeadings * 8;    // exact moves per heading (FP64)
     L.Dy = o; o += kHeadings * 8;
     L.Dz = o; o += kMaxActions * 8;  // exact climb per action (FP64)
     L.Dh = o; o += kHeadings * 4 * 4;     // the moves as double-float: xh, xl, yh, yl per heading
     L.Dz2 = o; o += kMaxActions * 2 * 4;  // climb as double-float
-    L.hna = o; o += kMaxActions * 4;      // heading index after each action's turn
-    L.sg = o; o += kMaxActions * 4;       // per action: sign class of Q (-1, 0, 1), -2 invalid
-    al(8);
-    L.Lk = o; o += kMaxActions * 8;       // per action: log2 |Q| (FP64, absolute)
-    L.Lq = o; o += kMaxActions * 8;       // per action: log2 of the term scale max(g, N)
-    L.Ls = o; o += kMaxActions * 8;       // per action: argmax key
-    L.misc = o; o += 256;
+    al(16);
+    L.list = o; o += kLookList * sizeof(LookItem);
+    L.misc = o; o += 512;
     L.total = (o + 127) & ~size_t(127);
     return L;
 }
@@ -85,41 +94,61 @@ struct LookState {
     double step, cap2;
     float shx, shy, shz, slx, sly, slz;  // s as double-float
     float Ghx, Ghy, Ghz, Glx, Gly, Glz;  // goal - s as double-float
-    float Gx, Gy, Gz, ds, phi;           // goal - s (fp32), its length, log2 g(s) - n0
+    float phi;                           // log2 g(s) - n0
+    int64_t step_no;                     // co-simulation: the step's number
+    int64_t t;                           // the step
     int n0;                              // integer part of log2 of the goal term at s
     int h, k, done, status, near_ties;
     int tie_k, tie_a1, tie_a2;  // near-tie test of step tie_k still to do (tie_k < 0: none)
     int tie_s1, tie_s2;
     double tie_L1, tie_L2, tie_T1, tie_T2;
     int64_t row0;     // ring row of t + 1 for the current step
+    int n_list;       // samples found in this step (may exceed kLookList)
+    int late;         // co-simulation: a wait for another aircraft's record expired
+    float well[kMaxWells][4];  // tau, R^2, log2 gamma, log2 |r|
+    float reach[kMaxWells];    // R
 };
+static_assert(sizeof(LookState) <= 512, "see look_layout");
 
-// Grid barrier of a cooperative launch (all CTAs resident), bounded: false when the wait
-// ran past about a second of SM cycles.
-__device__ bool look_grid_sync(int32_t* bar, int n_ctas, int& gen) {
-    __syncthreads();
-    int ok = 1;
-    if (threadIdx.x == 0) {
-        __threadfence();
-        const int g = gen;
-        if (atomicAdd(&bar[0], 1) == n_ctas - 1) {
-            atomicExch(&bar[0], 0);
-            __threadfence();
-            atomicExch(&bar[1], g + 1);
-        } else {
-            const long long t0 = clock64();
-            while (atomicAdd(&bar[1], 0) == g) {
-                if (clock64() - t0 > (1ll << 31)) {
-                    ok = 0;
-                    break;
-                }
-                __nanosleep(100);
-            }
+// Co-simulation: an aircraft's state at one step, as six 16-byte words {value, stamp}. The stamp
+// (2 x last step it holds for, + 1 when flying) is in every word and a word is read and written
+// as one access, so a reader needs no fence: it reads until every stamp is at least its step's.
+// Two records per aircraft, by step parity: the one of step t is overwritten for step t + 2,
+// by then every other aircraft has published step t + 1, so it has read step t.
+struct LookRecord {
+    double v[6];  // x, y, z, vx, vy, vz
+    bool flying;
+};
+constexpr int64_t kStampForever = INT64_MAX / 4;
+__device__ __forceinline__ void put_word(double* p, double v, int64_t stamp) {
+    asm volatile("{\n\t.reg .b128 t;\n\tmov.b128 t, {%1, %2};\n\tst.relaxed.gpu.global.b128 [%0], t;\n\t}" ::"l"(p),
+                 "l"(__double_as_longlong(v)), "l"(stamp)
+                 : "memory");
+}
+__device__ __forceinline__ int64_t get_word(const double* p, double& v) {
+    long long x, stamp;
+    asm volatile("{\n\t.reg .b128 t;\n\tld.relaxed.gpu.global.b128 t, [%2];\n\tmov.b128 {%0, %1}, t;\n\t}"
+                 : "=l"(x), "=l"(stamp)
+                 : "l"(p)
+                 : "memory");
+    v = __longlong_as_double(x);
+    return stamp;
+}
+// reads record p, once it holds for step `step` (counted from 1); false after about a second
+__device__ __forceinline__ bool look_read(const double* p, int64_t step, LookRecord& r, bool patient) {
+    const long long t0 = clock64();
+    for (;;) {
+        int64_t least = INT64_MAX;
+#pragma unroll
+        for (int i = 0; i < 6; ++i) {
+            const int64_t stamp = get_word(p + 2 * i, r.v[i]);
+            least = min(least, stamp);
+            if (i == 0) r.flying = stamp & 1;
         }
-        gen = g + 1;
-        __threadfence();
+        if ((least >> 1) >= step) return true;
+        if (clock64() - t0 > (1ll << 31)) return false;
+        if (patient) __nanosleep(200);
     }
-    return __syncthreads_and(ok) != 0;
 }
 
 __device__ __forceinline__ unsigned long long look_sum_term(float l, float ref) {
@@ -143,21 +172,26 @@ __device__ __forceinline__ void lk_df_add(float& hi, float& lo, float dh, float 
     e = __fadd_rn(e, __fadd_rn(lo, dl));
     lk_fast_two_sum(s, e, hi, lo);
 }
-// log2 of the goal term |r_g| gamma^|G| at a state whose goal vector is the double-float G,
-// split as n0 (integer) + phi (fraction in [0, 1)); also |G| in fp32
-__device__ __forceinline__ void lk_goal_log(const Model& m, float Ghx, float Ghy, float Ghz, float Glx, float Gly,
-                                            float Glz, int& n0, float& phi, float& dsf) {
-    const float lg_hi = (float)m.lg64, lg_lo = (float)(m.lg64 - (double)(float)m.lg64);
-    const float l2r_hi = (float)m.log2rg, l2r_lo = (float)(m.log2rg - (double)(float)m.log2rg);
+// |G|^2 of a double-float G as a double-float, and its fp32 root
+__device__ __forceinline__ float lk_goal_dist(float Ghx, float Ghy, float Ghz, float Glx, float Gly, float Glz, float& Sh,
+                                              float& Sl) {
     const float p0 = Ghx * Ghx, p1 = Ghy * Ghy, p2 = Ghz * Ghz;
     const float e0 = fmaf(Ghx, Ghx, -p0), e1 = fmaf(Ghy, Ghy, -p1), e2 = fmaf(Ghz, Ghz, -p2);
     float s1, t1, s2, t2;
     lk_two_sum(p0, p1, s1, t1);
     lk_two_sum(s1, p2, s2, t2);
     const float lo = t1 + t2 + e0 + e1 + e2 + 2.f * (Ghx * Glx + Ghy * Gly + Ghz * Glz);
-    float Sh, Sl;
     lk_fast_two_sum(s2, lo, Sh, Sl);
-    const float rt = Sh > 0.f ? sqrtf(Sh) : 0.f;
+    return Sh > 0.f ? sqrtf(Sh) : 0.f;
+}
+// log2 of the goal term |r_g| gamma^|G| at a state whose goal vector is the double-float G,
+// split as n0 (integer) + phi (fraction in [0, 1))
+__device__ __forceinline__ void lk_goal_log(const Model& m, float Ghx, float Ghy, float Ghz, float Glx, float Gly,
+                                            float Glz, int& n0, float& phi) {
+    const float lg_hi = (float)m.lg64, lg_lo = (float)(m.lg64 - (double)(float)m.lg64);
+    const float l2r_hi = (float)m.log2rg, l2r_lo = (float)(m.log2rg - (double)(float)m.log2rg);
+    float Sh, Sl;
+    const float rt = lk_goal_dist(Ghx, Ghy, Ghz, Glx, Gly, Glz, Sh, Sl);
     const float rr = fmaf(-rt, rt, Sh);
     const float rl = rt > 0.f ? (rr + Sl) * (0.5f / rt) : 0.f;
     const float p = rt * lg_hi;
@@ -174,7 +208,6 @@ __device__ __forceinline__ void lk_goal_log(const Model& m, float Ghx, float Ghy
     if (fr < 0.f) { fr += 1.f; fl -= 1.f; }
     n0 = (int)fl;
     phi = fr;
-    dsf = rt;
 }
 
 // The exact FP64 projected state x_(j+1) of a move (Dxa, Dya, Dza) from s: j + 1 rounded
@@ -283,11 +316,81 @@ __device__ __noinline__ bool look_near_tie(int s1, double L1, double T1, int s2,
     return gap < M - 13.287712379549449;  // log2(1e-4)
 }
 
+// Scores one sample (the same in every lane) for every action (lanes) at its sub-step. hn, Dxy,
+// Dzf: the lane's heading after its turn and its move.
+struct LookScore {
+    const LookState* st;
+    int* keys;
+    unsigned long long* sums;
+    const double *Dx, *Dy, *Dz;
+};
+__device__ __forceinline__ void look_score(const LookArgs& a, const LookScore& c, const LookItem& it, int hn, float4 Dxy,
+                                           float2 Dzf) {
+    const Model& m = a.m;
+    const LookState* st = c.st;
+    const int lane = threadIdx.x & 31;
+    if (lane >= m.A) return;
+    const unsigned wells = (unsigned)it.what & 0xffffu;
+    const int j = (it.what >> 16) & 0xff, kind = it.what >> 24;
+    const float fj = (float)(j + 1);
+    const float px = fmaf(fj, Dxy.x, fj * Dxy.y), py = fmaf(fj, Dxy.z, fj * Dxy.w), pz = fmaf(fj, Dzf.x, fj * Dzf.y);
+    float mb = -INFINITY;
+    unsigned long long sb = 0ull;
+    for (unsigned left = wells; left; left &= left - 1u) {
+        const int w = __ffs(left) - 1;
+        const float tau = st->well[w][0];
+        const float ux = px - fmaf(tau, it.vx, it.qx), uy = py - fmaf(tau, it.vy, it.qy), uz = pz - fmaf(tau, it.vz, it.qz);
+        const float d2 = fmaf(ux, ux, fmaf(uy, uy, uz * uz));
+        const float R2 = st->well[w][1];
+        bool in = d2 < R2;
+        if (fabsf(d2 - R2) <= m.w_band[w]) {
+            if (kind == kLookMember) {
+                const double* rc = a.mem + ((size_t)(st->step_no & 1) * a.n_req + it.ref) * 12;
+                double v[6];
+                for (int i = 0; i < 6; ++i) get_word(rc + 2 * i, v[i]);
+                in = look_member_exact(m, w, st->s, c.Dx[hn], c.Dy[hn], c.Dz[lane], j, v[0], v[1], v[2], v[3], v[4], v[5]);
+            } else {
+                int64_t r1 = st->row0 + j;
+                r1 -= r1 >= a.tab.T_win ? a.tab.T_win : 0;
+                float4 P1, P2;
+                if (kind == kLookIndex) {
+                    const float4* p = a.iv.items + ((size_t)r1 * a.tab.S_pad + it.ref) * 2;
+                    P1 = __ldcg(p);
+                    P2 = __ldcg(p + 1);
+                } else {
+                    const size_t o1 = (size_t)r1 * a.tab.S_pad + it.ref;
+                    P1 = make_float4(a.tab.X[o1], a.tab.Y[o1], a.tab.Z[o1], 0.f);
+                    P2 = make_float4(__int_as_float(0x7fc00000), 0.f, 0.f, 0.f);
+                    if (st->t + j + 2 < a.tab.t_base + a.tab.T_win) {
+                        const int64_t r2 = r1 + 1 >= a.tab.T_win ? 0 : r1 + 1;
+                        const size_t o2 = (size_t)r2 * a.tab.S_pad + it.ref;
+                        P2 = make_float4(a.tab.X[o2], a.tab.Y[o2], a.tab.Z[o2], 0.f);
+                    }
+                }
+                in = look_well_exact(m, w, st->s, c.Dx[hn], c.Dy[hn], c.Dz[lane], j, P1.x, P1.y, P1.z, P2.x, P2.y, P2.z,
+                                     P2.x == P2.x);
+            }
+        }
+        if (in) {
+            const float l = fmaf(sqrtf(d2), st->well[w][2], st->well[w][3]);
+            mb = fmaxf(mb, l);
+            if (m.combine) sb += look_sum_term(l, m.sum_ref);
+        }
+    }
+    const int q = lane * a.W + j;
+    if (mb > -INFINITY) atomicMax(&c.keys[q], float_key(mb));
+    if (sb) atomicAdd(&c.sums[q], sb);
+}
+__device__ __noinline__ void look_score_over(const LookArgs& a, const LookScore& c, const LookItem& it, int hn, float4 Dxy,
+                                             float2 Dzf) {
+    look_score(a, c, it, hn, Dxy, Dzf);
+}
+
 }  // namespace
 
 size_t lookahead_smem_bytes(int A, int W) { return look_layout(A, W).total; }
 
-__global__ void __launch_bounds__(kLookThreads) lookahead_kernel(const __grid_constant__ LookArgs a) {
+__global__ void __launch_bounds__(kLookThreads, 2) lookahead_kernel(const __grid_constant__ LookArgs a) {
     extern __shared__ __align__(128) unsigned char lsm[];
     const Model& m = a.m;
     const int A = m.A, W = a.W, AW = A * W;
@@ -297,10 +400,8 @@ __global__ void __launch_bounds__(kLookThreads) lookahead_kernel(const __grid_co
     float* oz = reinterpret_cast<float*>(lsm + L.oz);
     int* inb = reinterpret_cast<int*>(lsm + L.inb);
     float* rel = reinterpret_cast<float*>(lsm + L.rel);
-    float* lN = reinterpret_cast<float*>(lsm + L.lN);
     int* vsg = reinterpret_cast<int*>(lsm + L.vsg);
     float* vlv = reinterpret_cast<float*>(lsm + L.vlv);
-    float* vlr = reinterpret_cast<float*>(lsm + L.vlr);
     float* vls = reinterpret_cast<float*>(lsm + L.vls);
     int* keys = reinterpret_cast<int*>(lsm + L.keys);
     unsigned long long* sums = reinterpret_cast<unsigned long long*>(lsm + L.sums);
@@ -310,11 +411,8 @@ __global__ void __launch_bounds__(kLookThreads) lookahead_kernel(const __grid_co
     double* Dz = reinterpret_cast<double*>(lsm + L.Dz);
     float* Dh = reinterpret_cast<float*>(lsm + L.Dh);    // [24][4]: xh, xl, yh, yl
     float* Dz2 = reinterpret_cast<float*>(lsm + L.Dz2);  // [32][2]: zh, zl
-    int* hna = reinterpret_cast<int*>(lsm + L.hna);
-    int* sga = reinterpret_cast<int*>(lsm + L.sg);
-    double* Lka = reinterpret_cast<double*>(lsm + L.Lk);
-    double* Lqa = reinterpret_cast<double*>(lsm + L.Lq);
-    unsigned long long* Ksa = reinterpret_cast<unsigned long long*>(lsm + L.Ls);
+    float2* cmp = reinterpret_cast<float2*>(lsm + L.cmp);
+    LookItem* list = reinterpret_cast<LookItem*>(lsm + L.list);
     LookState* st = reinterpret_cast<LookState*>(lsm + L.misc);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int wi = blockIdx.x;
@@ -381,6 +479,8 @@ __global__ void __launch_bounds__(kLookThreads) lookahead_kernel(const __grid_co
         st->s[2] = req.oz;
         st->h = 0;
         st->k = 0;
+        st->n_list = 0;
+        st->late = 0;
         st->near_ties = 0;
         st->tie_k = -1;
         st->step = __dmul_rn(req.speed_mps, m.dt);
@@ -416,6 +516,17 @@ __global__ void __launch_bounds__(kLookThreads) lookahead_kernel(const __grid_co
         st->done = cap0 || req.horizon <= 0;
         st->status = cap0 ? kStatusCaptured : FMDP_REJ_HORIZON;
     }
+    if (tid < m.n_wells) {
+        st->well[tid][0] = m.w_tau[tid];
+        st->well[tid][1] = m.w_R2[tid];
+        st->well[tid][2] = m.w_lg[tid];
+        st->well[tid][3] = m.w_L[tid];
+        st->reach[tid] = sqrtf(m.w_R2[tid]);
+    }
+    for (int q = tid; q < AW; q += kLookThreads) {
+        keys[q] = KEY_NONE;
+        sums[q] = 0ull;
+    }
     __syncthreads();
     // largest horizontal + vertical move of one sub-step (culling bound)
     float lstep = 0.f;
@@ -428,85 +539,88 @@ __global__ void __launch_bounds__(kLookThreads) lookahead_kernel(const __grid_co
     auto well_mask = [&](float qx, float qy, float qz, float vx, float vy, float vz, float rho) {
         unsigned msk = 0u;
         for (int w = 0; w < m.n_wells; ++w) {
-            const float tau = m.w_tau[w];
+            const float tau = st->well[w][0];
             const float cx = fmaf(tau, vx, qx), cy = fmaf(tau, vy, qy), cz = fmaf(tau, vz, qz);
-            const float lim = sqrtf(m.w_R2[w]) + rho + 1.f;
+            const float lim = st->reach[w] + rho + 1.f;
             if (fmaf(cx, cx, fmaf(cy, cy, cz * cz)) < lim * lim) msk |= 1u << w;
         }
         return msk;
     };
 
-    int gen = 0;
-    const int n_mem = a.cosim ? a.n_req : 0;
-    for (int64_t tc = a.cosim ? a.t_start : req.depart_step;; ++tc) {
-        const double* recs = nullptr;  // co-simulation: every aircraft's record of this step
-        if (a.cosim) {
-            double* mine = a.mem + ((size_t)(tc & 1) * n_mem + r) * 8;
-            if (tid == 0) {
-                const bool flying = !st->done && tc >= req.depart_step;
-                for (int c = 0; c < 3; ++c) {
-                    mine[c] = st->s[c];
-                    mine[3 + c] = st->k > 0 ? __ddiv_rn(__dsub_rn(st->s[c], st->prev[c]), m.dt) : 0.0;
-                }
-                mine[6] = flying ? 1.0 : 0.0;
-                mine[7] = st->done ? 0.0 : 1.0;
-            }
-            if (!look_grid_sync(a.bar, a.n_req + a.absent, gen)) {
-                if (tid == 0) {
-                    atomicExch(a.err, FMDP_ERR_TIMEOUT);
-                    st->done = 1;
-                }
-                __syncthreads();
-                break;
-            }
-            recs = a.mem + (size_t)(tc & 1) * n_mem * 8;
-            int alive = 0;
-            for (int q = tid; q < n_mem; q += kLookThreads) alive |= __ldcg(recs + (size_t)q * 8 + 7) != 0.0;
-            if (!__syncthreads_or(alive)) break;
-            if (st->done || tc < req.depart_step) continue;  // waiting for departure, or finished
-        } else if (st->done) {
-            break;
+    const bool act = lane < A;
+    const DeckGrid grid = m.hm ? deck_grid(m) : DeckGrid{};
+    const LookScore sc{st, keys, sums, Dx, Dy, Dz};
+    // ---- co-simulation: records of the other aircraft (see LookRecord). Before it departs an
+    // aircraft's record holds up to the step before, afterwards for ever; then its CTA is done.
+    const int n_mem = a.cosim ? a.n_req : 0, n_wait = n_mem + (a.cosim ? a.absent : 0);
+    auto record_of = [&](int64_t step, int who) { return a.mem + ((size_t)(step & 1) * n_mem + who) * 12; };
+    auto publish = [&](int64_t step, int64_t until, bool flying) {  // lanes 0 .. 5 of warp 0
+        if (tid < 6) {
+            const double v = tid < 3 ? st->s[tid] : (st->k > 0 ? __ddiv_rn(__dsub_rn(st->s[tid - 3], st->prev[tid - 3]), m.dt) : 0.0);
+            put_word(record_of(step, r) + 2 * tid, v, 2 * until + (flying ? 1 : 0));
         }
+    };
+    auto wait_all = [&](int64_t step) {  // every thread; false when a record did not come
+        bool ok = true;
+        LookRecord rec;
+        for (int q = tid; q < n_wait; q += kLookThreads) {
+            if (q == r) continue;
+            // (the absent aircraft of the self-test: a record that nobody writes)
+            ok = look_read(q < n_mem ? record_of(step, q) : a.mem + (size_t)2 * n_mem * 12, step, rec, true) && ok;
+            if (!ok) break;
+        }
+        return __syncthreads_and(ok) != 0;
+    };
+    int64_t step_no = 0;  // the step's number from a.t_start, counted from 1
+    bool late = false;
+    if (a.cosim) {
+        step_no = req.depart_step - a.t_start + 1;
+        if (st->done || step_no > 1) {
+            const int64_t until = st->done ? kStampForever : step_no - 1;
+            publish(0, until, false);
+            publish(1, until, false);
+            // until it departs, step by step (each wait is bounded): every aircraft has reached the
+            // step before when its record is replaced
+            // (one that never flies only sees the others start)
+            for (int64_t q = 1; !late && q < (st->done ? 2 : step_no); ++q) late = !wait_all(q);
+        }
+    }
+    for (; !late && !st->done; ++step_no) {
+        if (a.cosim) publish(step_no, step_no, true);
         const int k = st->k;
         const int64_t t = req.depart_step + k;
         const int64_t row0 = st->row0;  // ring row of t + 1
-        // ---- 1. per step: the goal term at s, static-well offsets, each action's heading
-        if (tid < A) {
-            int hn = st->h + m.dh[tid];
-            hn += hn < 0 ? 24 : 0;
-            hn -= hn >= 24 ? 24 : 0;
-            hna[tid] = hn;
-        } else if (tid == 64) {
+        // ---- 1. projected states and samples within reach, side by side
+        if (tid == kLookThreads - 1) {
             int n0;
-            float phi, dsf;
-            lk_goal_log(m, st->Ghx, st->Ghy, st->Ghz, st->Glx, st->Gly, st->Glz, n0, phi, dsf);
+            float phi;
+            lk_goal_log(m, st->Ghx, st->Ghy, st->Ghz, st->Glx, st->Gly, st->Glz, n0, phi);
             st->n0 = n0;
             st->phi = phi;
-            st->ds = dsf;
-            st->Gx = st->Ghx + st->Glx;
-            st->Gy = st->Ghy + st->Gly;
-            st->Gz = st->Ghz + st->Glz;
-        } else if (tid == 32) {
-            deferred_tie();  // the previous step's near-tie flag
-        } else if (tid >= 96 && tid - 96 < m.n_static) {
-            const int w = tid - 96;
-            const double* c = m.statics + 6 * w;
-            stc[3 * w] = (float)__dsub_rn(c[0], st->s[0]);
-            stc[3 * w + 1] = (float)__dsub_rn(c[1], st->s[1]);
-            stc[3 * w + 2] = (float)__dsub_rn(c[2], st->s[2]);
+            st->step_no = step_no;
+            st->t = t;
         }
-        for (int q = tid; q < AW; q += kLookThreads) {
-            keys[q] = KEY_NONE;
-            sums[q] = 0ull;
+        if (m.n_static > 0) {
+            for (int w = tid; w < m.n_static; w += kLookThreads) {
+                const double* c = m.statics + 6 * w;
+                stc[3 * w] = (float)__dsub_rn(c[0], st->s[0]);
+                stc[3 * w + 1] = (float)__dsub_rn(c[1], st->s[1]);
+                stc[3 * w + 2] = (float)__dsub_rn(c[2], st->s[2]);
+            }
+            __syncthreads();
         }
-        __syncthreads();
+        const int h0 = st->h;
+        auto turned = [&](int ac) {
+            int hn = h0 + m.dh[ac];
+            hn += hn < 0 ? 24 : 0;
+            return hn - (hn >= 24 ? 24 : 0);
+        };
         const float shx = st->shx, shy = st->shy, shz = st->shz, slx = st->slx, sly = st->sly, slz = st->slz;
-
-        // ---- 2. projected states (fp32 offsets (j + 1) * move), box test, goal-term offset,
-        // static wells, per (action, sub-step)
+        const float Gx = st->Ghx + st->Glx, Gy = st->Ghy + st->Gly, Gz = st->Ghz + st->Glz;
+        // fp32 offsets (j + 1) * move, box test, goal-term offset, static wells
         for (int q = tid; q < AW; q += kLookThreads) {
             const int ac = q / W, j = q - ac * W;
-            const int hn = hna[ac];
+            const int hn = turned(ac);
             const float fj = (float)(j + 1);
             const float px = fmaf(fj, Dh[4 * hn], fj * Dh[4 * hn + 1]);
             const float py = fmaf(fj, Dh[4 * hn + 2], fj * Dh[4 * hn + 3]);
@@ -521,10 +635,12 @@ __global__ void __launch_bounds__(kLookThreads) lookahead_kernel(const __grid_co
             else if (mb < -kBoxBandL) in = 0;
             else in = look_box_exact(m, st->s, Dx[hn], Dy[hn], Dz[ac], j) ? 1 : 0;
             inb[q] = in;
-            const float ex = st->Gx - px, ey = st->Gy - py, ez = st->Gz - pz;
+            float Sh, Sl;
+            const float ds = lk_goal_dist(st->Ghx, st->Ghy, st->Ghz, st->Glx, st->Gly, st->Glz, Sh, Sl);
+            const float ex = Gx - px, ey = Gy - py, ez = Gz - pz;
             const float d = sqrtf(fmaf(ex, ex, fmaf(ey, ey, ez * ez)));
-            const float num = fmaf(px, px, fmaf(py, py, pz * pz)) - 2.f * fmaf(st->Gx, px, fmaf(st->Gy, py, st->Gz * pz));
-            const float den = d + st->ds;
+            const float num = fmaf(px, px, fmaf(py, py, pz * pz)) - 2.f * fmaf(Gx, px, fmaf(Gy, py, Gz * pz));
+            const float den = d + ds;
             const float dd = den > 0.f ? num / den : 0.f;  // d(x_j) - d(s)
             rel[q] = dd * m.lg32;
             // static negative peaks (restricted volumes / terrain wells)
@@ -545,166 +661,183 @@ __global__ void __launch_bounds__(kLookThreads) lookahead_kernel(const __grid_co
             if (mbw > -INFINITY) atomicMax(&keys[q], float_key(mbw));
             if (sb) atomicAdd(&sums[q], sb);
         }
-        __syncthreads();
-
-        // ---- 3. plan wells: every (sub-step, slot) pair, warp-cooperative scoring
-        const int npairs = W * S;
+        int hn_l = 0;  // this lane's action
+        float4 Dxy_l = make_float4(0.f, 0.f, 0.f, 0.f);
+        float2 Dzf_l = make_float2(0.f, 0.f);
+        if (act) {
+            hn_l = turned(lane);
+            Dxy_l = *reinterpret_cast<const float4*>(Dh + 4 * hn_l);
+            Dzf_l = *reinterpret_cast<const float2*>(Dz2 + 2 * lane);
+        }
+        // appends the lanes' samples that have wells in reach (a warp together); those that no
+        // longer fit are scored at once
+        auto add = [&](const LookItem& it, bool have) {
+            const unsigned mask = __ballot_sync(kFullMask, have);
+            if (!mask) return;
+            int at = 0;
+            if (lane == __ffs(mask) - 1) at = atomicAdd(&st->n_list, __popc(mask));
+            at = __shfl_sync(kFullMask, at, __ffs(mask) - 1) + __popc(mask & ((1u << lane) - 1u));
+            if (have && at < kLookList) list[at] = it;
+#pragma unroll 1
+            for (unsigned over = __ballot_sync(kFullMask, have && at >= kLookList); over; over &= over - 1u) {
+                const int b = __ffs(over) - 1;
+                LookItem o;
+                o.qx = __shfl_sync(kFullMask, it.qx, b), o.qy = __shfl_sync(kFullMask, it.qy, b);
+                o.qz = __shfl_sync(kFullMask, it.qz, b), o.what = __shfl_sync(kFullMask, it.what, b);
+                o.vx = __shfl_sync(kFullMask, it.vx, b), o.vy = __shfl_sync(kFullMask, it.vy, b);
+                o.vz = __shfl_sync(kFullMask, it.vz, b), o.ref = __shfl_sync(kFullMask, it.ref, b);
+                look_score_over(a, sc, o, hn_l, Dxy_l, Dzf_l);
+                __syncwarp();
+            }
+        };
+        // a plan sample (P2.x NaN: the plan's last) as an item of sub-step j
+        auto plan_item = [&](float4 P1, float4 P2, int j, int kind, int ref) {
+            LookItem it;
+            it.qx = (P1.x - shx) - slx, it.qy = (P1.y - shy) - sly, it.qz = (P1.z - shz) - slz;
+            const bool has2 = P2.x == P2.x;
+            it.vx = has2 ? (P2.x - P1.x) * inv_dt : 0.f;
+            it.vy = has2 ? (P2.y - P1.y) * inv_dt : 0.f;
+            it.vz = has2 ? (P2.z - P1.z) * inv_dt : 0.f;
+            it.what = (int)well_mask(it.qx, it.qy, it.qz, it.vx, it.vy, it.vz, (float)(j + 1) * lstep) | j << 16 | kind << 24;
+            it.ref = ref;
+            return it;
+        };
         const int64_t t_hi = a.tab.t_base + a.tab.T_win;
-        for (int base = warp * 32; base < npairs; base += kLookThreads) {
-            const int idx = base + lane;
-            int j = 0, i = 0;
-            unsigned wm = 0u;  // wells of this pair that can reach a projected state of sub-step j
-            float p1x = 0.f, p1y = 0.f, p1z = 0.f, p2x = 0.f, p2y = 0.f, p2z = 0.f;
-            if (idx < npairs) {
-                j = idx / S;
-                i = idx - j * S;
-                const int64_t t1 = t + j + 1, t2 = t1 + 1;
-                if (t1 >= a.tab.t_base && t1 < t_hi) {
-                    int64_t r1 = row0 + j;  // rows of t + j + 1 and t + j + 2 (j < T_win)
-                    r1 -= r1 >= a.tab.T_win ? a.tab.T_win : 0;
-                    const size_t o1 = (size_t)r1 * a.tab.S_pad + i;
-                    p1x = a.tab.X[o1];
-                    p1y = a.tab.Y[o1];
-                    p1z = a.tab.Z[o1];
-                    p2x = __int_as_float(0x7fc00000);
-                    if (t2 < t_hi) {
-                        int64_t r2 = r1 + 1;
-                        r2 -= r2 >= a.tab.T_win ? a.tab.T_win : 0;
-                        const size_t o2 = (size_t)r2 * a.tab.S_pad + i;
-                        p2x = a.tab.X[o2];
-                        p2y = a.tab.Y[o2];
-                        p2z = a.tab.Z[o2];
+        if (a.by_index) {
+            // one warp per sub-step (the last warps first: the first ones have the projected
+            // states): the cells within reach, as in the one-step rollout, and the extra list
+            const IndexView& iv = a.iv;
+            for (int j = kLookThreads / 32 - 1 - warp; j < W; j += kLookThreads / 32) {
+                const int64_t t1 = t + j + 1;
+                if (t1 < a.tab.t_base || t1 >= t_hi) continue;
+                int64_t r1 = row0 + j;
+                r1 -= r1 >= a.tab.T_win ? a.tab.T_win : 0;
+                const int32_t* cs_row = iv.cstart + r1 * ((int64_t)iv.ncell + 1);
+                const float Rq = m.reach_base + (float)(j + 1) * lstep + m.tau_absmax * iv.vmax * 1.0001f + 2.f;
+                const float x = shx + slx, y = shy + sly;
+                auto cell_of = [&](float v, float o, int n) {
+                    const float g = floorf((v - o) * iv.inv_cell);
+                    return g < 0.f ? 0 : (g > (float)(n - 1) ? n - 1 : (int)g);
+                };
+                const int cx0 = cell_of(x - Rq, iv.x0, iv.ncx), cx1 = cell_of(x + Rq, iv.x0, iv.ncx);
+                const int cy0 = cell_of(y - Rq, iv.y0, iv.ncy), cy1 = cell_of(y + Rq, iv.y0, iv.ncy);
+                const int nrows = cy1 - cy0 + 1;
+                int e0 = 0, e1 = 0;  // item ranges, one per lane (lane 31: the extra list)
+                if (nrows < 32) {
+                    if (lane < nrows) {
+                        e0 = __ldcg(cs_row + (cy0 + lane) * iv.ncx + cx0);
+                        e1 = __ldcg(cs_row + (cy0 + lane) * iv.ncx + cx1 + 1);
                     }
-                    if (p1x == p1x) {
-                        const float qx = (p1x - shx) - slx, qy = (p1y - shy) - sly, qz = (p1z - shz) - slz;
-                        float vx = 0.f, vy = 0.f, vz = 0.f;
-                        if (p2x == p2x) {
-                            vx = (p2x - p1x) * inv_dt;
-                            vy = (p2y - p1y) * inv_dt;
-                            vz = (p2z - p1z) * inv_dt;
-                        }
-                        wm = well_mask(qx, qy, qz, vx, vy, vz, (float)(j + 1) * lstep);
+                } else if (lane == 0) {  // one range over full cell rows
+                    e0 = __ldcg(cs_row + cy0 * iv.ncx);
+                    e1 = __ldcg(cs_row + (cy1 + 1) * iv.ncx);
+                }
+                if (lane == 31) {
+                    e0 = __ldcg(cs_row + iv.ncell);
+                    e1 = e0 + __ldcg(iv.nextra + r1);
+                }
+                const int num = max(0, e1 - e0);
+                int at = num;  // inclusive prefix of the ranges' item counts
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int v = __shfl_up_sync(kFullMask, at, o);
+                    if (lane >= o) at += v;
+                }
+                const int total = __shfl_sync(kFullMask, at, 31), base = e0 - (at - num);
+                const float4* items = iv.items + (size_t)r1 * a.tab.S_pad * 2;
+                for (int i0 = 0; i0 < total; i0 += 32) {
+                    const int i = i0 + lane;
+                    int lo = 0;  // the range of item i: the first whose prefix exceeds i
+#pragma unroll
+                    for (int o = 16; o; o >>= 1) lo += __shfl_sync(kFullMask, at, lo + o - 1) <= i ? o : 0;
+                    const int id = __shfl_sync(kFullMask, base, lo) + i;
+                    LookItem it{};
+                    bool have = false;
+                    if (i < total) {
+                        const float4 P1 = __ldcg(items + 2 * (size_t)id), P2 = __ldcg(items + 2 * (size_t)id + 1);
+                        it = plan_item(P1, P2, j, kLookIndex, id);
+                        have = tag_visible(__float_as_int(P1.w), INT_MAX) && (it.what & 0xffff);
                     }
+                    add(it, have);
                 }
             }
-            unsigned mask = __ballot_sync(kFullMask, wm != 0u);
-            while (mask) {
-                const int b = __ffs(mask) - 1;
-                mask &= mask - 1;
-                const int jb = __shfl_sync(kFullMask, j, b);
-                const unsigned bwm = __shfl_sync(kFullMask, wm, b);
-                const float b1x = __shfl_sync(kFullMask, p1x, b), b1y = __shfl_sync(kFullMask, p1y, b),
-                            b1z = __shfl_sync(kFullMask, p1z, b);
-                const float b2x = __shfl_sync(kFullMask, p2x, b), b2y = __shfl_sync(kFullMask, p2y, b),
-                            b2z = __shfl_sync(kFullMask, p2z, b);
-                if (lane < A) {
-                    const int q = lane * W + jb;
-                    const bool has2 = b2x == b2x;
-                    const float qx = (b1x - shx) - slx, qy = (b1y - shy) - sly, qz = (b1z - shz) - slz;
-                    float vx = 0.f, vy = 0.f, vz = 0.f;
-                    if (has2) {
-                        vx = (b2x - b1x) * inv_dt;
-                        vy = (b2y - b1y) * inv_dt;
-                        vz = (b2z - b1z) * inv_dt;
-                    }
-                    const float px = ox[q], py = oy[q], pz = oz[q];
-                    float mb = -INFINITY;
-                    unsigned long long sb = 0ull;
-                    for (int w = 0; w < m.n_wells; ++w) {
-                        if (!((bwm >> w) & 1u)) continue;
-                        const float tau = m.w_tau[w];
-                        const float ux = px - fmaf(tau, vx, qx), uy = py - fmaf(tau, vy, qy), uz = pz - fmaf(tau, vz, qz);
-                        const float d2 = fmaf(ux, ux, fmaf(uy, uy, uz * uz));
-                        const float R2 = m.w_R2[w];
-                        bool in = d2 < R2;
-                        if (fabsf(d2 - R2) <= m.w_band[w]) {
-                            const int hn = hna[lane];
-                            in = look_well_exact(m, w, st->s, Dx[hn], Dy[hn], Dz[lane], jb, b1x, b1y, b1z, b2x, b2y,
-                                                 b2z, has2);
-                        }
-                        if (in) {
-                            const float l = fmaf(sqrtf(d2), m.w_lg[w], m.w_L[w]);
-                            mb = fmaxf(mb, l);
-                            if (m.combine) sb += look_sum_term(l, m.sum_ref);
+        } else {
+            // every (sub-step, slot) pair, two per thread and turn: their loads are in flight together
+            const int npairs = W * S;
+            for (int base = warp * 32; base < npairs; base += 2 * kLookThreads) {
+                float4 P1[2], P2[2];
+                int js[2];
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    const int idx = base + u * kLookThreads + lane;
+                    P1[u] = P2[u] = make_float4(__int_as_float(0x7fc00000), 0.f, 0.f, 0.f);
+                    js[u] = idx / S;
+                    const int64_t t1 = t + js[u] + 1;
+                    if (idx < npairs && t1 >= a.tab.t_base && t1 < t_hi) {
+                        const int i = idx - js[u] * S;
+                        int64_t r1 = row0 + js[u];  // rows of t + j + 1 and t + j + 2 (j < T_win)
+                        r1 -= r1 >= a.tab.T_win ? a.tab.T_win : 0;
+                        const size_t o1 = (size_t)r1 * a.tab.S_pad + i;
+                        P1[u] = make_float4(a.tab.X[o1], a.tab.Y[o1], a.tab.Z[o1], 0.f);
+                        if (t1 + 1 < t_hi) {
+                            const size_t o2 = (size_t)(r1 + 1 >= a.tab.T_win ? 0 : r1 + 1) * a.tab.S_pad + i;
+                            P2[u] = make_float4(a.tab.X[o2], a.tab.Y[o2], a.tab.Z[o2], 0.f);
                         }
                     }
-                    if (mb > -INFINITY) atomicMax(&keys[q], float_key(mb));
-                    if (sb) atomicAdd(&sums[q], sb);
+                }
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    if (base + u * kLookThreads >= npairs) break;  // (the same in the whole warp)
+                    LookItem it{};
+                    bool have = P1[u].x == P1[u].x;
+                    if (have) {
+                        it = plan_item(P1[u], P2[u], js[u], kLookSlot, base + u * kLookThreads + lane - js[u] * S);
+                        have = (it.what & 0xffff) != 0;
+                    }
+                    add(it, have);
                 }
             }
         }
-
-        // ---- 3'. co-simulation: the wells of every other aircraft in flight, at its
-        // position at t plus tau times its last move (the same peaks for every sub-step)
-        if (recs) {
-            const int nmp = W * n_mem;
-            for (int base = warp * 32; base < nmp; base += kLookThreads) {
-                const int idx = base + lane;
-                int j = 0;
-                unsigned wm = 0u;
-                double msx = 0.0, msy = 0.0, msz = 0.0, mvx = 0.0, mvy = 0.0, mvz = 0.0;
-                if (idx < nmp) {
-                    j = idx / n_mem;
-                    const int mm = idx - j * n_mem;
-                    const double* rc = recs + (size_t)mm * 8;
-                    if (mm != r && __ldcg(rc + 6) != 0.0) {
-                        msx = __ldcg(rc);
-                        msy = __ldcg(rc + 1);
-                        msz = __ldcg(rc + 2);
-                        mvx = __ldcg(rc + 3);
-                        mvy = __ldcg(rc + 4);
-                        mvz = __ldcg(rc + 5);
-                        const float qx = (float)__dsub_rn(msx, st->s[0]), qy = (float)__dsub_rn(msy, st->s[1]),
-                                    qz = (float)__dsub_rn(msz, st->s[2]);
-                        wm = well_mask(qx, qy, qz, (float)mvx, (float)mvy, (float)mvz, (float)(j + 1) * lstep);
-                    }
-                }
-                unsigned mask = __ballot_sync(kFullMask, wm != 0u);
-                while (mask) {
-                    const int b = __ffs(mask) - 1;
-                    mask &= mask - 1;
-                    const int jb = __shfl_sync(kFullMask, j, b);
-                    const unsigned bwm = __shfl_sync(kFullMask, wm, b);
-                    const double bsx = __shfl_sync(kFullMask, msx, b), bsy = __shfl_sync(kFullMask, msy, b),
-                                 bsz = __shfl_sync(kFullMask, msz, b);
-                    const double bvx = __shfl_sync(kFullMask, mvx, b), bvy = __shfl_sync(kFullMask, mvy, b),
-                                 bvz = __shfl_sync(kFullMask, mvz, b);
-                    if (lane < A) {
-                        const int q = lane * W + jb;
-                        const float qx = (float)__dsub_rn(bsx, st->s[0]), qy = (float)__dsub_rn(bsy, st->s[1]),
-                                    qz = (float)__dsub_rn(bsz, st->s[2]);
-                        const float vx = (float)bvx, vy = (float)bvy, vz = (float)bvz;
-                        const float px = ox[q], py = oy[q], pz = oz[q];
-                        float mb = -INFINITY;
-                        unsigned long long sb = 0ull;
-                        for (int w = 0; w < m.n_wells; ++w) {
-                            if (!((bwm >> w) & 1u)) continue;
-                            const float tau = m.w_tau[w];
-                            const float ux = px - fmaf(tau, vx, qx), uy = py - fmaf(tau, vy, qy),
-                                        uz = pz - fmaf(tau, vz, qz);
-                            const float d2 = fmaf(ux, ux, fmaf(uy, uy, uz * uz));
-                            const float R2 = m.w_R2[w];
-                            bool in = d2 < R2;
-                            if (fabsf(d2 - R2) <= m.w_band[w]) {
-                                const int hn = hna[lane];
-                                in = look_member_exact(m, w, st->s, Dx[hn], Dy[hn], Dz[lane], jb, bsx, bsy, bsz, bvx,
-                                                       bvy, bvz);
-                            }
-                            if (in) {
-                                const float l = fmaf(sqrtf(d2), m.w_lg[w], m.w_L[w]);
-                                mb = fmaxf(mb, l);
-                                if (m.combine) sb += look_sum_term(l, m.sum_ref);
-                            }
-                        }
-                        if (mb > -INFINITY) atomicMax(&keys[q], float_key(mb));
-                        if (sb) atomicAdd(&sums[q], sb);
-                    }
-                }
+        // co-simulation: the wells of every other aircraft in flight, at its position at t plus tau
+        // times its last move (the same peaks for every sub-step)
+        for (int q0 = warp * 32; q0 < n_wait; q0 += kLookThreads) {
+            const int q = q0 + lane;
+            LookRecord rec;
+            rec.flying = false;
+            if (q < n_wait && q != r &&
+                !look_read(q < n_mem ? record_of(step_no, q) : a.mem + (size_t)2 * n_mem * 12, step_no, rec, false)) {
+                st->late = 1;
+                rec.flying = false;
+            }
+            __syncwarp();
+            LookItem it{};
+            if (rec.flying) {
+                it.qx = (float)__dsub_rn(rec.v[0], st->s[0]);
+                it.qy = (float)__dsub_rn(rec.v[1], st->s[1]);
+                it.qz = (float)__dsub_rn(rec.v[2], st->s[2]);
+                it.vx = (float)rec.v[3], it.vy = (float)rec.v[4], it.vz = (float)rec.v[5];
+                it.ref = q;
+            }
+            for (int j = 0; j < W; ++j) {
+                const unsigned wells =
+                    rec.flying ? well_mask(it.qx, it.qy, it.qz, it.vx, it.vy, it.vz, (float)(j + 1) * lstep) : 0u;
+                it.what = (int)wells | j << 16 | kLookMember << 24;
+                add(it, wells != 0u);
             }
         }
         __syncthreads();
+        if (st->late) {  // (the same in every thread)
+            late = true;
+            break;
+        }
 
-        // ---- penalty + deck per (action, sub-step), as log2
+        // ---- 2. the list, shared out between the warps
+        const int n_list = min(st->n_list, kLookList);
+        for (int e = warp; e < n_list; e += kLookThreads / 32) look_score(a, sc, list[e], hn_l, Dxy_l, Dzf_l);
+        __syncthreads();
+
+        // ---- 3. penalty + deck per (action, sub-step), as log2
+        if (tid == 0) st->n_list = 0;
+        if (tid == kLookThreads - 32) deferred_tie();  // the previous step's near-tie flag
         for (int q = tid; q < AW; q += kLookThreads) {
             float P = 0.f;
             if (m.combine) {
@@ -712,20 +845,32 @@ __global__ void __launch_bounds__(kLookThreads) lookahead_kernel(const __grid_co
             } else if (keys[q] != KEY_NONE) {
                 P = exp2f(key_float(keys[q]));
             }
+            keys[q] = KEY_NONE;  // for the next step
+            if (m.combine) sums[q] = 0ull;
             float D = 0.f;
             if (m.hm) {
                 const float sx = shx + (slx + ox[q]), sy = shy + (sly + oy[q]), sz = shz + (slz + oz[q]);
                 const float c32 = sz - terrain32(m, sx, sy);
                 if (fabsf(c32 - (float)m.clearance) <= kClrBand + kTerrBand) {
-                    const int ac = q / W, hn = hna[ac];
-                    D = look_deck_exact(m, st->s, Dx[hn], Dy[hn], Dz[ac], q - ac * W);
+                    const int ac = q / W, hn = turned(ac), j = q - ac * W;
+                    // the projected state as double-float: off from the exact one by a rounding per
+                    // step and per sub-step
+                    float hx = shx, lx = slx, hy = shy, ly = sly, hz = shz, lz = slz;
+                    for (int i = 0; i <= j; ++i) {
+                        df_add(hx, lx, Dh[4 * hn], Dh[4 * hn + 1]);
+                        df_add(hy, ly, Dh[4 * hn + 2], Dh[4 * hn + 3]);
+                        df_add(hz, lz, Dz2[2 * ac], Dz2[2 * ac + 1]);
+                    }
+                    TerrainCell tc = terrain_cell(hx, hy, box0, box1, m.hm_sx, m.hm_sy, m.hm_nx, m.hm_ny);
+                    terrain_nodes(tc, m.hm, m.hm_nx);
+                    D = deck_band(m, grid, tc, hx, lx, hy, ly, hz, lz, k + j);
+                    if (D < 0.f) D = look_deck_exact(m, st->s, Dx[hn], Dy[hn], Dz[ac], j);
                 } else if (c32 < (float)m.clearance) {
                     D = (float)m.deck - c32;
                 }
             }
             const float N = P + D;
             const float ln = N > 0.f ? log2f(N) : -INFINITY;
-            lN[q] = ln;
             // the value g - N at x_j relative to 2^n0 (g = 2^(phi + rel), N = 2^(ln - n0))
             const float lg = st->phi + rel[q];
             int sg;
@@ -762,83 +907,80 @@ __global__ void __launch_bounds__(kLookThreads) lookahead_kernel(const __grid_co
             }
             vsg[q] = (sg + 1) | (vabs ? 4 : 0);
             vlv[q] = lv;
-            vlr[q] = vabs ? lv - (float)st->n0 : lv;
             vls[q] = lsc;
+            // order of the values: by sign, then by size; a sub-step outside the box counts only as
+            // the first
+            const float lr = vabs ? lv - (float)st->n0 : lv;
+            cmp[q] = make_float2(q % W > 0 && !inb[q] ? -2.f : (float)sg, sg > 0 ? lr : (sg < 0 ? -lr : 0.f));
         }
         __syncthreads();
 
-        // ---- 4. per action: the largest value over its projected states inside the box.
+        // ---- 4. per action (lanes): the largest value over its projected states inside the box.
         // Values are held relative to 2^n0 (n0: integer part of log2 of the goal term at s):
         // g = 2^(phi + rel), N = 2^(lN - n0); g - N as (sign, log2 |g - N|), which keeps the
         // goal term's resolution when N at another sub-step is larger by hundreds of binary
-        // orders. Only the winner per action is turned into an absolute FP64 log2.
-        if (tid < A) {
-            const int q0 = tid * W;
-            int bq = -1, bs = -2;
-            float br = 0.f;
-            for (int j = 0; j < W; ++j) {
-                const int q = q0 + j;
-                if (j > 0 && !inb[q]) continue;
-                const int sg = (vsg[q] & 3) - 1;
-                const float lr = vlr[q];
-                bool better;
-                if (bs == -2) better = true;
-                else if (sg != bs) better = sg > bs;
-                else better = sg > 0 ? lr > br : (sg < 0 ? lr < br : false);
-                if (better) {
-                    bq = q;
-                    bs = sg;
-                    br = lr;
-                }
-            }
-            const bool valid = inb[q0] != 0;
-            const bool babs = (vsg[bq] & 4) != 0;
-            const double Lk = babs ? (double)vlv[bq] : __dadd_rn((double)st->n0, (double)vlv[bq]);
-            sga[tid] = valid ? bs : -2;
-            Lka[tid] = Lk;
-            Lqa[tid] = __dadd_rn((double)st->n0, (double)vls[bq]);
-            Ksa[tid] = valid ? look_key(bs, Lk) : 0ull;
-        }
-        __syncthreads();
-
-        // ---- 5. argmax, near-tie record, advance (warp 0)
+        // orders. Only the winner per action is turned into an absolute FP64 log2. Then argmax,
+        // near-tie record, advance.
         if (warp == 0) {
-            const unsigned long long kq = lane < A ? Ksa[lane] : 0ull;
-            unsigned long long mx = kq;
-            for (int o = 16; o; o >>= 1) {
-                const unsigned long long y = __shfl_xor_sync(kFullMask, mx, o);
-                mx = y > mx ? y : mx;
+            int sgl = -2;
+            double Lkl = 0.0, Lql = 0.0;
+            unsigned long long kq = 0ull;
+            if (act) {
+                const int q0 = lane * W;
+                float2 v[kMaxLookahead];
+#pragma unroll
+                for (int j = 0; j < kMaxLookahead; ++j) v[j] = cmp[q0 + (j < W ? j : 0)];
+                int bj = 0;
+                float2 b = v[0];
+#pragma unroll
+                for (int j = 1; j < kMaxLookahead; ++j) {
+                    const bool better = v[j].x > b.x || (v[j].x == b.x && v[j].y > b.y);  // (j >= W: v[0], never)
+                    bj = better ? j : bj;
+                    b = better ? v[j] : b;
+                }
+                const int bq = q0 + bj;
+                const bool valid = inb[q0] != 0;
+                const int sg = (vsg[bq] & 3) - 1;
+                Lkl = (vsg[bq] & 4) ? (double)vlv[bq] : __dadd_rn((double)st->n0, (double)vlv[bq]);
+                Lql = __dadd_rn((double)st->n0, (double)vls[bq]);
+                sgl = valid ? sg : -2;
+                kq = valid ? look_key(sg, Lkl) : 0ull;
             }
+            // the largest of the lanes' 64-bit keys, by halves
+            auto largest = [&](unsigned long long v) {
+                const unsigned hi = __reduce_max_sync(kFullMask, (unsigned)(v >> 32));
+                const unsigned lo = __reduce_max_sync(kFullMask, (unsigned)(v >> 32) == hi ? (unsigned)v : 0u);
+                return (unsigned long long)hi << 32 | lo;
+            };
+            const unsigned long long mx = largest(kq);
             const unsigned bm = __ballot_sync(kFullMask, lane < A && kq == mx && mx != 0ull);
             const int a1 = bm ? __ffs(bm) - 1 : -1;
-            unsigned long long k2 = (lane < A && lane != a1) ? kq : 0ull;
-            for (int o = 16; o; o >>= 1) {
-                const unsigned long long y = __shfl_xor_sync(kFullMask, k2, o);
-                k2 = y > k2 ? y : k2;
-            }
+            const unsigned long long k2 = largest(lane < A && lane != a1 ? kq : 0ull);
             const unsigned b2 = __ballot_sync(kFullMask, lane < A && lane != a1 && kq == k2 && k2 != 0ull);
             const int a2 = b2 ? __ffs(b2) - 1 : -1;
-            if (a.trace && lane < A) {
-                const int sgl = sga[lane];
-                q_trace[(size_t)k * A + lane] = sgl == -2 ? -INFINITY : (sgl == 0 ? 0.0 : (double)sgl * exp2(Lka[lane]));
-            }
+            if (a.trace && lane < A)
+                q_trace[(size_t)k * A + lane] = sgl == -2 ? -INFINITY : (sgl == 0 ? 0.0 : (double)sgl * exp2(Lkl));
+            const int c1 = max(a1, 0), c2 = max(a2, 0);
+            const int s1 = __shfl_sync(kFullMask, sgl, c1), s2 = __shfl_sync(kFullMask, sgl, c2);
+            const double L1 = __shfl_sync(kFullMask, Lkl, c1), L2 = __shfl_sync(kFullMask, Lkl, c2);
+            const double T1 = __shfl_sync(kFullMask, Lql, c1), T2 = __shfl_sync(kFullMask, Lql, c2);
             if (lane == 0) {
                 st->tie_k = k;  // tested during the next step (deferred_tie)
                 st->tie_a1 = a1;
                 st->tie_a2 = a2;
                 if (a1 >= 0 && a2 >= 0) {
-                    st->tie_s1 = sga[a1];
-                    st->tie_s2 = sga[a2];
-                    st->tie_L1 = Lka[a1];
-                    st->tie_L2 = Lka[a2];
-                    st->tie_T1 = Lqa[a1];
-                    st->tie_T2 = Lqa[a2];
+                    st->tie_s1 = s1;
+                    st->tie_s2 = s2;
+                    st->tie_L1 = L1;
+                    st->tie_L2 = L2;
+                    st->tie_T1 = T1;
+                    st->tie_T2 = T2;
                 }
                 if (a1 < 0) {
                     st->status = FMDP_REJ_NO_ACTION;
                     st->done = 1;
                 } else {
-                    const int hn = hna[a1];
+                    const int hn = turned(a1);
                     // exact advance (FP64, the oracle's x_1) and its double-float copies
                     st->prev[0] = st->s[0];
                     st->prev[1] = st->s[1];
@@ -882,6 +1024,14 @@ __global__ void __launch_bounds__(kLookThreads) lookahead_kernel(const __grid_co
         }
         __syncthreads();
     }
+    if (a.cosim && !late && step_no > req.depart_step - a.t_start + 1) {
+        // the record of the first step not flown, then, once every other aircraft has it or its own,
+        // the other one
+        publish(step_no, kStampForever, false);
+        late = !wait_all(step_no);
+        if (!late) publish(step_no + 1, kStampForever, false);
+    }
+    if (late && tid == 0) atomicExch(a.err, FMDP_ERR_TIMEOUT);
     if (tid == 0) {
         deferred_tie();
         RolloutOut o;

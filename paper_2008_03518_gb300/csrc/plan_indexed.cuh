@@ -338,83 +338,6 @@ __device__ __noinline__ void fold_overflow(const RolloutArgs& a, const IdxState*
     f.sloc = g.sloc;
 }
 
-// Heightmap origin, node spacing and nodes per metre as double-float.
-struct DeckGrid {
-    float bxh, bxl, byh, byl, cxh, cxl, cyh, cyl, sxh, sxl, syh, syl;
-};
-__device__ __forceinline__ DeckGrid deck_grid(const Model& m) {
-    DeckGrid g;
-    auto df = [](double v, float& h, float& l) {
-        h = (float)v;
-        l = (float)(v - (double)h);
-    };
-    const double wx = m.box[3] - m.box[0], wy = m.box[4] - m.box[1];
-    const double nx = (double)(m.hm_nx - 1), ny = (double)(m.hm_ny - 1);
-    df(m.box[0], g.bxh, g.bxl), df(m.box[1], g.byh, g.byl);
-    df(wx / nx, g.cxh, g.cxl), df(wy / ny, g.cyh, g.cyl);
-    df(nx / wx, g.sxh, g.sxl), df(ny / wy, g.syh, g.syl);
-    return g;
-}
-// double-float products and sums (relative error of a few 2^-46)
-__device__ __forceinline__ float2 df_mul(float2 a, float2 b) {
-    const float p = __fmul_rn(a.x, b.x);
-    const float e = fmaf(a.x, b.x, -p) + fmaf(a.x, b.y, __fmul_rn(a.y, b.x));
-    float2 r;
-    fast_two_sum(p, e, r.x, r.y);
-    return r;
-}
-__device__ __forceinline__ float2 df_sum(float2 a, float2 b) {
-    float s, e;
-    two_sum(a.x, b.x, s, e);
-    e = __fadd_rn(e, __fadd_rn(a.y, b.y));
-    float2 r;
-    fast_two_sum(s, e, r.x, r.y);
-    return r;
-}
-__device__ __forceinline__ float2 df_diff(float a, float b) {
-    float2 r;
-    two_sum(a, -b, r.x, r.y);
-    return r;
-}
-
-// Clearance penalty of a successor (double-float position) whose fp32 clearance lies in the FP64
-// band (one lane; step k). The band is wide because fp32 coordinates are, and a path along the
-// clearance limit enters it in a quarter of its steps; the FP64 evaluation takes some 5000
-// cycles here. In double-float the clearance c is good to nanometres plus what the position
-// has drifted from the exact state (one rounding per step), so both the decision c < clearance
-// and the fp32 value of deck - c are those of FP64 unless one lies within that error of a
-// threshold: then, and only then, FP64 decides. Returns the penalty, or -1 for FP64 to decide.
-__device__ __noinline__ float deck_band(const Model& m, const DeckGrid g, const TerrainCell t, float hx, float lx, float hy,
-                                        float ly, float hz, float lz, int k) {
-    // position in the cell: offset from its node (b + i c), times the nodes per metre
-    auto frac = [](float h, float l, int i, float bh, float bl, float ch, float cl, float sh, float sl) {
-        const float2 at = df_mul(make_float2((float)i, 0.f), make_float2(ch, cl));
-        const float2 u = df_sum(df_sum(make_float2(h, l), make_float2(-bh, -bl)), make_float2(-at.x, -at.y));
-        return df_mul(u, make_float2(sh, sl));
-    };
-    const float2 ax = frac(hx, lx, t.ix, g.bxh, g.bxl, g.cxh, g.cxl, g.sxh, g.sxl);
-    const float2 ay = frac(hy, ly, t.iy, g.byh, g.byl, g.cyh, g.cyl, g.syh, g.syl);
-    const float2 lo = df_sum(make_float2(t.h00, 0.f), df_mul(ax, df_diff(t.h10, t.h00)));
-    const float2 hi = df_sum(make_float2(t.h01, 0.f), df_mul(ax, df_diff(t.h11, t.h01)));
-    const float2 T = df_sum(lo, df_mul(ay, df_sum(hi, make_float2(-lo.x, -lo.y))));
-    const float2 c = df_sum(make_float2(hz, lz), make_float2(-T.x, -T.y));
-    const float2 over = df_sum(c, make_float2(-(float)m.clearance, -(float)(m.clearance - (double)(float)m.clearance)));
-    const float deckh = (float)m.deck;
-    const float2 V = df_sum(make_float2(deckh, (float)(m.deck - (double)deckh)), make_float2(-c.x, -c.y));
-    // error of c: the position's drift times the slope, and the arithmetic above
-    const float H = fmaxf(fmaxf(fabsf(t.h00), fabsf(t.h10)), fmaxf(fabsf(t.h01), fabsf(t.h11)));
-    const float slope = 1.f + 4.f * H * fmaxf(g.sxh, g.syh);
-    const float err = 1e-14f * (float)(k + 2) * (fabsf(hx) + fabsf(hy) + fabsf(hz)) * slope + 1e-11f * (H + fabsf(hz) + deckh) +
-                      1e-12f * slope * (fabsf(hx) + fabsf(hy) + fabsf(g.bxh) + fabsf(g.byh));
-    // half the spacing of fp32 numbers at V: the rounding of deck - c is certain if |V.y| is clear of it
-    const float half = 0.5f * (__uint_as_float(__float_as_uint(fabsf(V.x)) + 1u) - fabsf(V.x));
-    if (fabsf(over.x) > 2.f * err) {
-        if (over.x > 0.f) return 0.f;
-        if (fabsf(V.y) < half - 2.f * err && V.x > 1.f) return V.x;
-    }
-    return -1.f;
-}
-
 // Near-tie flag of step k0 + c (one warp).
 template <bool GEN>
 __device__ __forceinline__ void tie_step(const RolloutArgs& a, IdxState* st, int r, int k0, int c, int best) {

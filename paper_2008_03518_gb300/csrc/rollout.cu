@@ -31,6 +31,7 @@
 #include <climits>
 
 #include "fmdp_internal.cuh"
+#include "terrain.cuh"
 #include "sep_pair.cuh"
 
 namespace fmdp {
@@ -134,22 +135,6 @@ __device__ __forceinline__ void st_async_u64(uint32_t addr, unsigned long long v
 }
 
 // ---- double-float (fp32 pair) arithmetic: exact sums of fp32 numbers
-__device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
-    s = __fadd_rn(a, b);
-    const float bb = __fsub_rn(s, a);
-    e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
-}
-__device__ __forceinline__ void fast_two_sum(float a, float b, float& s, float& e) {
-    s = __fadd_rn(a, b);
-    e = __fsub_rn(b, __fsub_rn(s, a));
-}
-// (hi, lo) += (dh, dl)
-__device__ __forceinline__ void df_add(float& hi, float& lo, float dh, float dl) {
-    float s, e;
-    two_sum(hi, dh, s, e);
-    e = __fadd_rn(e, __fadd_rn(lo, dl));
-    fast_two_sum(s, e, hi, lo);
-}
 // a . b, the z product fused last and the y product rounded
 __device__ __forceinline__ float dot3(float ax, float ay, float az, float bx, float by, float bz) {
     return fmaf(az, bz, fmaf(ax, bx, __fmul_rn(ay, by)));
@@ -396,34 +381,6 @@ __device__ __forceinline__ unsigned long long sum_term(float l, float ref) {
 // with explicit fused operations: left to the compiler, which product of a sum is fused may
 // differ from one inlined copy to the next, and two actions' values often differ by less than
 // that rounding.
-struct TerrainCell {  // heightmap cell under a successor, and the position in it
-    int ix, iy;
-    float ax, ay;
-    float h00, h10, h01, h11;
-};
-__device__ __forceinline__ TerrainCell terrain_cell(float sx, float sy, float box0, float box1, float hm_sx, float hm_sy,
-                                                    int hm_nx, int hm_ny) {
-    TerrainCell t;
-    const float ux = __fsub_rn(sx, box0), uy = __fsub_rn(sy, box1);
-    t.ix = (int)floorf(__fmul_rn(ux, hm_sx)), t.iy = (int)floorf(__fmul_rn(uy, hm_sy));
-    t.ix = min(max(t.ix, 0), hm_nx - 2);
-    t.iy = min(max(t.iy, 0), hm_ny - 2);
-    t.ax = fmaf(ux, hm_sx, -(float)t.ix);
-    t.ay = fmaf(uy, hm_sy, -(float)t.iy);
-    return t;
-}
-__device__ __forceinline__ void terrain_nodes(TerrainCell& t, const float* __restrict__ hm, int hm_nx) {
-    const float* r0 = hm + (size_t)t.iy * hm_nx + t.ix;
-    t.h00 = __ldg(r0);
-    t.h10 = __ldg(r0 + 1);
-    t.h01 = __ldg(r0 + hm_nx);
-    t.h11 = __ldg(r0 + hm_nx + 1);
-}
-__device__ __forceinline__ float terrain_height(const TerrainCell& t) {
-    const float bx = __fsub_rn(1.f, t.ax), by = __fsub_rn(1.f, t.ay);
-    const float lo = fmaf(bx, t.h00, __fmul_rn(t.ax, t.h10)), hi = fmaf(bx, t.h01, __fmul_rn(t.ax, t.h11));
-    return fmaf(by, lo, __fmul_rn(t.ay, hi));
-}
 // least distance of a successor to a box face (negative outside)
 __device__ __forceinline__ float box_margin(float sx, float sy, float sz, float box0, float box1, float box2, float box3,
                                             float box4, float box5) {
