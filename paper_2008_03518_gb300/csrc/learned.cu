@@ -56,7 +56,10 @@ __global__ void __launch_bounds__(256) collect_kernel(const __grid_constant__ Co
             const float* p = a.traj + ((size_t)r * a.cap + k) * 3;
             float hc, hs;
             heading_cs(c0, s0, head[k - k0], hc, hs);
-            warp_features(a.m, a.iv, a.tab, req.depart_step + k + 1, p[0], p[1], p[2], hc, hs,
+            const int64_t T1 = req.depart_step + k + 1;
+            const int64_t row1 = T1 % a.tab.T_win;
+            const bool held = T1 >= a.tab.t_base && T1 < a.tab.t_base + a.tab.T_win;
+            warp_features(a.m, a.iv, a.tab, held ? (int)(row1 < 0 ? row1 + a.tab.T_win : row1) : -1, p[0], p[1], p[2], hc, hs,
                           (float)req.speed_mps, (float)req.gx, (float)req.gy, (float)req.gz, inv_dt, feat[warp],
                           skey[warp]);
             const size_t row = (size_t)a.row0[r] + k;
@@ -158,7 +161,8 @@ namespace {
 // activations of a layer are written to all four CTAs (distributed shared memory, one cluster
 // barrier per layer). Each CTA keeps the states of a quarter of the rows, reads the index for
 // their features, and chooses and takes their actions.
-// On GB300, 256 requests against 20 000 plans: 27 us per step before, 12.8 us now.
+// On GB300, 256 requests against 20 000 plans: 27 us per step before, 11.3 us now (12.8 with one
+// warp per state reading the index).
 constexpr int kActPad = kHid + 8;  // bf16 per activation row (bank-conflict-free fragment reads)
 constexpr int kPolicyCols = kHid / kPolicyCluster;    // columns of a hidden layer per CTA
 constexpr int kPolicyOut = kOutPad / kPolicyCluster;  // logits per CTA
@@ -169,7 +173,8 @@ struct PolicyRow {
     double s[3];
     double c0, s0, step, cap2;
     double gx, gy, gz;          // the request's goal, kept so a step reads no request
-    int64_t t1;                 // time step of the next sample
+    int32_t row1;               // index row of the first step's samples
+    int32_t k_lo, k_hi;         // steps whose samples lie in the table window: [k_lo, k_hi)
     float speed;
     int32_t horizon;
     int32_t req, k, h, status;  // req < 0: empty
@@ -284,7 +289,11 @@ __global__ void __cluster_dims__(kPolicyCluster, 1, 1) __launch_bounds__(kPolicy
                 R.gx = q.gx;
                 R.gy = q.gy;
                 R.gz = q.gz;
-                R.t1 = q.depart_step + 1;
+                const int64_t T1 = q.depart_step + 1, T0 = a.tab.t_base;
+                const int64_t row1 = T1 % a.tab.T_win;
+                R.row1 = (int32_t)(row1 < 0 ? row1 + a.tab.T_win : row1);
+                R.k_lo = (int32_t)min(max(T0 - T1, (int64_t)0), (int64_t)INT_MAX);
+                R.k_hi = (int32_t)min(max(T0 + a.tab.T_win - T1, (int64_t)0), (int64_t)INT_MAX);
                 R.speed = (float)q.speed_mps;
                 R.horizon = q.horizon;
                 if (a.step_bound) {  // the judge rejects anything longer: stop there
@@ -318,19 +327,23 @@ __global__ void __cluster_dims__(kPolicyCluster, 1, 1) __launch_bounds__(kPolicy
         if (tid < kPolicyCluster)  // (two sets: a CTA may be one step ahead of a peer's reads)
             peer_store(peer_addr(smem_addr(&S.flags[it & 1][rank]), tid), (uint32_t)(any | 2 * S.more));
         // ---- features of this CTA's rows (one warp per row) into every CTA's act[0]
-        for (int rr = warp; rr < own; rr += NWp) {
-            const PolicyRow R = rows[rr];
+        // (with at most four rows per CTA two warps share each row's samples)
+        const int parts = 2 * own <= NWp ? 2 : 1, part = parts == 2 ? warp / (NWp / 2) : 0;
+        for (int rr = parts == 2 ? warp % (NWp / 2) : warp; rr < own; rr += NWp / parts) {
+            const PolicyRow& R = rows[rr];
             uint2 v = make_uint2(0u, 0u);
+            float* feat = S.feat[rr % NWp];
             if (R.req >= 0) {
                 float hc, hs;
                 heading_cs((float)R.c0, (float)R.s0, R.h, hc, hs);
-                float* feat = S.feat[warp];
-                warp_features(m, a.iv, a.tab, R.t1 + R.k, (float)R.s[0], (float)R.s[1], (float)R.s[2], hc, hs, R.speed,
-                              (float)R.gx, (float)R.gy, (float)R.gz, inv_dt, feat, S.skey[warp]);
-                __syncwarp();
+                const bool held = R.k >= R.k_lo && R.k < R.k_hi;
+                const int row = R.row1 + R.k - (R.row1 + R.k >= a.tab.T_win ? a.tab.T_win : 0);
+                warp_features(m, a.iv, a.tab, held ? row : -1, (float)R.s[0], (float)R.s[1], (float)R.s[2], hc, hs, R.speed,
+                              (float)R.gx, (float)R.gy, (float)R.gz, inv_dt, feat, S.skey[rr % NWp], part, parts, 1 + rr);
                 v = make_uint2(pack_bf16(feat[4 * lane], feat[4 * lane + 1]), pack_bf16(feat[4 * lane + 2], feat[4 * lane + 3]));
                 __syncwarp();
             }
+            if (part > 0) continue;
             const uint32_t off = (uint32_t)(((first + rr) * kActPad + 4 * lane) * sizeof(__nv_bfloat16));
 #pragma unroll
             for (int c = 0; c < kPolicyCluster; ++c) peer_store(act_peer[c] + off, v);
