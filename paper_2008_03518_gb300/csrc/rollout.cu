@@ -1162,26 +1162,50 @@ __device__ void pipe_finish(const RolloutArgs& a, int r, int token, int* red, lo
         const int cx0 = cell_of(px - reach, iv.x0, iv.ncx), cx1 = cell_of(px + reach, iv.x0, iv.ncx);
         const int cy0 = cell_of(py - reach, iv.y0, iv.ncy), cy1 = cell_of(py + reach, iv.y0, iv.ncy);
         bool hit = false;
-        for (int cy = cy0; cy <= cy1 + 1 && !hit; ++cy) {
-            int b, e;
-            if (cy <= cy1) {
-                b = __ldcg(cs_row + cy * iv.ncx + cx0);
-                e = __ldcg(cs_row + cy * iv.ncx + cx1 + 1);
-            } else {  // the extra list
-                b = __ldcg(cs_row + iv.ncell);
-                e = b + __ldcg(iv.nextra + row);
-            }
-            for (int j = b; j < e; ++j) {
-                const float4 Q = __ldcg(items + 2 * (size_t)j);
-                if (!tag_visible(__float_as_int(Q.w), my_ord)) continue;
-                float h2, dz;
-                bool hin, vin;
-                sep_pair(sk, px, py, pz, Q.x, Q.y, Q.z, h2, dz, hin, vin);
-                if (hin && vin) {
-                    hit = true;
-                    break;
+        // Nothing here but the latency of dependent loads (a thread has a few samples only): the
+        // bounds of three cell rows and the extra list are loaded together, then items eight at
+        // a time. One load after another, the end of a 1200-step plan took 70 to 100 us of its
+        // 1.4 ms with 130 items to a row; 1000 requests against 3000 plans: 119 -> 109 ms.
+        for (int cy = cy0; !hit; cy += 3) {
+            const bool last = cy + 3 > cy1;
+            int b[4], e[4];
+#pragma unroll
+            for (int q = 0; q < 3; ++q) {
+                b[q] = e[q] = 0;
+                if (cy + q <= cy1) {
+                    b[q] = __ldcg(cs_row + (cy + q) * iv.ncx + cx0);
+                    e[q] = __ldcg(cs_row + (cy + q) * iv.ncx + cx1 + 1);
                 }
             }
+            b[3] = e[3] = 0;
+            if (last) {  // the extra list
+                b[3] = __ldcg(cs_row + iv.ncell);
+                e[3] = __ldcg(iv.nextra + row);
+                e[3] += b[3];
+            }
+#pragma unroll 1
+            for (int q = 0; q < 4 && !hit; ++q) {
+                const int bq = q == 0 ? b[0] : (q == 1 ? b[1] : (q == 2 ? b[2] : b[3]));
+                const int eq = q == 0 ? e[0] : (q == 1 ? e[1] : (q == 2 ? e[2] : e[3]));
+                constexpr int U = 8;
+                for (int j = bq; j < eq && !hit; j += U) {
+                    float4 Q[U];
+#pragma unroll
+                    for (int u = 0; u < U; ++u) {
+                        Q[u].w = __int_as_float(-1);  // (no plan)
+                        if (j + u < eq) Q[u] = __ldcg(items + 2 * (size_t)(j + u));
+                    }
+#pragma unroll
+                    for (int u = 0; u < U; ++u) {
+                        if (!tag_visible(__float_as_int(Q[u].w), my_ord)) continue;
+                        float h2, dz;
+                        bool hin, vin;
+                        sep_pair(sk, px, py, pz, Q[u].x, Q[u].y, Q[u].z, h2, dz, hin, vin);
+                        hit = hit || (hin && vin);
+                    }
+                }
+            }
+            if (last) break;
         }
         if (hit) first = i;
     }
