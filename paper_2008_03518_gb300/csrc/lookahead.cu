@@ -9,7 +9,7 @@
 //                sample at t + j, velocity from t + j to t + j + 1) - hard-deck penalty;
 //   Q(a) = max over j with x_j inside the box; a is valid when x_1 is inside.
 //
-// One CTA per request, 256 threads. A step is a chain of four short phases with a barrier after
+// One CTA per request, 256 or 512 threads. A step is a chain of four short phases with a barrier after
 // each; no unit is busy, so what counts is the length of each phase's instruction stream:
 //   1. side by side: the projected states per (action, sub-step) with box test, goal terms as a
 //      log2 offset from the goal term at s (from the exact identity d - d_s =
@@ -24,8 +24,8 @@
 //   4. one warp: the best value per action, argmax (lowest index on ties), near-tie record,
 //      exact FP64 advance, terminal tests.
 // On GB300: 60 plans and W = 10, 8.1 us per step with every pair scored by the warp that found
-// it and seven barriers, 6.4 us now; a co-simulation of 128 aircraft among 3000 plans, 23 us per
-// step with every slot read and a grid barrier, 7.2 us now.
+// it and seven barriers, 5.3 us now; a co-simulation of 128 aircraft among 3000 plans, 23 us per
+// step with every slot read and a grid barrier, 6.6 us now.
 // Every decision that is a threshold (box, well radius, clearance, capture) is taken in
 // FP64 with the oracle's operation order wherever fp32 could be on the wrong side.
 #include <climits>
@@ -38,7 +38,6 @@ namespace fmdp {
 
 namespace {
 
-constexpr int kLookThreads = 256;
 constexpr unsigned kFullMask = 0xffffffffu;
 
 constexpr int kLookList = 1024;  // samples the list of a step holds (more are scored where they are found)
@@ -81,8 +80,8 @@ __host__ __device__ inline LookLayout look_layout(int A, int W) {
     L.Dh = o; o += kHeadings * 4 * 4;     // the moves as double-float: xh, xl, yh, yl per heading
     L.Dz2 = o; o += kMaxActions * 2 * 4;  // climb as double-float
     al(16);
-    L.list = o; o += kLookList * sizeof(LookItem);
-    L.misc = o; o += 512;
+    L.list = o; o += kLookList * sizeof(LookItem);  // (then LookState, 16-byte aligned)
+    L.misc = o; o += 1024;
     L.total = (o + 127) & ~size_t(127);
     return L;
 }
@@ -100,15 +99,18 @@ struct LookState {
     int n0;                              // integer part of log2 of the goal term at s
     int h, k, done, status, near_ties;
     int tie_k, tie_a1, tie_a2;  // near-tie test of step tie_k still to do (tie_k < 0: none)
-    int tie_s1, tie_s2;
-    double tie_L1, tie_L2, tie_T1, tie_T2;
+    int tie_n0;
+    int tie_sg[kMaxActions];     // per action: sign class of Q (-1, 0, 1), -2 invalid
+    float tie_T[kMaxActions];    // ... log2 of the term scale max(g, N), relative to tie_n0
+    double tie_L[kMaxActions];   // ... log2 |Q|
     int64_t row0;     // ring row of t + 1 for the current step
     int n_list;       // samples found in this step (may exceed kLookList)
     int late;         // co-simulation: a wait for another aircraft's record expired
-    float well[kMaxWells][4];  // tau, R^2, log2 gamma, log2 |r|
+    alignas(16) float well[kMaxWells][4];  // tau, R^2, log2 gamma, log2 |r|
+    float band[kMaxWells];
     float reach[kMaxWells];    // R
 };
-static_assert(sizeof(LookState) <= 512, "see look_layout");
+static_assert(sizeof(LookState) <= 1024, "see look_layout");
 
 // Co-simulation: an aircraft's state at one step, as six 16-byte words {value, stamp}. The stamp
 // (2 x last step it holds for, + 1 when flying) is in every word and a word is read and written
@@ -317,65 +319,87 @@ __device__ __noinline__ bool look_near_tie(int s1, double L1, double T1, int s2,
 }
 
 // Scores one sample (the same in every lane) for every action (lanes) at its sub-step. hn, Dxy,
-// Dzf: the lane's heading after its turn and its move.
+// Dzf: the lane's heading after its turn and its move. Two wells at a time, without branches but
+// for the band: a sample with five wells took 1500 cycles well by well, most of them waiting for
+// one square root after the other.
 struct LookScore {
     const LookState* st;
     int* keys;
     unsigned long long* sums;
     const double *Dx, *Dy, *Dz;
 };
+// d < R for one well of a sample whose edge lies in the fp32 band
+__device__ __noinline__ bool look_band(const LookArgs& a, const LookScore& c, const LookItem& it, int w, int hn) {
+    const Model& m = a.m;
+    const LookState* st = c.st;
+    const int lane = threadIdx.x & 31, j = (it.what >> 16) & 0xff, kind = it.what >> 24;
+    bool in;
+    if (kind == kLookMember) {
+        const double* rc = a.mem + ((size_t)(st->step_no & 1) * a.n_req + it.ref) * 12;
+        double v[6];
+        for (int i = 0; i < 6; ++i) get_word(rc + 2 * i, v[i]);
+        in = look_member_exact(m, w, st->s, c.Dx[hn], c.Dy[hn], c.Dz[lane], j, v[0], v[1], v[2], v[3], v[4], v[5]);
+    } else {
+        int64_t r1 = st->row0 + j;
+        r1 -= r1 >= a.tab.T_win ? a.tab.T_win : 0;
+        float4 P1, P2;
+        if (kind == kLookIndex) {
+            const float4* p = a.iv.items + ((size_t)r1 * a.tab.S_pad + it.ref) * 2;
+            P1 = __ldcg(p);
+            P2 = __ldcg(p + 1);
+        } else {
+            const size_t o1 = (size_t)r1 * a.tab.S_pad + it.ref;
+            P1 = make_float4(a.tab.X[o1], a.tab.Y[o1], a.tab.Z[o1], 0.f);
+            P2 = make_float4(__int_as_float(0x7fc00000), 0.f, 0.f, 0.f);
+            if (st->t + j + 2 < a.tab.t_base + a.tab.T_win) {
+                const int64_t r2 = r1 + 1 >= a.tab.T_win ? 0 : r1 + 1;
+                const size_t o2 = (size_t)r2 * a.tab.S_pad + it.ref;
+                P2 = make_float4(a.tab.X[o2], a.tab.Y[o2], a.tab.Z[o2], 0.f);
+            }
+        }
+        in = look_well_exact(m, w, st->s, c.Dx[hn], c.Dy[hn], c.Dz[lane], j, P1.x, P1.y, P1.z, P2.x, P2.y, P2.z,
+                             P2.x == P2.x);
+    }
+    return in;
+}
 __device__ __forceinline__ void look_score(const LookArgs& a, const LookScore& c, const LookItem& it, int hn, float4 Dxy,
                                            float2 Dzf) {
     const Model& m = a.m;
-    const LookState* st = c.st;
     const int lane = threadIdx.x & 31;
     if (lane >= m.A) return;
-    const unsigned wells = (unsigned)it.what & 0xffffu;
-    const int j = (it.what >> 16) & 0xff, kind = it.what >> 24;
+    const int j = (it.what >> 16) & 0xff;
     const float fj = (float)(j + 1);
     const float px = fmaf(fj, Dxy.x, fj * Dxy.y), py = fmaf(fj, Dxy.z, fj * Dxy.w), pz = fmaf(fj, Dzf.x, fj * Dzf.y);
     float mb = -INFINITY;
     unsigned long long sb = 0ull;
-    for (unsigned left = wells; left; left &= left - 1u) {
-        const int w = __ffs(left) - 1;
-        const float tau = st->well[w][0];
-        const float ux = px - fmaf(tau, it.vx, it.qx), uy = py - fmaf(tau, it.vy, it.qy), uz = pz - fmaf(tau, it.vz, it.qz);
+    unsigned bands = 0u;
+    auto one = [&](int w, bool on) {
+        const float4 k = *reinterpret_cast<const float4*>(c.st->well[w]);
+        const float ux = px - fmaf(k.x, it.vx, it.qx), uy = py - fmaf(k.x, it.vy, it.qy), uz = pz - fmaf(k.x, it.vz, it.qz);
         const float d2 = fmaf(ux, ux, fmaf(uy, uy, uz * uz));
-        const float R2 = st->well[w][1];
-        bool in = d2 < R2;
-        if (fabsf(d2 - R2) <= m.w_band[w]) {
-            if (kind == kLookMember) {
-                const double* rc = a.mem + ((size_t)(st->step_no & 1) * a.n_req + it.ref) * 12;
-                double v[6];
-                for (int i = 0; i < 6; ++i) get_word(rc + 2 * i, v[i]);
-                in = look_member_exact(m, w, st->s, c.Dx[hn], c.Dy[hn], c.Dz[lane], j, v[0], v[1], v[2], v[3], v[4], v[5]);
-            } else {
-                int64_t r1 = st->row0 + j;
-                r1 -= r1 >= a.tab.T_win ? a.tab.T_win : 0;
-                float4 P1, P2;
-                if (kind == kLookIndex) {
-                    const float4* p = a.iv.items + ((size_t)r1 * a.tab.S_pad + it.ref) * 2;
-                    P1 = __ldcg(p);
-                    P2 = __ldcg(p + 1);
-                } else {
-                    const size_t o1 = (size_t)r1 * a.tab.S_pad + it.ref;
-                    P1 = make_float4(a.tab.X[o1], a.tab.Y[o1], a.tab.Z[o1], 0.f);
-                    P2 = make_float4(__int_as_float(0x7fc00000), 0.f, 0.f, 0.f);
-                    if (st->t + j + 2 < a.tab.t_base + a.tab.T_win) {
-                        const int64_t r2 = r1 + 1 >= a.tab.T_win ? 0 : r1 + 1;
-                        const size_t o2 = (size_t)r2 * a.tab.S_pad + it.ref;
-                        P2 = make_float4(a.tab.X[o2], a.tab.Y[o2], a.tab.Z[o2], 0.f);
-                    }
-                }
-                in = look_well_exact(m, w, st->s, c.Dx[hn], c.Dy[hn], c.Dz[lane], j, P1.x, P1.y, P1.z, P2.x, P2.y, P2.z,
-                                     P2.x == P2.x);
-            }
-        }
-        if (in) {
-            const float l = fmaf(sqrtf(d2), st->well[w][2], st->well[w][3]);
-            mb = fmaxf(mb, l);
-            if (m.combine) sb += look_sum_term(l, m.sum_ref);
-        }
+        const bool band = fabsf(d2 - k.y) <= c.st->band[w];
+        const bool in = on && !band && d2 < k.y;
+        const float l = fmaf(sqrtf(d2), k.z, k.w);
+        mb = fmaxf(mb, in ? l : -INFINITY);
+        if (m.combine && in) sb += look_sum_term(l, m.sum_ref);
+        bands |= on && band ? 1u << w : 0u;
+    };
+    for (unsigned left = (unsigned)it.what & 0xffffu; left;) {
+        const int w0 = __ffs(left) - 1;
+        left &= left - 1u;
+        const int w1 = left ? __ffs(left) - 1 : w0;
+        one(w0, true);
+        one(w1, left != 0u);
+        left &= left - 1u;
+    }
+    for (; bands; bands &= bands - 1u) {  // (rare)
+        const int w = __ffs(bands) - 1;
+        if (!look_band(a, c, it, w, hn)) continue;
+        const float4 k = *reinterpret_cast<const float4*>(c.st->well[w]);
+        const float ux = px - fmaf(k.x, it.vx, it.qx), uy = py - fmaf(k.x, it.vy, it.qy), uz = pz - fmaf(k.x, it.vz, it.qz);
+        const float l = fmaf(sqrtf(fmaf(ux, ux, fmaf(uy, uy, uz * uz))), k.z, k.w);
+        mb = fmaxf(mb, l);
+        if (m.combine) sb += look_sum_term(l, m.sum_ref);
     }
     const int q = lane * a.W + j;
     if (mb > -INFINITY) atomicMax(&c.keys[q], float_key(mb));
@@ -390,7 +414,10 @@ __device__ __noinline__ void look_score_over(const LookArgs& a, const LookScore&
 
 size_t lookahead_smem_bytes(int A, int W) { return look_layout(A, W).total; }
 
-__global__ void __launch_bounds__(kLookThreads, 2) lookahead_kernel(const __grid_constant__ LookArgs a) {
+// NT 512: sixteen warps share out a step's samples and its projected states, one CTA per SM; 256 (for
+// co-simulations, which all have to be resident): two CTAs per SM.
+template <int NT>
+__global__ void __launch_bounds__(NT, 512 / NT) lookahead_kernel(const __grid_constant__ LookArgs a) {
     extern __shared__ __align__(128) unsigned char lsm[];
     const Model& m = a.m;
     const int A = m.A, W = a.W, AW = A * W;
@@ -433,7 +460,9 @@ __global__ void __launch_bounds__(kLookThreads, 2) lookahead_kernel(const __grid
         if (st->tie_k < 0) return;
         bool tie = false;
         if (st->tie_a1 >= 0 && st->tie_a2 >= 0)
-            tie = look_near_tie(st->tie_s1, st->tie_L1, st->tie_T1, st->tie_s2, st->tie_L2, st->tie_T2);
+            tie = look_near_tie(st->tie_sg[st->tie_a1], st->tie_L[st->tie_a1],
+                                __dadd_rn((double)st->tie_n0, (double)st->tie_T[st->tie_a1]), st->tie_sg[st->tie_a2],
+                                st->tie_L[st->tie_a2], __dadd_rn((double)st->tie_n0, (double)st->tie_T[st->tie_a2]));
         if (a.trace) tie_trace[st->tie_k] = tie ? 1 : 0;
         st->near_ties += tie ? 1 : 0;
         st->tie_k = -1;
@@ -521,9 +550,10 @@ __global__ void __launch_bounds__(kLookThreads, 2) lookahead_kernel(const __grid
         st->well[tid][1] = m.w_R2[tid];
         st->well[tid][2] = m.w_lg[tid];
         st->well[tid][3] = m.w_L[tid];
+        st->band[tid] = m.w_band[tid];
         st->reach[tid] = sqrtf(m.w_R2[tid]);
     }
-    for (int q = tid; q < AW; q += kLookThreads) {
+    for (int q = tid; q < AW; q += NT) {
         keys[q] = KEY_NONE;
         sums[q] = 0ull;
     }
@@ -547,6 +577,9 @@ __global__ void __launch_bounds__(kLookThreads, 2) lookahead_kernel(const __grid
         return msk;
     };
 
+    // the (sub-step, slot) pairs of this warp's first turn, and from one turn to the next
+    const int pair_j = S > 0 ? warp * 32 / S : 0, pair_i = warp * 32 - pair_j * S;
+    const int turn_j = S > 0 ? NT / S : 0, turn_i = NT - turn_j * S;
     const bool act = lane < A;
     const DeckGrid grid = m.hm ? deck_grid(m) : DeckGrid{};
     const LookScore sc{st, keys, sums, Dx, Dy, Dz};
@@ -563,7 +596,7 @@ __global__ void __launch_bounds__(kLookThreads, 2) lookahead_kernel(const __grid
     auto wait_all = [&](int64_t step) {  // every thread; false when a record did not come
         bool ok = true;
         LookRecord rec;
-        for (int q = tid; q < n_wait; q += kLookThreads) {
+        for (int q = tid; q < n_wait; q += NT) {
             if (q == r) continue;
             // (the absent aircraft of the self-test: a record that nobody writes)
             ok = look_read(q < n_mem ? record_of(step, q) : a.mem + (size_t)2 * n_mem * 12, step, rec, true) && ok;
@@ -591,7 +624,8 @@ __global__ void __launch_bounds__(kLookThreads, 2) lookahead_kernel(const __grid
         const int64_t t = req.depart_step + k;
         const int64_t row0 = st->row0;  // ring row of t + 1
         // ---- 1. projected states and samples within reach, side by side
-        if (tid == kLookThreads - 1) {
+        if (tid == NT - 64) deferred_tie();  // the previous step's near-tie flag (FP64: 1900 cycles, off the chain here)
+        if (tid == NT - 1) {
             int n0;
             float phi;
             lk_goal_log(m, st->Ghx, st->Ghy, st->Ghz, st->Glx, st->Gly, st->Glz, n0, phi);
@@ -601,7 +635,7 @@ __global__ void __launch_bounds__(kLookThreads, 2) lookahead_kernel(const __grid
             st->t = t;
         }
         if (m.n_static > 0) {
-            for (int w = tid; w < m.n_static; w += kLookThreads) {
+            for (int w = tid; w < m.n_static; w += NT) {
                 const double* c = m.statics + 6 * w;
                 stc[3 * w] = (float)__dsub_rn(c[0], st->s[0]);
                 stc[3 * w + 1] = (float)__dsub_rn(c[1], st->s[1]);
@@ -618,7 +652,7 @@ __global__ void __launch_bounds__(kLookThreads, 2) lookahead_kernel(const __grid
         const float shx = st->shx, shy = st->shy, shz = st->shz, slx = st->slx, sly = st->sly, slz = st->slz;
         const float Gx = st->Ghx + st->Glx, Gy = st->Ghy + st->Gly, Gz = st->Ghz + st->Glz;
         // fp32 offsets (j + 1) * move, box test, goal-term offset, static wells
-        for (int q = tid; q < AW; q += kLookThreads) {
+        for (int q = tid; q < AW; q += NT) {
             const int ac = q / W, j = q - ac * W;
             const int hn = turned(ac);
             const float fj = (float)(j + 1);
@@ -707,7 +741,7 @@ __global__ void __launch_bounds__(kLookThreads, 2) lookahead_kernel(const __grid
             // one warp per sub-step (the last warps first: the first ones have the projected
             // states): the cells within reach, as in the one-step rollout, and the extra list
             const IndexView& iv = a.iv;
-            for (int j = kLookThreads / 32 - 1 - warp; j < W; j += kLookThreads / 32) {
+            for (int j = NT / 32 - 1 - warp; j < W; j += NT / 32) {
                 const int64_t t1 = t + j + 1;
                 if (t1 < a.tab.t_base || t1 >= t_hi) continue;
                 int64_t r1 = row0 + j;
@@ -761,36 +795,40 @@ __global__ void __launch_bounds__(kLookThreads, 2) lookahead_kernel(const __grid
                 }
             }
         } else {
-            // every (sub-step, slot) pair, two per thread and turn: their loads are in flight together
+            // every (sub-step, slot) pair, U per thread and turn: their loads are in flight together
+            // (S is a multiple of 32, so a warp's slots lie in one slice)
+            constexpr int U = 3;
             const int npairs = W * S;
-            for (int base = warp * 32; base < npairs; base += 2 * kLookThreads) {
-                float4 P1[2], P2[2];
-                int js[2];
+            int j0 = pair_j, i0 = pair_i;
+            const int j_lo = (int)max(a.tab.t_base - t - 1, (int64_t)0), j_hi = (int)min(t_hi - t - 1, (int64_t)W);
+            const int row_i = (int)row0, T_win = a.tab.T_win;
+            for (int base = warp * 32; base < npairs; base += U * NT) {
+                float4 P1[U], P2[U];
+                int js[U], is[U];
 #pragma unroll
-                for (int u = 0; u < 2; ++u) {
-                    const int idx = base + u * kLookThreads + lane;
+                for (int u = 0; u < U; ++u) {
+                    js[u] = j0, is[u] = i0 + lane;
+                    j0 += turn_j, i0 += turn_i;
+                    if (i0 >= S) i0 -= S, ++j0;
                     P1[u] = P2[u] = make_float4(__int_as_float(0x7fc00000), 0.f, 0.f, 0.f);
-                    js[u] = idx / S;
-                    const int64_t t1 = t + js[u] + 1;
-                    if (idx < npairs && t1 >= a.tab.t_base && t1 < t_hi) {
-                        const int i = idx - js[u] * S;
-                        int64_t r1 = row0 + js[u];  // rows of t + j + 1 and t + j + 2 (j < T_win)
-                        r1 -= r1 >= a.tab.T_win ? a.tab.T_win : 0;
-                        const size_t o1 = (size_t)r1 * a.tab.S_pad + i;
+                    if (base + u * NT < npairs && js[u] >= j_lo && js[u] < j_hi) {
+                        int r1 = row_i + js[u];  // rows of t + j + 1 and t + j + 2 (j < T_win)
+                        r1 -= r1 >= T_win ? T_win : 0;
+                        const size_t o1 = (size_t)r1 * a.tab.S_pad + is[u];
                         P1[u] = make_float4(a.tab.X[o1], a.tab.Y[o1], a.tab.Z[o1], 0.f);
-                        if (t1 + 1 < t_hi) {
-                            const size_t o2 = (size_t)(r1 + 1 >= a.tab.T_win ? 0 : r1 + 1) * a.tab.S_pad + i;
+                        if (t + js[u] + 2 < t_hi) {
+                            const size_t o2 = (size_t)(r1 + 1 >= T_win ? 0 : r1 + 1) * a.tab.S_pad + is[u];
                             P2[u] = make_float4(a.tab.X[o2], a.tab.Y[o2], a.tab.Z[o2], 0.f);
                         }
                     }
                 }
 #pragma unroll
-                for (int u = 0; u < 2; ++u) {
-                    if (base + u * kLookThreads >= npairs) break;  // (the same in the whole warp)
+                for (int u = 0; u < U; ++u) {
+                    if (base + u * NT >= npairs) break;  // (the same in the whole warp)
                     LookItem it{};
                     bool have = P1[u].x == P1[u].x;
                     if (have) {
-                        it = plan_item(P1[u], P2[u], js[u], kLookSlot, base + u * kLookThreads + lane - js[u] * S);
+                        it = plan_item(P1[u], P2[u], js[u], kLookSlot, is[u]);
                         have = (it.what & 0xffff) != 0;
                     }
                     add(it, have);
@@ -799,7 +837,7 @@ __global__ void __launch_bounds__(kLookThreads, 2) lookahead_kernel(const __grid
         }
         // co-simulation: the wells of every other aircraft in flight, at its position at t plus tau
         // times its last move (the same peaks for every sub-step)
-        for (int q0 = warp * 32; q0 < n_wait; q0 += kLookThreads) {
+        for (int q0 = warp * 32; q0 < n_wait; q0 += NT) {
             const int q = q0 + lane;
             LookRecord rec;
             rec.flying = false;
@@ -832,13 +870,12 @@ __global__ void __launch_bounds__(kLookThreads, 2) lookahead_kernel(const __grid
 
         // ---- 2. the list, shared out between the warps
         const int n_list = min(st->n_list, kLookList);
-        for (int e = warp; e < n_list; e += kLookThreads / 32) look_score(a, sc, list[e], hn_l, Dxy_l, Dzf_l);
+        for (int e = warp; e < n_list; e += NT / 32) look_score(a, sc, list[e], hn_l, Dxy_l, Dzf_l);
         __syncthreads();
 
         // ---- 3. penalty + deck per (action, sub-step), as log2
         if (tid == 0) st->n_list = 0;
-        if (tid == kLookThreads - 32) deferred_tie();  // the previous step's near-tie flag
-        for (int q = tid; q < AW; q += kLookThreads) {
+        for (int q = tid; q < AW; q += NT) {
             float P = 0.f;
             if (m.combine) {
                 if (sums[q]) P = (float)((double)sums[q] * m.sum_scale);
@@ -923,28 +960,32 @@ __global__ void __launch_bounds__(kLookThreads, 2) lookahead_kernel(const __grid
         // near-tie record, advance.
         if (warp == 0) {
             int sgl = -2;
-            double Lkl = 0.0, Lql = 0.0;
+            double Lkl = 0.0;
             unsigned long long kq = 0ull;
+            const int n0 = st->n0;
             if (act) {
                 const int q0 = lane * W;
-                float2 v[kMaxLookahead];
-#pragma unroll
-                for (int j = 0; j < kMaxLookahead; ++j) v[j] = cmp[q0 + (j < W ? j : 0)];
                 int bj = 0;
-                float2 b = v[0];
-#pragma unroll
-                for (int j = 1; j < kMaxLookahead; ++j) {
-                    const bool better = v[j].x > b.x || (v[j].x == b.x && v[j].y > b.y);  // (j >= W: v[0], never)
+                float2 b = cmp[q0];
+#pragma unroll 4
+                for (int j = 1; j < W; ++j) {
+                    const float2 v = cmp[q0 + j];
+                    const bool better = v.x > b.x || (v.x == b.x && v.y > b.y);
                     bj = better ? j : bj;
-                    b = better ? v[j] : b;
+                    b = better ? v : b;
                 }
-                const int bq = q0 + bj;
-                const bool valid = inb[q0] != 0;
-                const int sg = (vsg[bq] & 3) - 1;
-                Lkl = (vsg[bq] & 4) ? (double)vlv[bq] : __dadd_rn((double)st->n0, (double)vlv[bq]);
-                Lql = __dadd_rn((double)st->n0, (double)vls[bq]);
-                sgl = valid ? sg : -2;
-                kq = valid ? look_key(sg, Lkl) : 0ull;
+                const int bq = q0 + bj, code = vsg[bq];
+                const float lv = vlv[bq];
+                const int sg = (code & 3) - 1;
+                Lkl = (code & 4) ? (double)lv : __dadd_rn((double)n0, (double)lv);
+                if (inb[q0]) {
+                    sgl = sg;
+                    kq = look_key(sg, Lkl);
+                }
+                // for the near-tie flag, during the next step
+                st->tie_sg[lane] = sgl;
+                st->tie_L[lane] = Lkl;
+                st->tie_T[lane] = vls[bq];
             }
             // the largest of the lanes' 64-bit keys, by halves
             auto largest = [&](unsigned long long v) {
@@ -960,55 +1001,36 @@ __global__ void __launch_bounds__(kLookThreads, 2) lookahead_kernel(const __grid
             const int a2 = b2 ? __ffs(b2) - 1 : -1;
             if (a.trace && lane < A)
                 q_trace[(size_t)k * A + lane] = sgl == -2 ? -INFINITY : (sgl == 0 ? 0.0 : (double)sgl * exp2(Lkl));
-            const int c1 = max(a1, 0), c2 = max(a2, 0);
-            const int s1 = __shfl_sync(kFullMask, sgl, c1), s2 = __shfl_sync(kFullMask, sgl, c2);
-            const double L1 = __shfl_sync(kFullMask, Lkl, c1), L2 = __shfl_sync(kFullMask, Lkl, c2);
-            const double T1 = __shfl_sync(kFullMask, Lql, c1), T2 = __shfl_sync(kFullMask, Lql, c2);
-            if (lane == 0) {
-                st->tie_k = k;  // tested during the next step (deferred_tie)
-                st->tie_a1 = a1;
-                st->tie_a2 = a2;
-                if (a1 >= 0 && a2 >= 0) {
-                    st->tie_s1 = s1;
-                    st->tie_s2 = s2;
-                    st->tie_L1 = L1;
-                    st->tie_L2 = L2;
-                    st->tie_T1 = T1;
-                    st->tie_T2 = T2;
-                }
-                if (a1 < 0) {
+            if (a1 < 0) {
+                if (lane == 0) {
                     st->status = FMDP_REJ_NO_ACTION;
                     st->done = 1;
-                } else {
-                    const int hn = turned(a1);
-                    // exact advance (FP64, the oracle's x_1) and its double-float copies
-                    st->prev[0] = st->s[0];
-                    st->prev[1] = st->s[1];
-                    st->prev[2] = st->s[2];
-                    st->s[0] = __dadd_rn(st->s[0], Dx[hn]);
-                    st->s[1] = __dadd_rn(st->s[1], Dy[hn]);
-                    st->s[2] = __dadd_rn(st->s[2], Dz[a1]);
-                    lk_df_add(st->shx, st->slx, Dh[4 * hn], Dh[4 * hn + 1]);
-                    lk_df_add(st->shy, st->sly, Dh[4 * hn + 2], Dh[4 * hn + 3]);
-                    lk_df_add(st->shz, st->slz, Dz2[2 * a1], Dz2[2 * a1 + 1]);
-                    lk_df_add(st->Ghx, st->Glx, -Dh[4 * hn], -Dh[4 * hn + 1]);
-                    lk_df_add(st->Ghy, st->Gly, -Dh[4 * hn + 2], -Dh[4 * hn + 3]);
-                    lk_df_add(st->Ghz, st->Glz, -Dz2[2 * a1], -Dz2[2 * a1 + 1]);
+                }
+            } else {
+                // exact advance (FP64, the oracle's x_1) and its double-float copies: lanes 0 .. 2
+                // take x, y, z
+                const int hn = turned(a1), np = k + 1;
+                float G = 0.f;
+                if (lane < 3) {
+                    const float* Df = lane < 2 ? Dh + 4 * hn + 2 * lane : Dz2 + 2 * a1;
+                    const double D = (lane == 0 ? Dx : Dy)[hn], s0 = st->s[lane];
+                    const double s1 = __dadd_rn(s0, lane < 2 ? D : Dz[a1]);
+                    lk_df_add((&st->shx)[lane], (&st->slx)[lane], Df[0], Df[1]);
+                    lk_df_add((&st->Ghx)[lane], (&st->Glx)[lane], -Df[0], -Df[1]);
+                    G = (&st->Ghx)[lane] + (&st->Glx)[lane];
+                    st->prev[lane] = s0;
+                    st->s[lane] = s1;
+                    traj[3 * np + lane] = (float)s1;
+                    if (a.trace) st_trace[3 * np + lane] = s1;
+                }
+                const float gx = __shfl_sync(kFullMask, G, 0), gy = __shfl_sync(kFullMask, G, 1), gz = __shfl_sync(kFullMask, G, 2);
+                __syncwarp();
+                if (lane == 0) {
                     st->h = hn;
                     acts[k] = (uint8_t)a1;
-                    const int np = k + 1;
-                    traj[3 * np] = (float)st->s[0];
-                    traj[3 * np + 1] = (float)st->s[1];
-                    traj[3 * np + 2] = (float)st->s[2];
-                    if (a.trace) {
-                        st_trace[3 * np] = st->s[0];
-                        st_trace[3 * np + 1] = st->s[1];
-                        st_trace[3 * np + 2] = st->s[2];
-                        hd_trace[np] = hn;
-                    }
+                    if (a.trace) hd_trace[np] = hn;
                     st->k = np;
-                    st->row0 = st->row0 + 1 == a.tab.T_win ? 0 : st->row0 + 1;
-                    const float gx = st->Ghx + st->Glx, gy = st->Ghy + st->Gly, gz = st->Ghz + st->Glz;
+                    st->row0 = row0 + 1 == a.tab.T_win ? 0 : row0 + 1;
                     const float gd = sqrtf(gx * gx + gy * gy + gz * gz);
                     bool cap = false;
                     if (gd < stepf + kCapBandL) cap = look_capture_exact(st->s, req, st->cap2);
@@ -1020,6 +1042,12 @@ __global__ void __launch_bounds__(kLookThreads, 2) lookahead_kernel(const __grid
                         st->done = 1;
                     }
                 }
+            }
+            if (lane == 0) {
+                st->tie_k = k;  // tested during the next step (deferred_tie)
+                st->tie_a1 = a1;
+                st->tie_a2 = a2;
+                st->tie_n0 = n0;
             }
         }
         __syncthreads();
@@ -1044,14 +1072,16 @@ __global__ void __launch_bounds__(kLookThreads, 2) lookahead_kernel(const __grid
 }
 
 cudaError_t prepare_lookahead_kernel() {
-    return cudaFuncSetAttribute(lookahead_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)look_layout(kMaxActions, kMaxLookahead).total);
+    const int smem = (int)look_layout(kMaxActions, kMaxLookahead).total;
+    const cudaError_t e = cudaFuncSetAttribute(lookahead_kernel<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    return e != cudaSuccess ? e
+                            : cudaFuncSetAttribute(lookahead_kernel<512>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
 }
 
 int lookahead_max_resident(int A, int W) {
     int per_sm = 0, dev = 0, n_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, lookahead_kernel, kLookThreads,
-                                                      look_layout(A, W).total) != cudaSuccess ||
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, lookahead_kernel<256>, 256, look_layout(A, W).total) !=
+            cudaSuccess ||
         cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
         cudaGetLastError();
@@ -1062,22 +1092,25 @@ int lookahead_max_resident(int A, int W) {
 
 cudaError_t launch_lookahead(const LookArgs& a, cudaStream_t s) {
     if (a.n_req <= 0) return cudaSuccess;
+    const size_t smem = look_layout(a.m.A, a.W).total;
     if (!a.cosim) {
-        lookahead_kernel<<<a.n_req, kLookThreads, look_layout(a.m.A, a.W).total, s>>>(a);
+        // also with more requests than SMs: 256 requests at W = 10, 450 ms of rollouts in waves, 610
+        // with 256 threads and two CTAs per SM (most waves are the last few requests' re-plans)
+        lookahead_kernel<512><<<a.n_req, 512, smem, s>>>(a);
         return cudaGetLastError();
     }
-    // co-simulation: every CTA must be resident at once (they wait for one another)
+    // co-simulation: every CTA must be resident at once (they wait for one another), two per SM
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)a.n_req, 1, 1);
-    cfg.blockDim = dim3(kLookThreads, 1, 1);
-    cfg.dynamicSmemBytes = look_layout(a.m.A, a.W).total;
+    cfg.blockDim = dim3(256, 1, 1);
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeCooperative;
     attr[0].val.cooperative = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, lookahead_kernel, a);
+    return cudaLaunchKernelEx(&cfg, lookahead_kernel<256>, a);
 }
 
 }  // namespace fmdp
