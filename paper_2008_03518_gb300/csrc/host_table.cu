@@ -210,11 +210,13 @@ int32_t batch_size_of(const fmdp_ctx* c) { return c->opt.batch_size > 0 ? c->opt
 // lookahead window of the rollouts (Sec. IV "Forward project"); 1 is the one-step rule
 int32_t window_of(const fmdp_ctx* c) { return c->opt.lookahead_W > 1 ? c->opt.lookahead_W : 1; }
 
-// Lookahead rollouts read the plan samples within reach from the index once a slice has more
-// slots than a CTA has threads: up to there one load per thread covers a
-// slice (3136 slots: 30 000 cycles of a co-simulated step, 600 beside the other work by index).
+// Lookahead rollouts read the plan samples within reach from the index once the W slices of a step
+// have more than kLookScanPairs slots: up to there two loads per thread cover them and no index
+// row has to be looked up first. Per step, every slot against index: W = 2, 300 plans 4.5 and 5.0
+// us, 600 plans 5.15 and 5.14, 1200 plans 6.5 and 5.8; W = 10, 300 plans 8.4 and 5.8 us, 1200 plans
+// 19.5 and 8.0.
 void set_look_index(fmdp_ctx* c, LookArgs& la) {
-    if (!c->index_on || la.S_scan <= kLookScanSlots) return;
+    if (!c->index_on || (int64_t)window_of(c) * la.S_scan <= kLookScanPairs) return;
     la.by_index = 1;
     la.iv = index_view(c);
 }

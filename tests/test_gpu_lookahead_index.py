@@ -61,7 +61,7 @@ def test_more_samples_than_the_list_holds():
 @pytest.mark.parametrize("departures", ["together", "one by one", "after the others"])
 @pytest.mark.parametrize("window", [1, 3])
 def test_cosim_equals_every_slot(window, departures):
-    sc = scene(700, 24, spread=800.0)
+    sc = scene(1100, 24, spread=800.0)
     n = len(sc.requests)
     sc.requests["depart"] = {"together": np.full(n, 10), "one by one": 10 + 3 * np.arange(n)[::-1],
                              "after the others": 10 + 400 * (np.arange(n) % 2)}[departures]
