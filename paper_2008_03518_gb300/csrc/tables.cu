@@ -477,10 +477,13 @@ struct CellScan {
     }
 };
 
-// squared distance bound of a report in progress (other warps lower it), rounded up
+// Squared distance bound of a report in progress, rounded up (a warp together). Other warps lower
+// it meanwhile, and the cells of a square and the loops over them follow from it, so the lanes
+// take one value: two lanes with squares of their own would skip or double cell rows.
 __device__ __forceinline__ float known_bound2(const SepOut* out) {
+    __syncwarp();
     const float h = __uint_as_float(*(const volatile uint32_t*)&out->min_h_bits);
-    return h * h * 1.000001f;
+    return __shfl_sync(0xffffffffu, h * h * 1.000001f, 0);
 }
 
 // One trajectory: one warp per sample. After its samples' first squares a block publishes the
@@ -530,7 +533,7 @@ __global__ void __launch_bounds__(kCellThreads) sepcheck_cells_kernel(const __gr
     float bound2 = __uint_as_float(s_minh);
     __syncthreads();
     if (far * far < bound2) {  // (the same in every lane)
-        bound2 = fminf(bound2, __shfl_sync(0xffffffffu, known_bound2(out), 0));
+        bound2 = fminf(bound2, known_bound2(out));
         while (far < INFINITY && far * far < bound2) {
             far = S.wider_square(far, bound2);
             bound2 = fminf(bound2, S.least2());
@@ -667,7 +670,7 @@ __global__ void __launch_bounds__(kCellThreads) sepcheck_row_cells_kernel(const 
         float far = pfar[q];
         if (far == INFINITY) continue;
         SepOut* out = a.out + pr[q];
-        float bound2 = __shfl_sync(0xffffffffu, known_bound2(out), 0);
+        float bound2 = known_bound2(out);
         if (far * far >= bound2) continue;
         const float known2 = bound2;
         begin(q);
