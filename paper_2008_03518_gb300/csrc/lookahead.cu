@@ -94,8 +94,9 @@ struct LookState {
     float shx, shy, shz, slx, sly, slz;  // s as double-float
     float Ghx, Ghy, Ghz, Glx, Gly, Glz;  // goal - s as double-float
     float phi;                           // log2 g(s) - n0
-    int64_t step_no;                     // co-simulation: the step's number
-    int64_t t;                           // the step
+    // the step's number (co-simulation) and the step: written a barrier ahead of the step, because
+    // its first phase already scores samples (those the list cannot take)
+    int64_t step_no, t;
     int n0;                              // integer part of log2 of the goal term at s
     int h, k, done, status, near_ties;
     int tie_k, tie_a1, tie_a2;  // near-tie test of step tie_k still to do (tie_k < 0: none)
@@ -532,6 +533,8 @@ __global__ void __launch_bounds__(NT, 512 / NT) lookahead_kernel(const __grid_co
             gh[c] = (float)G;
             gl[c] = (float)__dsub_rn(G, (double)gh[c]);
         }
+        st->t = req.depart_step;
+        st->step_no = req.depart_step - a.t_start + 1;
         int64_t row = (req.depart_step + 1) % a.tab.T_win;
         st->row0 = row < 0 ? row + a.tab.T_win : row;
         if (a.trace) {
@@ -631,8 +634,6 @@ __global__ void __launch_bounds__(NT, 512 / NT) lookahead_kernel(const __grid_co
             lk_goal_log(m, st->Ghx, st->Ghy, st->Ghz, st->Glx, st->Gly, st->Glz, n0, phi);
             st->n0 = n0;
             st->phi = phi;
-            st->step_no = step_no;
-            st->t = t;
         }
         if (m.n_static > 0) {
             for (int w = tid; w < m.n_static; w += NT) {
@@ -1030,6 +1031,8 @@ __global__ void __launch_bounds__(NT, 512 / NT) lookahead_kernel(const __grid_co
                     acts[k] = (uint8_t)a1;
                     if (a.trace) hd_trace[np] = hn;
                     st->k = np;
+                    st->t = t + 1;
+                    st->step_no = step_no + 1;
                     st->row0 = row0 + 1 == a.tab.T_win ? 0 : row0 + 1;
                     const float gd = sqrtf(gx * gx + gy * gy + gz * gz);
                     bool cap = false;
