@@ -98,7 +98,8 @@ __device__ __forceinline__ float2 df_diff(float a, float b) {
 // cycles here. In double-float the clearance c is good to nanometres plus what the position
 // has drifted from the exact state (one rounding per step), so both the decision c < clearance
 // and the fp32 value of deck - c are those of FP64 unless one lies within that error of a
-// threshold: then, and only then, FP64 decides. Returns the penalty, or -1 for FP64 to decide.
+// threshold, or the position beside the cell t: then, and only then, FP64 decides. Returns the
+// penalty, or -1 for FP64 to decide. Compared with FP64 on the host in test_deck_band_cpu.py.
 static __device__ __noinline__ float deck_band(const Model& m, const DeckGrid g, const TerrainCell t, float hx, float lx, float hy,
                                         float ly, float hz, float lz, int k) {
     // position in the cell: offset from its node (b + i c), times the nodes per metre
@@ -109,6 +110,13 @@ static __device__ __noinline__ float deck_band(const Model& m, const DeckGrid g,
     };
     const float2 ax = frac(hx, lx, t.ix, g.bxh, g.bxl, g.cxh, g.cxl, g.sxh, g.sxl);
     const float2 ay = frac(hy, ly, t.iy, g.byh, g.byl, g.cyh, g.cyl, g.syh, g.syl);
+    // the cell comes from an fp32 position: within that rounding of a node line it may be the
+    // neighbour of the one FP64 takes, whose surface is another one (not on the grid's border,
+    // where FP64 goes on with the last cell too)
+    auto beside = [](float2 f, int i, int n) {
+        return (f.x < 0.f && i > 0) || ((f.x > 1.f || (f.x == 1.f && f.y > 0.f)) && i < n - 2);
+    };
+    if (beside(ax, t.ix, m.hm_nx) || beside(ay, t.iy, m.hm_ny)) return -1.f;
     const float2 lo = df_sum(make_float2(t.h00, 0.f), df_mul(ax, df_diff(t.h10, t.h00)));
     const float2 hi = df_sum(make_float2(t.h01, 0.f), df_mul(ax, df_diff(t.h11, t.h01)));
     const float2 T = df_sum(lo, df_mul(ay, df_sum(hi, make_float2(-lo.x, -lo.y))));
