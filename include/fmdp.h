@@ -280,7 +280,8 @@ fmdp_status fmdp_learned_init(fmdp_ctx* ctx, uint64_t seed);
 fmdp_status fmdp_learned_set_params(fmdp_ctx* ctx, const float* params, int32_t n);
 fmdp_status fmdp_learned_get_params(fmdp_ctx* ctx, float* params, int32_t n);
 /* Adam on the mean cross-entropy of the training set, shuffled with `seed` each epoch;
- * loss_per_epoch (optional, epochs floats): mean batch loss of each epoch. */
+ * loss_per_epoch (optional, epochs floats): mean batch loss of each epoch. FMDP_ERR_TIMEOUT when
+ * a bounded device wait expired; the parameters are those of the last step before it. */
 fmdp_status fmdp_learned_train(fmdp_ctx* ctx, int32_t epochs, int32_t batch, float lr, uint64_t seed,
                                float* loss_per_epoch);
 /* Loss and gradient on the given rows (host X [rows][128], bf16-rounded on the device; y),
@@ -350,6 +351,9 @@ fmdp_status fmdp_schedule_cosim(fmdp_ctx* ctx, const fmdp_request* reqs, int32_t
  * when that status was FMDP_ERR_TIMEOUT and nothing was admitted; the context stays
  * usable. Takes about one second. */
 fmdp_status fmdp_selftest_wait_timeout(fmdp_ctx* ctx, int32_t* observed);
+/* Sets the context's device error word, as a kernel whose wait expired does (no kernel runs): the
+ * next call that plans or trains reports FMDP_ERR_TIMEOUT, changes nothing and clears it. */
+fmdp_status fmdp_selftest_expired_wait(fmdp_ctx* ctx);
 
 /* ---- Autotuner of the batched rollout's launch shape (no counterpart in the paper; the
  * rollout is Alg. 1 whatever the shape, and results are bit-identical across shapes).

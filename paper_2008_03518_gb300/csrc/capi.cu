@@ -705,6 +705,15 @@ fmdp_status fmdp_selftest_wait_timeout(fmdp_ctx* c, int32_t* observed) {
     });
 }
 
+fmdp_status fmdp_selftest_expired_wait(fmdp_ctx* c) {
+    if (!c) return FMDP_ERR_ARG;
+    return guard(c, [&] {
+        const int32_t e = FMDP_ERR_TIMEOUT;
+        CK(cudaMemcpyAsync(c->err, &e, sizeof(e), cudaMemcpyHostToDevice, c->stream));
+        CK(cudaStreamSynchronize(c->stream));
+    });
+}
+
 fmdp_status fmdp_autotune(fmdp_ctx* c, const fmdp_request* sample, int32_t n, int32_t force,
                           fmdp_tune_report* report) {
     if (!c) return FMDP_ERR_ARG;

@@ -78,12 +78,12 @@ void mlp_train(fmdp_ctx* c, int32_t epochs, int32_t batch, float lr, uint64_t se
             LAUNCH(c, launch_gather_rows(c->tX.p, c->tr_idx.p + b0, Bn, c->trX.p, c->ty.p, c->tr_y.p, c->stream));
             mlp_fwd_bwd(c, nullptr, c->trX.p, c->tr_y.p, Bn);
             LAUNCH(c, launch_adam(c->mlp_p.p, c->mlp_g.p, c->mlp_m1.p, c->mlp_m2.p, n_params_total(), lr, 0.9f, 0.999f,
-                                  1e-8f, (int)++c->adam_t, c->stream));
+                                  1e-8f, (int)++c->adam_t, c->err, c->stream));
             LAUNCH(c, launch_export_weights(c->mlp_p.p, c->mlp_wp.p, c->stream));
         }
         float tot = 0.f;
         CK(cudaMemcpyAsync(&tot, c->tr_loss.p, sizeof(float), cudaMemcpyDeviceToHost, c->stream));
-        CK(cudaStreamSynchronize(c->stream));
+        require(read_error_word(c) == 0, FMDP_ERR_TIMEOUT, "a bounded device wait expired in the training");
         if (losses) losses[e] = nb ? tot / (float)nb : 0.f;
     }
     CK(cudaStreamSynchronize(c->stream));

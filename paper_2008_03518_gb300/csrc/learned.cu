@@ -93,8 +93,10 @@ cudaError_t launch_gather_rows(const __nv_bfloat16* X, const int32_t* idx, int M
     return cudaGetLastError();
 }
 
+// (no step on the gradient of a batch whose kernels gave up a wait: *err is set then)
 __global__ void adam_kernel(float* p, const float* g, float* m1, float* m2, size_t n, float lr, float b1, float b2,
-                            float eps, float c1, float c2) {
+                            float eps, float c1, float c2, const int32_t* err) {
+    if (*(volatile const int32_t*)err != 0) return;
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
         const float gi = g[i];
         const float a = b1 * m1[i] + (1.f - b1) * gi;
@@ -105,9 +107,9 @@ __global__ void adam_kernel(float* p, const float* g, float* m1, float* m2, size
     }
 }
 cudaError_t launch_adam(float* p, const float* g, float* m1, float* m2, size_t n, float lr, float b1, float b2,
-                        float eps, int t, cudaStream_t s) {
+                        float eps, int t, const int32_t* err, cudaStream_t s) {
     const float c1 = 1.f - powf(b1, (float)t), c2 = 1.f - powf(b2, (float)t);
-    adam_kernel<<<592, 256, 0, s>>>(p, g, m1, m2, n, lr, b1, b2, eps, c1, c2);
+    adam_kernel<<<592, 256, 0, s>>>(p, g, m1, m2, n, lr, b1, b2, eps, c1, c2, err);
     return cudaGetLastError();
 }
 

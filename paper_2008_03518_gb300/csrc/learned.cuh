@@ -317,9 +317,10 @@ cudaError_t prepare_train_kernels();
 cudaError_t launch_train(const TrainArgs& a, cudaStream_t s);
 cudaError_t launch_gather_rows(const __nv_bfloat16* X, const int32_t* idx, int M, __nv_bfloat16* out,
                                const uint8_t* y, uint8_t* y_out, cudaStream_t s);
-// Adam on the fp32 master parameters, then the bf16 copy in the chunk layout
+// Adam on the fp32 master parameters (nothing once *err is set), then the bf16 copy in the chunk
+// layout
 cudaError_t launch_adam(float* p, const float* g, float* m1, float* m2, size_t n, float lr, float b1, float b2,
-                        float eps, int t, cudaStream_t s);
+                        float eps, int t, const int32_t* err, cudaStream_t s);
 cudaError_t launch_export_weights(const float* p, __nv_bfloat16* Wp, cudaStream_t s);
 
 // Policy rollouts: a cluster of CTAs carries up to kPolicyRows requests in lock step (one

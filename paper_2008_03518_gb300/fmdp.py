@@ -176,7 +176,7 @@ EXPORTS = ("fmdp_options_default", "fmdp_create", "fmdp_destroy", "fmdp_last_err
            "fmdp_learned_evaluate", "fmdp_schedule_learned",
            "fmdp_autotune", "fmdp_tune_cache_get", "fmdp_tune_cache_put", "fmdp_schedule_departures",
            "fmdp_schedule_departures_batch",
-           "fmdp_schedule_cosim", "fmdp_selftest_wait_timeout",
+           "fmdp_schedule_cosim", "fmdp_selftest_wait_timeout", "fmdp_selftest_expired_wait",
            "fmdp_get_plan", "fmdp_save_plans", "fmdp_load_plans", "fmdp_expire", "fmdp_snapshot", "fmdp_restore", "fmdp_clear", "fmdp_rollout_trace",
            "fmdp_sep_check", "fmdp_sep_check_noalloc", "fmdp_set_profiling", "fmdp_get_stats",
            "fmdp_set_batch_mode", "fmdp_last_call_times", "fmdp_probe_peaks")
@@ -231,6 +231,7 @@ def load(build_if_missing: bool = True):
     L.fmdp_autotune.argtypes = [vp, P(Request), c.c_int32, c.c_int32, P(TuneReport)]
     L.fmdp_schedule_cosim.argtypes = [vp, P(Request), c.c_int32, P(Result)]
     L.fmdp_selftest_wait_timeout.argtypes = [vp, P(c.c_int32)]
+    L.fmdp_selftest_expired_wait.argtypes = [vp]
     L.fmdp_schedule_departures.argtypes = [vp, P(Request), c.c_int32, P(c.c_int64), c.c_int32, P(Result),
                                            P(c.c_int32), P(c.c_int32)]
     L.fmdp_schedule_departures_batch.argtypes = L.fmdp_schedule_departures.argtypes
@@ -653,6 +654,10 @@ class Scheduler:
         st = ctypes.c_int32(0)
         self._check(self._L.fmdp_selftest_wait_timeout(self._h, ctypes.byref(st)))
         return st.value
+
+    def selftest_expired_wait(self):
+        """Leaves the device error word set, as an expired wait does."""
+        self._check(self._L.fmdp_selftest_expired_wait(self._h))
 
     def schedule_cosim(self, reqs, points=True):
         """The batch co-simulated on one clock (each request sees the others' wells), then
