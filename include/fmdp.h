@@ -352,7 +352,8 @@ fmdp_status fmdp_schedule_cosim(fmdp_ctx* ctx, const fmdp_request* reqs, int32_t
  * usable. Takes about one second. */
 fmdp_status fmdp_selftest_wait_timeout(fmdp_ctx* ctx, int32_t* observed);
 /* Sets the context's device error word, as a kernel whose wait expired does (no kernel runs): the
- * next call that plans or trains reports FMDP_ERR_TIMEOUT, changes nothing and clears it. */
+ * next call that plans or trains reports FMDP_ERR_TIMEOUT, changes nothing and clears it. Known
+ * plans are stored all the same. */
 fmdp_status fmdp_selftest_expired_wait(fmdp_ctx* ctx);
 
 /* ---- Autotuner of the batched rollout's launch shape (no counterpart in the paper; the

@@ -221,7 +221,7 @@ struct AdmitArgs {
     const int64_t* offs;   // force mode: per plan offset into traj (points)
     const int32_t* idx;    // request index of work item y (nullptr: identity)
     const int32_t* n_dev;  // number of work items on the device (nullptr: all launched)
-    const int32_t* err;    // device error word: nothing is stored once a wait has expired
+    const int32_t* err;    // device error word: nothing is stored once a wait has expired (or nullptr)
     int32_t* slot_ord;     // if set: slot_ord[slot] = ord for an admitted trajectory
     int32_t ord;           // FCFS ordinal of the admitted request (see SepRowsArgs)
 };

@@ -556,7 +556,7 @@ void store_plans(fmdp_ctx* c, int32_t n_plans, const int64_t* t0s, const int32_t
         CK(cudaMemcpyAsync(c->counts.p, counts, n_plans * sizeof(int32_t), cudaMemcpyHostToDevice, c->stream));
         CK(cudaMemcpyAsync(c->slots.p, sl.data(), n_plans * sizeof(int32_t), cudaMemcpyHostToDevice, c->stream));
         AdmitArgs aa{};
-        aa.err = c->err;
+        aa.err = nullptr;  // (a known plan does not come from a rollout: no wait before it can have expired)
         aa.tab = table_view(c);
         aa.cap = 0;
         aa.traj = c->traj.p;
