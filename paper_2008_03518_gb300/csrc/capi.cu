@@ -104,7 +104,7 @@ fmdp_status fmdp_create(const fmdp_airspace* air, double gamma, const fmdp_actio
         CK(preload_index_kernels());
         CK(preload_table_kernels());
         CK(prepare_sepcheck_rows(sepcheck_rows_smem(kBatchMax)));
-        CK(prepare_policy_kernel());
+        CK(prepare_policy_kernels());
         CK(prepare_train_kernels());
         CK(prepare_lookahead_kernel());
 

@@ -104,11 +104,11 @@ void enqueue_wave(fmdp_ctx* c, const Geometry& g, int n_clusters, BatchBuffers& 
         pa.traj = c->p_traj.p;
         pa.acts = c->p_acts.p;
         pa.out = c->p_rout.p;
-            pa.rows = policy_rows_for(n_cap, c->n_sm);
+        pa.err = c->err;
         pa.step_bound = 1;  // learned FCFS: proposals beyond the judge's bound are never taken
         pa.slack = c->slack;
         pa.climb_step = climb_step(c);
-        LAUNCH(c, launch_policy(pa, policy_ctas_for(n_cap, pa.rows, c->n_sm), s));
+        LAUNCH(c, launch_policy(pa, n_cap, c->n_sm, s));
         SepRowsArgs sp{};
         sp.m = c->model;
         sp.tab = tv;

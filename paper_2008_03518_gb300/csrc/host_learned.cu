@@ -169,9 +169,9 @@ void learned_evaluate(fmdp_ctx* c, const fmdp_request* reqs, int32_t n, double s
     pa.traj = c->p_traj.p;
     pa.acts = c->p_acts.p;
     pa.out = c->p_rout.p;
-    pa.rows = policy_rows_for(n, c->n_sm);
+    pa.err = c->err;
     CK(cudaEventRecord(e[0], c->stream));
-    LAUNCH(c, launch_policy(pa, policy_ctas_for(n, pa.rows, c->n_sm), c->stream));
+    LAUNCH(c, launch_policy(pa, n, c->n_sm, c->stream));
     CK(cudaEventRecord(e[1], c->stream));
     // their separation checks and the judge (decisions only), in chunks of the row kernel's size
     LAUNCH(c, launch_sep_reset(c->p_sep.p, n, c->stream));

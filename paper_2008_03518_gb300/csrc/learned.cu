@@ -182,6 +182,12 @@ struct PolicyRow {
     int32_t req, k, h, status;  // req < 0: empty
 };
 
+struct PolicyTurns {  // the actions' moves
+    double cks[48];   // cos, sin of 15 degree steps (FP64)
+    double climb_dt[kMaxActions];
+    int dh[kMaxActions];
+};
+
 struct PolicySmem {
     __nv_bfloat16 w0[kPolicyCols * (kFeat + 8)];               // [column][input]
     __nv_bfloat16 w[kLayers - 2][kPolicyCols * kActPad];
@@ -191,10 +197,8 @@ struct PolicySmem {
     float feat[kPolicyThreads / 32][kFeat];
     unsigned long long skey[kPolicyThreads / 32][kSectors];
     PolicyRow rows[kPolicyOwn];                   // this CTA's share of the rows
-    double cks[48];                               // cos, sin of 15 degree steps (FP64)
-    double climb_dt[kMaxActions];
+    PolicyTurns turns;
     float bias[(kLayers - 1) * kHid + kOutPad];   // every layer's bias (fp32), in parameter order
-    int dh[kMaxActions];
     int choice[kPolicyOwn];
     int flags[2][kPolicyCluster];  // per CTA of the cluster: 1 rows in flight, 2 the queue may hold work
     int more;
@@ -225,6 +229,151 @@ __device__ __forceinline__ uint32_t pack_bf16(float x, float y) {
     return *reinterpret_cast<const uint32_t*>(&v);
 }
 
+// Takes the next work item into an empty row (one thread); false when the queue is empty. A row
+// whose plan ends at once stays empty and pulls again in the next round.
+__device__ __forceinline__ bool policy_refill(const PolicyArgs& a, PolicyRow& R) {
+    const Model& m = a.m;
+    const int w = atomicAdd(a.queue, 1);
+    if (w >= (a.n_dev ? *a.n_dev : a.n_items)) return false;
+    const int r = a.idx ? a.idx[w] : w;
+    const fmdp_request q = a.reqs[r];
+    R.req = r;
+    R.k = 0;
+    R.h = 0;
+    R.s[0] = q.ox;
+    R.s[1] = q.oy;
+    R.s[2] = q.oz;
+    const double dx = __dsub_rn(q.gx, q.ox), dy = __dsub_rn(q.gy, q.oy);
+    const double Lh = __dsqrt_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)));
+    R.c0 = Lh > 0.0 ? __ddiv_rn(dx, Lh) : 1.0;
+    R.s0 = Lh > 0.0 ? __ddiv_rn(dy, Lh) : 0.0;
+    R.step = __dmul_rn(q.speed_mps, m.dt);
+    R.cap2 = __dmul_rn(R.step, R.step);
+    R.gx = q.gx;
+    R.gy = q.gy;
+    R.gz = q.gz;
+    const int64_t T1 = q.depart_step + 1, T0 = a.tab.t_base;
+    const int64_t row1 = T1 % a.tab.T_win;
+    R.row1 = (int32_t)(row1 < 0 ? row1 + a.tab.T_win : row1);
+    R.k_lo = (int32_t)min(max(T0 - T1, (int64_t)0), (int64_t)INT_MAX);
+    R.k_hi = (int32_t)min(max(T0 + a.tab.T_win - T1, (int64_t)0), (int64_t)INT_MAX);
+    R.speed = (float)q.speed_mps;
+    R.horizon = q.horizon;
+    if (a.step_bound) {  // the judge rejects anything longer: stop there
+        const double b = judge_step_bound(q, m.dt, a.climb_step, a.slack);
+        if (b < (double)R.horizon) R.horizon = (int32_t)fmax(b, 0.0);
+    }
+    float* tr = a.traj + (size_t)r * a.cap * 3;
+    tr[0] = (float)q.ox;
+    tr[1] = (float)q.oy;
+    tr[2] = (float)q.oz;
+    R.status = -1;
+    const double ex = __dsub_rn(q.gx, q.ox), ey = __dsub_rn(q.gy, q.oy), ez = __dsub_rn(q.gz, q.oz);
+    const bool cap0 = __dadd_rn(__dadd_rn(__dmul_rn(ex, ex), __dmul_rn(ey, ey)), __dmul_rn(ez, ez)) <= R.cap2;
+    if (cap0 || R.horizon <= 0) {  // done before the first step
+        RolloutOut o;
+        o.n_points = 1;
+        o.status = cap0 ? kStatusCaptured : FMDP_REJ_HORIZON;
+        o.near_ties = 0;
+        o.steps = 0;
+        a.out[r] = o;
+        R.req = -1;  // the row pulls again next round
+    }
+    return true;
+}
+// The best action by logits among those that keep the successor inside the box, -1: none (a warp,
+// lanes = actions). The sums of products are written out, see sum2.
+__device__ __forceinline__ int policy_choice(const Model& m, const PolicyRow& R, const PolicyTurns& T, const float* logits) {
+    const int lane = threadIdx.x & 31, A = m.A;
+    const double* cks = T.cks;
+    float v = -INFINITY;
+    if (lane < A) {
+        int hn = R.h + T.dh[lane];
+        hn += hn < 0 ? 24 : 0;
+        hn -= hn >= 24 ? 24 : 0;
+        const float C = sum2((float)R.c0, (float)cks[2 * hn], -(float)R.s0, (float)cks[2 * hn + 1]);
+        const float Sn = sum2((float)R.s0, (float)cks[2 * hn], (float)R.c0, (float)cks[2 * hn + 1]);
+        const float x = fmaf((float)R.step, C, (float)R.s[0]), y = fmaf((float)R.step, Sn, (float)R.s[1]);
+        const float z = (float)R.s[2] + (float)T.climb_dt[lane];
+        const float mg = 1.0f;  // metres kept from the box faces
+        const bool inside = x > (float)m.box[0] + mg && x < (float)m.box[3] - mg && y > (float)m.box[1] + mg &&
+                            y < (float)m.box[4] - mg && z > (float)m.box[2] + mg && z < (float)m.box[5] - mg;
+        v = inside ? logits[lane] : -INFINITY;
+    }
+    float mx = v;
+    for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(kFull, mx, o));
+    const unsigned bm = __ballot_sync(kFull, v == mx && mx > -INFINITY);
+    return bm ? __ffs(bm) - 1 : -1;
+}
+// Exact FP64 advance of the chosen action (FastMDP's successor rule, Alg. 1; one thread)
+__device__ __forceinline__ void policy_advance(const PolicyArgs& a, PolicyRow& R, const PolicyTurns& T, int ch) {
+    const double* cks = T.cks;
+    bool done = false;
+    if (ch < 0) {
+        R.status = FMDP_REJ_NO_ACTION;
+        done = true;
+    } else {
+        int hn = R.h + T.dh[ch];
+        hn += hn < 0 ? 24 : 0;
+        hn -= hn >= 24 ? 24 : 0;
+        const double C = __dsub_rn(__dmul_rn(R.c0, cks[2 * hn]), __dmul_rn(R.s0, cks[2 * hn + 1]));
+        const double Sn = __dadd_rn(__dmul_rn(R.s0, cks[2 * hn]), __dmul_rn(R.c0, cks[2 * hn + 1]));
+        R.s[0] = __dadd_rn(R.s[0], __dmul_rn(R.step, C));
+        R.s[1] = __dadd_rn(R.s[1], __dmul_rn(R.step, Sn));
+        R.s[2] = __dadd_rn(R.s[2], T.climb_dt[ch]);
+        R.h = hn;
+        a.acts[(size_t)R.req * a.cap + R.k] = (uint8_t)ch;
+        R.k += 1;
+        float* tr = a.traj + ((size_t)R.req * a.cap + R.k) * 3;
+        tr[0] = (float)R.s[0];
+        tr[1] = (float)R.s[1];
+        tr[2] = (float)R.s[2];
+        const double ex = __dsub_rn(R.gx, R.s[0]), ey = __dsub_rn(R.gy, R.s[1]), ez = __dsub_rn(R.gz, R.s[2]);
+        if (__dadd_rn(__dadd_rn(__dmul_rn(ex, ex), __dmul_rn(ey, ey)), __dmul_rn(ez, ez)) <= R.cap2) {
+            R.status = kStatusCaptured;
+            done = true;
+        } else if (R.k >= R.horizon) {
+            R.status = FMDP_REJ_HORIZON;
+            done = true;
+        }
+    }
+    if (done) {
+        RolloutOut o;
+        o.n_points = R.k + 1;
+        o.status = R.status;
+        o.near_ties = 0;
+        o.steps = R.k;
+        a.out[R.req] = o;
+        R.req = -1;
+    }
+}
+// Features of an active row's state (one warp, or the `parts` warps that share it) into feat;
+// lane i's four of them as bf16
+__device__ __forceinline__ uint2 policy_features(const PolicyArgs& a, const PolicyRow& R, float inv_dt, float* feat,
+                                              unsigned long long* skey, int part, int parts, int bar) {
+    const int lane = threadIdx.x & 31;
+    float hc, hs;
+    heading_cs((float)R.c0, (float)R.s0, R.h, hc, hs);
+    const bool held = R.k >= R.k_lo && R.k < R.k_hi;
+    const int row = R.row1 + R.k - (R.row1 + R.k >= a.tab.T_win ? a.tab.T_win : 0);
+    warp_features(a.m, a.iv, a.tab, held ? row : -1, (float)R.s[0], (float)R.s[1], (float)R.s[2], hc, hs, R.speed, (float)R.gx,
+                  (float)R.gy, (float)R.gz, inv_dt, feat, skey, part, parts, bar);
+    const uint2 v = make_uint2(pack_bf16(feat[4 * lane], feat[4 * lane + 1]), pack_bf16(feat[4 * lane + 2], feat[4 * lane + 3]));
+    __syncwarp();
+    return v;
+}
+// the moves and every layer's bias into shared memory
+__device__ __forceinline__ void policy_tables(const PolicyArgs& a, PolicyTurns& T, float* bias) {
+    const int tid = threadIdx.x, A = a.m.A;
+    if (tid < 24) unit15(tid, T.cks[2 * tid], T.cks[2 * tid + 1]);
+    if (tid < kMaxActions) {
+        T.climb_dt[tid] = tid < A ? __dmul_rn(a.m.climb[tid], a.m.dt) : 0.0;
+        T.dh[tid] = tid < A ? a.m.dh[tid] : 0;
+    }
+    for (int l = 0, o = 0; l < kLayers; o += layer_out(l), ++l)
+        for (int j = tid; j < layer_out(l); j += kPolicyThreads) bias[o + j] = a.params[param_offset_b(l) + j];
+}
+
 }  // namespace
 
 __global__ void __cluster_dims__(kPolicyCluster, 1, 1) __launch_bounds__(kPolicyThreads, 1)
@@ -232,12 +381,10 @@ __global__ void __cluster_dims__(kPolicyCluster, 1, 1) __launch_bounds__(kPolicy
     extern __shared__ __align__(128) unsigned char psm[];
     PolicySmem& S = *reinterpret_cast<PolicySmem*>(psm);
     PolicyRow* rows = S.rows;
-    const double* cks = S.cks;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, NWp = kPolicyThreads / 32;
     const int g = lane >> 2, t = lane & 3;
     const int rank = (int)cta_rank();
     const Model& m = a.m;
-    const int A = m.A;
     const int MT = a.rows >> 4;                  // 16-row tiles
     const int own = a.rows / kPolicyCluster;     // rows whose states this CTA keeps
     const int first = rank * own;                // the first of them among the cluster's rows
@@ -245,14 +392,8 @@ __global__ void __cluster_dims__(kPolicyCluster, 1, 1) __launch_bounds__(kPolicy
     uint32_t act_peer[kPolicyCluster];
 #pragma unroll
     for (int c = 0; c < kPolicyCluster; ++c) act_peer[c] = peer_addr(smem_addr(S.act), c);
-    if (tid < 24) unit15(tid, S.cks[2 * tid], S.cks[2 * tid + 1]);
     if (tid < kPolicyOwn) rows[tid].req = -1;
-    if (tid < kMaxActions) {
-        S.climb_dt[tid] = tid < A ? __dmul_rn(m.climb[tid], m.dt) : 0.0;
-        S.dh[tid] = tid < A ? m.dh[tid] : 0;
-    }
-    for (int l = 0, o = 0; l < kLayers; o += layer_out(l), ++l)
-        for (int j = tid; j < layer_out(l); j += kPolicyThreads) S.bias[o + j] = a.params[param_offset_b(l) + j];
+    policy_tables(a, S.turns, S.bias);
     // this CTA's columns of every layer, once per launch
     for (int l = 0; l < kLayers; ++l) {
         const int cols = l == kLayers - 1 ? kPolicyOut : kPolicyCols, per = layer_in(l) / 8;
@@ -270,58 +411,7 @@ __global__ void __cluster_dims__(kPolicyCluster, 1, 1) __launch_bounds__(kPolicy
     cluster_sync();  // every CTA of the cluster is running before its memory is written
     for (int it = 0;; ++it) {
         // ---- refill empty rows from the work queue (one thread per row)
-        if (tid < own && rows[tid].req < 0 && S.more) {
-            const int w = atomicAdd(a.queue, 1);
-            if (w < (a.n_dev ? *a.n_dev : a.n_items)) {
-                const int r = a.idx ? a.idx[w] : w;
-                const fmdp_request q = a.reqs[r];
-                PolicyRow& R = rows[tid];
-                R.req = r;
-                R.k = 0;
-                R.h = 0;
-                R.s[0] = q.ox;
-                R.s[1] = q.oy;
-                R.s[2] = q.oz;
-                const double dx = __dsub_rn(q.gx, q.ox), dy = __dsub_rn(q.gy, q.oy);
-                const double Lh = __dsqrt_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)));
-                R.c0 = Lh > 0.0 ? __ddiv_rn(dx, Lh) : 1.0;
-                R.s0 = Lh > 0.0 ? __ddiv_rn(dy, Lh) : 0.0;
-                R.step = __dmul_rn(q.speed_mps, m.dt);
-                R.cap2 = __dmul_rn(R.step, R.step);
-                R.gx = q.gx;
-                R.gy = q.gy;
-                R.gz = q.gz;
-                const int64_t T1 = q.depart_step + 1, T0 = a.tab.t_base;
-                const int64_t row1 = T1 % a.tab.T_win;
-                R.row1 = (int32_t)(row1 < 0 ? row1 + a.tab.T_win : row1);
-                R.k_lo = (int32_t)min(max(T0 - T1, (int64_t)0), (int64_t)INT_MAX);
-                R.k_hi = (int32_t)min(max(T0 + a.tab.T_win - T1, (int64_t)0), (int64_t)INT_MAX);
-                R.speed = (float)q.speed_mps;
-                R.horizon = q.horizon;
-                if (a.step_bound) {  // the judge rejects anything longer: stop there
-                    const double b = judge_step_bound(q, m.dt, a.climb_step, a.slack);
-                    if (b < (double)R.horizon) R.horizon = (int32_t)fmax(b, 0.0);
-                }
-                float* tr = a.traj + (size_t)r * a.cap * 3;
-                tr[0] = (float)q.ox;
-                tr[1] = (float)q.oy;
-                tr[2] = (float)q.oz;
-                R.status = -1;
-                const double ex = __dsub_rn(q.gx, q.ox), ey = __dsub_rn(q.gy, q.oy), ez = __dsub_rn(q.gz, q.oz);
-                const bool cap0 = __dadd_rn(__dadd_rn(__dmul_rn(ex, ex), __dmul_rn(ey, ey)), __dmul_rn(ez, ez)) <= R.cap2;
-                if (cap0 || R.horizon <= 0) {  // done before the first step
-                    RolloutOut o;
-                    o.n_points = 1;
-                    o.status = cap0 ? kStatusCaptured : FMDP_REJ_HORIZON;
-                    o.near_ties = 0;
-                    o.steps = 0;
-                    a.out[r] = o;
-                    R.req = -1;  // the row pulls again next round
-                }
-            } else {
-                S.more = 0;
-            }
-        }
+        if (tid < own && rows[tid].req < 0 && S.more && !policy_refill(a, rows[tid])) S.more = 0;
         __syncthreads();
         int any = 0;
         for (int i = lane; i < own; i += 32) any |= rows[i].req >= 0;
@@ -334,17 +424,7 @@ __global__ void __cluster_dims__(kPolicyCluster, 1, 1) __launch_bounds__(kPolicy
         for (int rr = parts == 2 ? warp % (NWp / 2) : warp; rr < own; rr += NWp / parts) {
             const PolicyRow& R = rows[rr];
             uint2 v = make_uint2(0u, 0u);
-            float* feat = S.feat[rr % NWp];
-            if (R.req >= 0) {
-                float hc, hs;
-                heading_cs((float)R.c0, (float)R.s0, R.h, hc, hs);
-                const bool held = R.k >= R.k_lo && R.k < R.k_hi;
-                const int row = R.row1 + R.k - (R.row1 + R.k >= a.tab.T_win ? a.tab.T_win : 0);
-                warp_features(m, a.iv, a.tab, held ? row : -1, (float)R.s[0], (float)R.s[1], (float)R.s[2], hc, hs, R.speed,
-                              (float)R.gx, (float)R.gy, (float)R.gz, inv_dt, feat, S.skey[rr % NWp], part, parts, 1 + rr);
-                v = make_uint2(pack_bf16(feat[4 * lane], feat[4 * lane + 1]), pack_bf16(feat[4 * lane + 2], feat[4 * lane + 3]));
-                __syncwarp();
-            }
+            if (R.req >= 0) v = policy_features(a, R, inv_dt, S.feat[rr % NWp], S.skey[rr % NWp], part, parts, 1 + rr);
             if (part > 0) continue;
             const uint32_t off = (uint32_t)(((first + rr) * kActPad + 4 * lane) * sizeof(__nv_bfloat16));
 #pragma unroll
@@ -420,84 +500,189 @@ __global__ void __cluster_dims__(kPolicyCluster, 1, 1) __launch_bounds__(kPolicy
         cluster_sync();
         // ---- argmax over the actions that keep the successor inside the box (one warp per row)
         for (int rr = warp; rr < own; rr += NWp) {
-            const PolicyRow R = rows[rr];
+            const PolicyRow& R = rows[rr];
             if (R.req < 0) continue;
-            float v = -INFINITY;
-            if (lane < A) {
-                int hn = R.h + S.dh[lane];
-                hn += hn < 0 ? 24 : 0;
-                hn -= hn >= 24 ? 24 : 0;
-                const float C = (float)R.c0 * (float)cks[2 * hn] - (float)R.s0 * (float)cks[2 * hn + 1];
-                const float Sn = (float)R.s0 * (float)cks[2 * hn] + (float)R.c0 * (float)cks[2 * hn + 1];
-                const float x = (float)R.s[0] + (float)R.step * C, y = (float)R.s[1] + (float)R.step * Sn;
-                const float z = (float)R.s[2] + (float)S.climb_dt[lane];
-                const float mg = 1.0f;  // metres kept from the box faces
-                const bool inside = x > (float)m.box[0] + mg && x < (float)m.box[3] - mg && y > (float)m.box[1] + mg &&
-                                    y < (float)m.box[4] - mg && z > (float)m.box[2] + mg && z < (float)m.box[5] - mg;
-                v = inside ? S.logits[rr][lane] : -INFINITY;
-            }
-            float mx = v;
-            for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(kFull, mx, o));
-            const unsigned bm = __ballot_sync(kFull, v == mx && mx > -INFINITY);
-            if (lane == 0) S.choice[rr] = bm ? __ffs(bm) - 1 : -1;
+            const int ch = policy_choice(m, R, S.turns, S.logits[rr]);
+            if (lane == 0) S.choice[rr] = ch;
         }
         __syncthreads();
         // ---- exact FP64 advance of the chosen action (FastMDP's successor rule, Alg. 1)
-        if (tid < own && rows[tid].req >= 0) {
-            PolicyRow& R = rows[tid];
-            const int ch = S.choice[tid];
-            bool done = false;
-            if (ch < 0) {
-                R.status = FMDP_REJ_NO_ACTION;
-                done = true;
-            } else {
-                int hn = R.h + S.dh[ch];
-                hn += hn < 0 ? 24 : 0;
-                hn -= hn >= 24 ? 24 : 0;
-                const double C = __dsub_rn(__dmul_rn(R.c0, cks[2 * hn]), __dmul_rn(R.s0, cks[2 * hn + 1]));
-                const double Sn = __dadd_rn(__dmul_rn(R.s0, cks[2 * hn]), __dmul_rn(R.c0, cks[2 * hn + 1]));
-                R.s[0] = __dadd_rn(R.s[0], __dmul_rn(R.step, C));
-                R.s[1] = __dadd_rn(R.s[1], __dmul_rn(R.step, Sn));
-                R.s[2] = __dadd_rn(R.s[2], S.climb_dt[ch]);
-                R.h = hn;
-                a.acts[(size_t)R.req * a.cap + R.k] = (uint8_t)ch;
-                R.k += 1;
-                float* tr = a.traj + ((size_t)R.req * a.cap + R.k) * 3;
-                tr[0] = (float)R.s[0];
-                tr[1] = (float)R.s[1];
-                tr[2] = (float)R.s[2];
-                const double ex = __dsub_rn(R.gx, R.s[0]), ey = __dsub_rn(R.gy, R.s[1]), ez = __dsub_rn(R.gz, R.s[2]);
-                if (__dadd_rn(__dadd_rn(__dmul_rn(ex, ex), __dmul_rn(ey, ey)), __dmul_rn(ez, ez)) <= R.cap2) {
-                    R.status = kStatusCaptured;
-                    done = true;
-                } else if (R.k >= R.horizon) {
-                    R.status = FMDP_REJ_HORIZON;
-                    done = true;
-                }
-            }
-            if (done) {
-                RolloutOut o;
-                o.n_points = R.k + 1;
-                o.status = R.status;
-                o.near_ties = 0;
-                o.steps = R.k;
-                a.out[R.req] = o;
-                R.req = -1;
-            }
-        }
+        if (tid < own && rows[tid].req >= 0) policy_advance(a, rows[tid], S.turns, S.choice[tid]);
         __syncthreads();
     }
 }
 
-size_t policy_smem_bytes() { return sizeof(PolicySmem); }
+// Many proposals at once: 32 rows per CTA, every CTA by itself, all weights streamed past its rows in
+// every step (18 chunks by bulk copies, four buffers, three chunks ahead). It is bound by that stream
+// and a step takes longer than the cluster's, but the chip carries twice as many rows: see
+// policy_streamed.
+namespace {
+constexpr int kStreamRows = 32, kStreamBufs = 4;
+constexpr int kStreamChunks = kFeat / kChunkK + (kLayers - 1) * (kHid / kChunkK);  // per step
 
-cudaError_t prepare_policy_kernel() {
-    return cudaFuncSetAttribute(policy_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)policy_smem_bytes());
+struct PolicyStreamSmem {
+    __nv_bfloat16 w[kStreamBufs][kHid * kChunkPad];
+    __nv_bfloat16 act[2][kStreamRows * kActPad];
+    float logits[kStreamRows][kOutPad];
+    float feat[kPolicyThreads / 32][kFeat];
+    unsigned long long skey[kPolicyThreads / 32][kSectors];
+    PolicyRow rows[kStreamRows];
+    PolicyTurns turns;
+    float bias[(kLayers - 1) * kHid + kOutPad];
+    uint64_t bars[kStreamBufs];
+    int choice[kStreamRows];
+    int more;
+};
+static_assert(sizeof(PolicyStreamSmem) <= 232448, "shared memory of one CTA");
+}  // namespace
+
+__global__ void __launch_bounds__(kPolicyThreads, 1) policy_stream_kernel(const __grid_constant__ PolicyArgs a) {
+    extern __shared__ __align__(128) unsigned char psm[];
+    PolicyStreamSmem& S = *reinterpret_cast<PolicyStreamSmem*>(psm);
+    PolicyRow* rows = S.rows;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, NWp = kPolicyThreads / 32;
+    const int g = lane >> 2, t = lane & 3;
+    const float inv_dt = (float)(1.0 / a.m.dt);
+    constexpr int MT = kStreamRows / 16;
+    // Chunks are numbered across steps: chunk q is in buffer q mod kStreamBufs, its (q / kStreamBufs)-th
+    // fill. The buffer of chunk q + 3 was read last as chunk q - 1, and every thread has passed the
+    // barrier after that when chunk q is waited for.
+    long long q = 0, issued = 0;
+    auto issue = [&]() {  // thread 0
+        int l = 0, kc = (int)(issued % kStreamChunks);
+        while (kc >= layer_in(l) / kChunkK) kc -= layer_in(l++) / kChunkK;
+        const uint32_t bytes = (uint32_t)(wp_chunk_elems(l) * sizeof(__nv_bfloat16));
+        uint64_t* bar = &S.bars[issued % kStreamBufs];
+        bar_expect(bar, bytes);
+        bulk_load(S.w[issued % kStreamBufs], a.Wp + wp_layer_offset(l) + (size_t)kc * wp_chunk_elems(l), bytes, bar);
+        ++issued;
+    };
+    auto chunk_came = [&](long long c) { return bar_wait(&S.bars[c % kStreamBufs], (uint32_t)((c / kStreamBufs) & 1)); };
+    if (tid < kStreamRows) rows[tid].req = -1;
+    policy_tables(a, S.turns, S.bias);
+    if (tid == 0) {
+        for (int b = 0; b < kStreamBufs; ++b) bar_init(&S.bars[b]);
+        S.more = 1;  // 1 while the queue may hold work
+        for (int b = 0; b < kStreamBufs - 1; ++b) issue();
+    }
+    __syncthreads();
+    bool failed = false;
+    while (!failed) {
+        // ---- refill empty rows from the work queue (one thread per row)
+        if (tid < kStreamRows && rows[tid].req < 0 && S.more && !policy_refill(a, rows[tid])) S.more = 0;
+        __syncthreads();
+        const bool any = __any_sync(kFull, rows[lane].req >= 0), more = S.more != 0;
+        __syncthreads();
+        if (!any && !more) break;
+        if (!any) continue;
+        // ---- features of every active row (one warp per row)
+        for (int rr = warp; rr < kStreamRows; rr += NWp) {
+            uint2 v = make_uint2(0u, 0u);
+            if (rows[rr].req >= 0) v = policy_features(a, rows[rr], inv_dt, S.feat[warp], S.skey[warp], 0, 1, 0);
+            *reinterpret_cast<uint2*>(S.act[0] + (size_t)rr * kActPad + 4 * lane) = v;
+        }
+        __syncthreads();
+        // ---- the MLP, layer by layer, chunk by chunk
+        for (int l = 0; l < kLayers && !failed; ++l) {
+            const __nv_bfloat16* xin = S.act[l & 1];
+            const bool last = l == kLayers - 1;
+            float acc[MT][4][4];
+#pragma unroll
+            for (int i = 0; i < MT * 16; ++i) acc[i >> 4][(i >> 2) & 3][i & 3] = 0.f;
+            for (int kc = 0; kc < layer_in(l) / kChunkK && !failed; ++kc, ++q) {
+                const bool came = chunk_came(q);
+                if (!came && lane == 0) atomicExch(a.err, FMDP_ERR_TIMEOUT);
+                if (tid == 0 && came) issue();
+                const __nv_bfloat16* wb = S.w[q % kStreamBufs];
+                if (!last) {  // warp: columns [32 warp, 32 warp + 32), all rows
+#pragma unroll
+                    for (int kk = 0; kk < kChunkK; kk += 16) {
+                        uint32_t af[MT][4], b0[4], b1[4];
+                        const __nv_bfloat16* p =
+                            wb + (size_t)(warp * 32 + (lane >> 4) * 8 + (lane & 7)) * kChunkPad + kk + ((lane >> 3) & 1) * 8;
+                        ldsm4(b0, p);
+                        ldsm4(b1, p + 16 * kChunkPad);
+#pragma unroll
+                        for (int mt = 0; mt < MT; ++mt) {
+                            frag_a(af[mt], xin + (size_t)mt * 16 * kActPad, kActPad, kc * kChunkK + kk, lane);
+                            mma_bf16(acc[mt][0], af[mt], b0);
+                            mma_bf16(acc[mt][1], af[mt], b0 + 2);
+                            mma_bf16(acc[mt][2], af[mt], b1);
+                            mma_bf16(acc[mt][3], af[mt], b1 + 2);
+                        }
+                    }
+                } else if (warp < MT * 4) {  // warp: 16 rows, 8 of the 32 logits
+#pragma unroll
+                    for (int kk = 0; kk < kChunkK; kk += 32) {
+                        uint32_t af[4], b[4];
+                        const __nv_bfloat16* x = xin + (size_t)(warp >> 2) * 16 * kActPad;
+                        ldsm4(b, wb + (size_t)((warp & 3) * 8 + (lane & 7)) * kChunkPad + kk + (lane >> 3) * 8);
+                        frag_a(af, x, kActPad, kc * kChunkK + kk, lane);
+                        mma_bf16(acc[0][0], af, b);
+                        frag_a(af, x, kActPad, kc * kChunkK + kk + 16, lane);
+                        mma_bf16(acc[0][0], af, b + 2);
+                    }
+                }
+                // the chunk's buffer is free again; a wait that expired anywhere stops every thread
+                failed = __syncthreads_or(came ? 0 : 1) != 0;
+            }
+            const float* bias = S.bias + l * kHid;
+            if (!last) {
+                __nv_bfloat16* out = S.act[(l + 1) & 1];
+#pragma unroll
+                for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const int col = warp * 32 + j * 8 + 2 * t;
+                        const float c0 = bias[col], c1 = bias[col + 1];
+#pragma unroll
+                        for (int u = 0; u < 2; ++u)
+                            *reinterpret_cast<uint32_t*>(out + (size_t)(mt * 16 + g + 8 * u) * kActPad + col) =
+                                pack_bf16(fmaxf(acc[mt][j][2 * u] + c0, 0.f), fmaxf(acc[mt][j][2 * u + 1] + c1, 0.f));
+                    }
+            } else if (warp < MT * 4) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int r = (warp >> 2) * 16 + g + (i >= 2 ? 8 : 0), col = (warp & 3) * 8 + 2 * t + (i & 1);
+                    S.logits[r][col] = col < kOut ? acc[0][0][i] + bias[col] : -INFINITY;
+                }
+            }
+            __syncthreads();
+        }
+        if (failed) break;
+        // ---- actions and advance
+        for (int rr = warp; rr < kStreamRows; rr += NWp) {
+            if (rows[rr].req < 0) continue;
+            const int ch = policy_choice(a.m, rows[rr], S.turns, S.logits[rr]);
+            if (lane == 0) S.choice[rr] = ch;
+        }
+        __syncthreads();
+        if (tid < kStreamRows && rows[tid].req >= 0) policy_advance(a, rows[tid], S.turns, S.choice[tid]);
+        __syncthreads();
+    }
+    // the copies still in flight, before the block's shared memory is given back
+    // (after an expired wait the chunk waited for is among them)
+    if (tid == 0)
+        for (long long c = q > 0 ? q - 1 : 0; c < issued; ++c) chunk_came(c);
 }
 
-cudaError_t launch_policy(const PolicyArgs& a, int n_ctas, cudaStream_t s) {
-    if (a.n_items <= 0 || n_ctas <= 0) return cudaSuccess;
-    policy_kernel<<<n_ctas, kPolicyThreads, policy_smem_bytes(), s>>>(a);
+cudaError_t prepare_policy_kernels() {
+    const cudaError_t e =
+        cudaFuncSetAttribute(policy_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(PolicySmem));
+    return e != cudaSuccess ? e
+                            : cudaFuncSetAttribute(policy_stream_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   (int)sizeof(PolicyStreamSmem));
+}
+
+cudaError_t launch_policy(PolicyArgs a, int n, int n_sm, cudaStream_t s) {
+    if (n <= 0) return cudaSuccess;
+    if (policy_streamed(n, n_sm)) {
+        const int ctas = (n + kStreamRows - 1) / kStreamRows;
+        policy_stream_kernel<<<ctas < n_sm ? ctas : n_sm, kPolicyThreads, sizeof(PolicyStreamSmem), s>>>(a);
+    } else {
+        a.rows = policy_rows_for(n, n_sm);
+        policy_kernel<<<policy_ctas_for(n, a.rows, n_sm), kPolicyThreads, sizeof(PolicySmem), s>>>(a);
+    }
     return cudaGetLastError();
 }
 

@@ -110,6 +110,13 @@ __device__ __forceinline__ uint32_t sample_hash(float x, float y, float z) {
     return __float_as_uint(x) ^ (__float_as_uint(y) * 2654435761u) ^ (__float_as_uint(z) * 40503u);
 }
 __device__ __forceinline__ float clampf(float v, float lo, float hi) { return fminf(fmaxf(v, lo), hi); }
+// a b + c d with the first product fused, and sums of three squares: written out, because the
+// features are inlined into several kernels and have to be the same bits in each (which product of
+// a sum is fused would be the compiler's choice in each copy)
+__device__ __forceinline__ float sum2(float a, float b, float c, float d) { return fmaf(a, b, __fmul_rn(c, d)); }
+__device__ __forceinline__ float squares3(float x, float y, float z) { return fmaf(z, z, sum2(x, x, y, y)); }
+// (one copy for every kernel, for the same reason)
+static __device__ __noinline__ float feature_ground(const Model& m, float x, float y) { return terrain32(m, x, y); }
 // Features of one state, computed by one warp into out[kFeat] (shared memory). s: position;
 // (hc, hs): heading cos / sin; skey: kSectors words of scratch in shared memory. The order of
 // reading and of the index's items does not change the result: each sector keeps its minimum of
@@ -153,11 +160,11 @@ __device__ inline void warp_features(const Model& m, const IndexView& iv, const 
     if (lane == 0 && part == parts - 1) {  // own state, while the bounds arrive
         const float z0 = (float)m.box[2], z1 = (float)m.box[5];
         out[0] = (sz - z0) / (z1 - z0);
-        const float clr = m.hm ? sz - terrain32(m, sx, sy) : sz - z0;
+        const float clr = m.hm ? sz - feature_ground(m, sx, sy) : sz - z0;
         out[1] = clampf(clr / 200.f, -1.f, 4.f);
         const float Gx = gx - sx, Gy = gy - sy, Gz = gz - sz;
-        const float gf = Gx * hc + Gy * hs, gl = -Gx * hs + Gy * hc;
-        const float gh = sqrtf(gf * gf + gl * gl);
+        const float gf = sum2(Gx, hc, Gy, hs), gl = sum2(Gy, hc, -Gx, hs);
+        const float gh = sqrtf(sum2(gf, gf, gl, gl));
         out[2] = clampf(gf / 5000.f, -4.f, 4.f);
         out[3] = clampf(gl / 5000.f, -4.f, 4.f);
         out[4] = clampf(Gz / 200.f, -4.f, 4.f);
@@ -202,14 +209,14 @@ __device__ inline void warp_features(const Model& m, const IndexView& iv, const 
     // sector feature of the nearest sample P1 (and the same plan's next sample P2)
     auto emit = [&](float4 P1, float4 P2, float d2, int sec) {
         const float rx = P1.x - sx, ry = P1.y - sy, rz = P1.z - sz;
-        const float rf = rx * hc + ry * hs, rl = -rx * hs + ry * hc;
+        const float rf = sum2(ry, hs, rx, hc), rl = sum2(ry, hc, -rx, hs);
         float vx = 0.f, vy = 0.f, vz = 0.f;
         if (P2.x == P2.x) {
             vx = (P2.x - P1.x) * inv_dt;
             vy = (P2.y - P1.y) * inv_dt;
             vz = (P2.z - P1.z) * inv_dt;
         }
-        const float vf = vx * hc + vy * hs, vl = -vx * hs + vy * hc;
+        const float vf = sum2(vx, hc, vy, hs), vl = sum2(vy, hc, -vx, hs);
         const float w = 1.f - sqrtf(d2) / kRF;
         float* o = out + kOwn + 6 * sec;
         o[0] = rf * (1.f / 500.f) * w;
@@ -222,9 +229,9 @@ __device__ inline void warp_features(const Model& m, const IndexView& iv, const 
     // key of sample P1: (squared distance, position hash), all-ones beyond R_F
     auto key_of = [&](float4 P1, float& d2, int& sec) {
         const float rx = P1.x - sx, ry = P1.y - sy, rz = P1.z - sz;
-        d2 = rx * rx + ry * ry + rz * rz;
+        d2 = squares3(rx, ry, rz);
         if (!(d2 < R2)) return ~0ull;
-        sec = sector_of(rx * hc + ry * hs, -rx * hs + ry * hc, rz);
+        sec = sector_of(sum2(rx, hc, ry, hs), sum2(ry, hc, -rx, hs), rz);
         return ((unsigned long long)__float_as_uint(d2) << 32) | sample_hash(P1.x, P1.y, P1.z);
     };
     // pass 1: every sector's least key; a lane keeps its first two in-range samples
@@ -271,8 +278,8 @@ __device__ __forceinline__ void heading_cs(float c0, float s0, int h, float& hc,
     const float a = (float)h * (3.14159265358979f / 12.f);
     float sk, ck;
     sincosf(a, &sk, &ck);
-    hc = c0 * ck - s0 * sk;
-    hs = s0 * ck + c0 * sk;
+    hc = sum2(c0, ck, -s0, sk);
+    hs = sum2(s0, ck, c0, sk);
 }
 
 // ---- device entry points (learned.cu)
@@ -344,7 +351,8 @@ struct PolicyArgs {
     float* traj;              // [n][cap][3]
     uint8_t* acts;            // [n][cap]
     RolloutOut* out;          // [n]
-    int32_t rows;             // requests per cluster: a multiple of 16 up to kPolicyRows
+    int32_t* err;             // device error word
+    int32_t rows;             // requests per cluster: a multiple of 16 up to kPolicyRows (set by the launch)
     // 1: stop a proposal at the judge's step bound (a longer one would be rejected anyway)
     int32_t step_bound;
     double slack, climb_step;
@@ -361,9 +369,16 @@ inline int policy_ctas_for(int n, int rows, int n_sm) {
     const int clusters = n_sm / kPolicyCluster > 0 ? n_sm / kPolicyCluster : 1, want = (n + rows - 1) / rows;
     return kPolicyCluster * (want < clusters ? want : clusters);
 }
-size_t policy_smem_bytes();
-cudaError_t prepare_policy_kernel();
-cudaError_t launch_policy(const PolicyArgs& a, int n_ctas, cudaStream_t s);
+// n work items by policy_stream_kernel instead, whose CTAs share nothing and carry 32 rows each (4864
+// at once, the clusters 2432): past the clusters' first round of rows by a fifth. Among 3000 plans
+// 2432 proposals take 35.0 ms by clusters, 3000 take 39.4, 5000 51 and 10 000 75; streamed 38.0 up to
+// 4864 and 55 for 10 000. (20 000 plans: 42, 46, 60 and 96; 46.3 and 69.)
+inline bool policy_streamed(int n, int n_sm) {
+    const int clusters = n_sm / kPolicyCluster > 0 ? n_sm / kPolicyCluster : 1;
+    return n > 6 * kPolicyRows * clusters / 5;
+}
+cudaError_t prepare_policy_kernels();
+cudaError_t launch_policy(PolicyArgs a, int n, int n_sm, cudaStream_t s);  // n: the most work items there may be
 
 // Judge: a proposal is accepted when it reaches the goal, passes the separation and
 // terrain checks, and takes at most (1 + slack) times the fewest steps any trajectory
