@@ -345,7 +345,7 @@ fmdp_status fmdp_schedule_cosim(fmdp_ctx* ctx, const fmdp_request* reqs, int32_t
 /* Failure-detection self-test (no counterpart in the paper). Every wait of the library's
  * kernels is bounded (about a second of SM cycles) and an expired wait ends the call with
  * FMDP_ERR_TIMEOUT instead of hanging the device. This call makes one such wait run out on
- * purpose without a fault: it co-simulates two requests whose grid barrier also waits for
+ * purpose without a fault: it co-simulates two requests that also wait for the record of
  * a third aircraft that is never launched, so every CTA's wait expires and the kernel
  * returns. observed (optional) receives the status that call produced. Returns FMDP_OK
  * when that status was FMDP_ERR_TIMEOUT and nothing was admitted; the context stays
@@ -493,7 +493,9 @@ typedef struct {
     double rollout_ms, sepcheck_ms, admit_ms; /* summed CUDA-event durations */
     int64_t rollout_steps;                    /* rollout steps executed */
     int64_t slots_scanned;                    /* (step, slot) pairs scanned by rollouts */
-    int64_t sep_pairs;                        /* (sample, slot) pairs scanned by sep_check */
+    int64_t sep_pairs;                        /* (sample, slot) pairs decided by separation checks
+                                                 (with the spatial index most of them by their
+                                                 cell, unread) */
     int32_t cluster_size, threads_per_cta, slots_per_cta;
     int32_t reserved;
     int64_t phase_cycles[6];  /* on = 2: summed SM cycles of rollout phases. Spatial index: control

@@ -674,8 +674,8 @@ fmdp_status fmdp_schedule_cosim(fmdp_ctx* c, const fmdp_request* reqs, int32_t n
 fmdp_status fmdp_selftest_wait_timeout(fmdp_ctx* c, int32_t* observed) {
     if (!c) return FMDP_ERR_ARG;
     return guard(c, [&] {
-        // two requests far from everything, co-simulated with a barrier that also waits for
-        // a third aircraft that is never launched: every wait must run out and report
+        // two requests far from everything, co-simulated while waiting for the record of a third
+        // aircraft that is never launched: every wait must run out and report
         fmdp_request r[2] = {};
         const double cx = 0.5 * (c->air.x0 + c->air.x1), cy = 0.5 * (c->air.y0 + c->air.y1);
         const double cz = 0.5 * (c->air.z0 + c->air.z1);

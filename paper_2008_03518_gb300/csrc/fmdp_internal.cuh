@@ -182,7 +182,7 @@ struct RolloutArgs {
     const int32_t* n_dev;  // batch mode: number of work items, read on the device (nullptr: n_req)
     unsigned long long* phase;  // [6] per-phase cycle counters (diagnostic) or nullptr
     int32_t indexed;  // 1: read the items near the state from the spatial index (cs must be 1)
-    int32_t icap;     // indexed mode: options.index_stage_items; a step's list holds icap / 8 candidate wells
+    int32_t icap;     // indexed mode: options.index_stage_items; a step's list holds icap / 8 plan samples
     IndexView iv;
     unsigned long long* items_ctr;  // indexed mode: items read by the steps (statistics) or nullptr
     unsigned long long* qe_ctr;     // indexed mode (statistics) or nullptr: [0] items culled, [1] items

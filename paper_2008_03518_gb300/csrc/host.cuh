@@ -215,7 +215,7 @@ struct fmdp_ctx {
     std::map<std::array<int32_t, 4>, fmdp_tune_entry> tune;
     int32_t try_threads = 0, try_icap = 0;
 
-    // batch co-simulation: per-step aircraft records and the grid barrier words
+    // batch co-simulation: per-step aircraft records
     DevArray<double> cs_mem;
 
     // one-launch separation check (fmdp_sep_check): trajectory and report in mapped host memory

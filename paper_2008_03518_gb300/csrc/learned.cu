@@ -1,7 +1,8 @@
 // Learned proposal kernels (sm_103a): training-set collection from FastMDP rollouts, the
 // optimiser (loss and gradient: train.cu), and policy rollouts that run
-// many requests in lock step through the MLP (mma.sync m16n8k16, weights staged by bulk
-// copy). The network, its inputs and its loss are stated in plain FP64 in the oracle.
+// many requests in lock step through the MLP (mma.sync m16n8k16; the weights resident in a
+// cluster's shared memory, or streamed by bulk copies past many rows). The network, its inputs
+// and its loss are stated in plain FP64 in the oracle.
 #include <climits>
 
 #include "learned.cuh"

@@ -159,32 +159,16 @@ __device__ __forceinline__ unsigned long long look_sum_term(float l, float ref) 
     return (unsigned long long)__float2ull_rn(t);
 }
 
-// ---- double-float (fp32 pair) arithmetic: exact sums of fp32 numbers
-__device__ __forceinline__ void lk_two_sum(float a, float b, float& s, float& e) {
-    s = __fadd_rn(a, b);
-    const float bb = __fsub_rn(s, a);
-    e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
-}
-__device__ __forceinline__ void lk_fast_two_sum(float a, float b, float& s, float& e) {
-    s = __fadd_rn(a, b);
-    e = __fsub_rn(b, __fsub_rn(s, a));
-}
-__device__ __forceinline__ void lk_df_add(float& hi, float& lo, float dh, float dl) {
-    float s, e;
-    lk_two_sum(hi, dh, s, e);
-    e = __fadd_rn(e, __fadd_rn(lo, dl));
-    lk_fast_two_sum(s, e, hi, lo);
-}
 // |G|^2 of a double-float G as a double-float, and its fp32 root
 __device__ __forceinline__ float lk_goal_dist(float Ghx, float Ghy, float Ghz, float Glx, float Gly, float Glz, float& Sh,
                                               float& Sl) {
     const float p0 = Ghx * Ghx, p1 = Ghy * Ghy, p2 = Ghz * Ghz;
     const float e0 = fmaf(Ghx, Ghx, -p0), e1 = fmaf(Ghy, Ghy, -p1), e2 = fmaf(Ghz, Ghz, -p2);
     float s1, t1, s2, t2;
-    lk_two_sum(p0, p1, s1, t1);
-    lk_two_sum(s1, p2, s2, t2);
+    two_sum(p0, p1, s1, t1);
+    two_sum(s1, p2, s2, t2);
     const float lo = t1 + t2 + e0 + e1 + e2 + 2.f * (Ghx * Glx + Ghy * Gly + Ghz * Glz);
-    lk_fast_two_sum(s2, lo, Sh, Sl);
+    fast_two_sum(s2, lo, Sh, Sl);
     return Sh > 0.f ? sqrtf(Sh) : 0.f;
 }
 // log2 of the goal term |r_g| gamma^|G| at a state whose goal vector is the double-float G,
@@ -201,10 +185,10 @@ __device__ __forceinline__ void lk_goal_log(const Model& m, float Ghx, float Ghy
     const float pe = fmaf(rt, lg_hi, -p);
     const float lo2 = pe + rt * lg_lo + rl * lg_hi;
     float Lh, Le;
-    lk_two_sum(p, l2r_hi, Lh, Le);
+    two_sum(p, l2r_hi, Lh, Le);
     Le = Le + (lo2 + l2r_lo);
     float LH, LL;
-    lk_fast_two_sum(Lh, Le, LH, LL);
+    fast_two_sum(Lh, Le, LH, LL);
     float fl = floorf(LH);
     float fr = (LH - fl) + LL;
     if (fr >= 1.f) { fr -= 1.f; fl += 1.f; }
@@ -416,7 +400,8 @@ __device__ __noinline__ void look_score_over(const LookArgs& a, const LookScore&
 size_t lookahead_smem_bytes(int A, int W) { return look_layout(A, W).total; }
 
 // NT 512: sixteen warps share out a step's samples and its projected states, one CTA per SM; 256 (for
-// co-simulations, which all have to be resident): two CTAs per SM.
+// co-simulations, which all have to be resident): two CTAs per SM. Both leave 128 registers a thread;
+// some 120 bytes of a thread's state are spilled.
 template <int NT>
 __global__ void __launch_bounds__(NT, 512 / NT) lookahead_kernel(const __grid_constant__ LookArgs a) {
     extern __shared__ __align__(128) unsigned char lsm[];
@@ -1016,8 +1001,8 @@ __global__ void __launch_bounds__(NT, 512 / NT) lookahead_kernel(const __grid_co
                     const float* Df = lane < 2 ? Dh + 4 * hn + 2 * lane : Dz2 + 2 * a1;
                     const double D = (lane == 0 ? Dx : Dy)[hn], s0 = st->s[lane];
                     const double s1 = __dadd_rn(s0, lane < 2 ? D : Dz[a1]);
-                    lk_df_add((&st->shx)[lane], (&st->slx)[lane], Df[0], Df[1]);
-                    lk_df_add((&st->Ghx)[lane], (&st->Glx)[lane], -Df[0], -Df[1]);
+                    df_add((&st->shx)[lane], (&st->slx)[lane], Df[0], Df[1]);
+                    df_add((&st->Ghx)[lane], (&st->Glx)[lane], -Df[0], -Df[1]);
                     G = (&st->Ghx)[lane] + (&st->Glx)[lane];
                     st->prev[lane] = s0;
                     st->s[lane] = s1;
