@@ -385,6 +385,7 @@ void grow_keep(fmdp_ctx* c, DevArray<T>& a, size_t want, size_t keep) {
 constexpr int32_t kBatchDefault = 256;
 constexpr int32_t kBatchMax = 1024;
 constexpr int32_t kLookScanPairs = 1024;  // see set_look_index
+constexpr int64_t kCheckScanPairs = 3 << 18;  // see launch_check
 constexpr int32_t kMaxStageItems = 2234;  // options.index_stage_items beyond this are refused when a plan starts
 
 // ------------------------------------------------------------------ host runtime (host_table.cu)
