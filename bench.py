@@ -99,10 +99,11 @@ class ClockSampler:
         return {"sm_mhz": statistics.median(sm), "sm_max_mhz": max(mx), "samples": len(sm), "reasons": sorted(reasons)}
 
 
-def traffic_from_profile(kernel_src):
+def traffic_from_profile(csrc):
     """DRAM traffic per algorithmic byte recorded from an ncu capture, valid only while the
-    kernel's source is unchanged (the profile records the source digest)."""
-    digest = hashlib.sha256(open(kernel_src, "rb").read()).hexdigest()[:16]
+    kernel's sources are unchanged (the profile records their digest)."""
+    sources = [open(os.path.join(csrc, f), "rb").read() for f in ("rollout.cu", "plan_indexed.cuh")]
+    digest = hashlib.sha256(b"".join(sources)).hexdigest()[:16]
     path = os.path.join(ROOT, "profiles", "rollout_kernel_c2.md")
     try:
         for line in open(path):
@@ -379,7 +380,7 @@ def main():
                     help="also append the result line to this file (one JSON line per run)")
     ap.add_argument("--case", default=None, choices=["policy20k", "sepcheck20k"],
                     help="a small profiling case instead of the benchmark (one JSON line): the policy kernel "
-                         "or the row-major separation check at 20k known plans")
+                         "or the separation check of a batch, row by row, at 20k known plans")
     args = ap.parse_args()
     args.warmup = max(args.warmup, 3)
     if args.case:
@@ -463,7 +464,7 @@ def main():
     indexed = kt["items_scanned"] > 0
     bytes_per_launch = (32.0 * kt["items_scanned"] if indexed else 12.0 * kt["slots_scanned"]) / launches
     achieved = bytes_per_launch / (avg_ms / 1e3) / 1e9
-    tr = traffic_from_profile(os.path.join(ROOT, "paper_2008_03518_gb300", "csrc", "rollout.cu"))
+    tr = traffic_from_profile(os.path.join(ROOT, "paper_2008_03518_gb300", "csrc"))
     kernel_ms = {k: kt[k] for k in ("rollout_ms", "sepcheck_ms", "admit_ms", "influence_ms")}
     roofline = {"kernel": "rollout_kernel", "bound": "hbm", "achieved": achieved, "peak": peaks["hbm_gbs"],
                 "unit": "GB/s", "frac": achieved / peaks["hbm_gbs"],
@@ -492,7 +493,7 @@ def main():
         rows, ep, tsec = tr3["rows"], tr3["epochs"], tr3["seconds"]
         # a training row-epoch: forward, then gradients of the inputs and of the weights
         train_tflops = 3.0 * mlp_flops_per_row() * rows * ep / tsec / 1e12
-        mlp = {"kernel": "MLP training (bf16 mma.sync GEMM, 64 x 64 tiles) and policy rollouts", "bound": "tensor",
+        mlp = {"kernel": "MLP training (bf16 mma.sync, three launches per batch) and policy rollouts", "bound": "tensor",
                "training": {"achieved": train_tflops, "peak": peaks["bf16_tflops"], "unit": "TFLOP/s",
                             "frac": train_tflops / peaks["bf16_tflops"], "rows": rows, "epochs": ep,
                             "seconds": tsec, "final_loss": tr3["final_loss"]},
@@ -527,7 +528,7 @@ def main():
         res3 = s3.fetch_staged()
         items = sum(len(p.xyz) for p in sc3.plans) + sum(r["n_points"] for r in res3 if r["verdict"] == 0)
         samples = sum(r["n_points"] for r in res3)
-        # (request sample, plan sample of the same step) pairs the check measures
+        # (request sample, plan sample of the same step) pairs the check decides, most of them by cell
         per_row = np.zeros(sc3.n_slices_window + 1)
         for t0_, n_ in [(p.t0, len(p.xyz)) for p in sc3.plans] + \
                 [(int(q["depart"]), r["n_points"]) for q, r in zip(sc3.requests, res3) if r["verdict"] == 0]:
@@ -538,19 +539,11 @@ def main():
                           for q, r in zip(sc3.requests, res3)))
         if k3["sepcheck_launches"] > 0 and k3["sepcheck_ms"] > 0:
             per = k3["sepcheck_ms"] / k3["sepcheck_launches"]
-            b = 16.0 * items + 16.0 * samples
-            fl = 10.0 * pairs / (per / 1e3) / 1e12
             sweep["sepcheck_rows_20k"] = {
-                "kernel": "sepcheck_rows_kernel", "bound": "alu",
-                "hbm": {"achieved": b / (per / 1e3) / 1e9, "peak": peaks["hbm_gbs"], "unit": "GB/s",
-                        "frac": b / (per / 1e3) / 1e9 / peaks["hbm_gbs"], "algorithmic_bytes_per_launch": b,
-                        "bytes_from": "16 B per plan sample of every row (each row's items streamed once per "
-                                      "launch) + 16 B per request sample"},
-                "fp32": {"achieved": fl, "peak": peaks_dev["fp32_tflops"], "unit": "TFLOP/s",
-                         "frac": fl / peaks_dev["fp32_tflops"], "pairs_per_launch": pairs,
-                         "ops_from": "10 FP32 operations per (request sample, plan sample) pair: offsets, squared "
-                                     "horizontal distance, |dz|, two threshold tests, two minima"},
-                "avg_launch_ms": per, "launches": k3["sepcheck_launches"]}
+                "kernel": "sepcheck_row_cells_kernel", "bound": "latency of the cells' dependent loads",
+                "request_samples": samples, "plan_samples": items, "pairs_decided_per_launch": pairs,
+                "pairs_decided_per_s": pairs / (per / 1e3), "avg_launch_ms": per,
+                "launches": k3["sepcheck_launches"]}
         s3.close()
         sc4 = S.c4_serving()
         s4 = Scheduler.from_scenario(sc4)
@@ -649,7 +642,7 @@ def main():
         modes["cosim"] = {"known_plans": len(sc.plans), "value": world * nc / (mcs / 1e3), "unit": UNIT,
                           "ms_per_step": mcs, "requests_per_step": nc,
                           "admitted": int(sum(r["verdict"] == 0 for r in rcs)),
-                          "mode": "one cooperative launch, one CTA per request, grid barrier per step"}
+                          "mode": "one cooperative launch, one CTA per request, records exchanged per step"}
     if "lookahead" in want:
         sce = S.e1_fine(n_requests=48)
         se = Scheduler.from_scenario(sce, lookahead_W=sce.meta["lookahead_W"])
