@@ -1047,6 +1047,8 @@ __device__ __forceinline__ void plan_indexed(const RolloutArgs& a, const int r, 
             // of this for every length: on a full chip the warps' code, six roles side by side, waits
             // for instructions. 4000 rollouts among 20 000 plans: 55.8 ms with copies for 32, 64 and
             // 128 items, 40.5 with one for 64 (one for 32: 45, for 96: 50); one rollout: unchanged.
+            // (152 CTAs: 65 and 78 % of the instruction cache's requests hit, 5.1 and 1.7 warps per
+            // issue wait for an instruction.)
             constexpr int U = 2;
             for (int i0 = 0; i0 < total; i0 += 32 * U) {
                 float4 P1[U], P2[U];
